@@ -62,9 +62,17 @@ typedef enum {
  * exactly (an error-free splitting in the manner of Ozaki et al.), 40 bits below its scale;
  * FP64 stays for the gather, the scaling, the column output and its residual, the p = 1
  * refinement and the eigendecomposition fallback.
+ *
+ * Only column pos of each root is kept, so rows whose spectrum allows it take a Krylov method
+ * for that column (Lanczos and a quadrature of the root, O(k m^2) instead of O(m^3)): in FP64
+ * mode every order, in FP64 arithmetic; in MIXED_F16 mode, p >= 2, orders up to 192 with
+ * double-float arithmetic (FP32 pairs).  A row that it refuses (lambda_bar / lambda_min above
+ * 2000, or above kappa_max in the mixed mode; not positive definite) and every row of a plan
+ * whose options steer the coupled iteration (k_max, tol, refine_steps, size buckets) takes the
+ * coupled iteration.
  */
 enum {
-  SUBMAT_PREC_FP64 = 0,       /* coupled Newton iteration entirely in FP64 (CUDA cores)     */
+  SUBMAT_PREC_FP64 = 0,       /* everything in FP64 (CUDA cores)                            */
   SUBMAT_PREC_MIXED_F16 = 1,  /* coupled Newton iteration on the tensor cores (tcgen05) with
                                  every matrix split into four FP16 planes of 10-bit integers,
                                  accumulated per level (10 FP16 products per product),
@@ -145,10 +153,12 @@ typedef struct {
   int64_t n_rows;          /* submatrices processed by the last forward                  */
   int32_t m_max;           /* largest submatrix order                                    */
   int32_t iters_max;       /* largest iteration count of the last forward                */
-  int64_t iters_sum;       /* sum of iteration counts                                    */
+  int64_t iters_sum;       /* sum of iteration counts (a row of the Krylov engine counts the
+                              steps that the coupled iteration takes on its interval)     */
   int64_t n_fallback;      /* rows recomputed by the FP64 eigendecomposition fallback    */
   int64_t n_notspd;        /* rows with a non-positive eigenvalue or non-finite input    */
-  double max_resid;        /* largest FP64 column residual seen before the fallback      */
+  double max_resid;        /* largest FP64 column residual seen before the fallback (Krylov
+                              engine: the error bound at which its recurrence stopped)    */
   double sum_m3;           /* sum over rows of m^3 (true sizes)                           */
   double flops_tensor;     /* tensor-core flops executed by the last forward: sum over
                               rows of (GEMMs executed) * 10 FP16 slice products *
@@ -160,9 +170,10 @@ typedef struct {
                               from CUDA events recorded around it on the launch stream   */
   float ms_fallback;       /* device time of the last forward's fallback kernel          */
   int64_t n_illcond;       /* rows sent to the fallback by the condition estimate        */
-  double flops_alg;        /* the method's flops of the last forward, independent of the
-                              engine: sum over rows of k_j (p+1) 2 m_j^3 with the executed
-                              iteration count k_j and the true order m_j, every product
+  double flops_alg;        /* the flops of the coupled iteration on the last forward's rows,
+                              whatever engine computed them: sum over rows of
+                              k_j (p+1) 2 m_j^3 with the iteration count k_j (see
+                              iters_sum) and the true order m_j, every product
                               counted as a dense GEMM (p = 1 adds 2 m_j^3 for its final X
                               product); divide by ms_kernel for the roofline rate        */
 } submat_report;

@@ -13,6 +13,7 @@
 
 #include "common.cuh"
 #include "engine_table.h"
+#include "krylov.cuh"
 
 namespace submat {
 cudaError_t set_attr_mixed();
@@ -40,12 +41,16 @@ submat_status fail(submat_status s, const std::string& msg) {
     }                                                                                   \
   } while (0)
 
-// One persistent launch of the mixed forward: an engine over order[begin, begin + count).
+// One persistent launch of the forward: an engine over order[begin, begin + count).
 struct EngineRun {
   int engine = 0;
   int32_t begin = 0, count = 0;
   int grid = 0;
+  kry::Class cls;                       // Krylov engine: size class and its scratch
+  size_t scratch_off = 0, stride = 0;
 };
+constexpr int kMaxRuns = 9;             // tcgen05, mma.sync, small and six Krylov classes
+static_assert(kMaxRuns <= (int)(sizeof(DevCounters::run_queue) / sizeof(int32_t)), "queue heads");
 
 struct GraphEntry {
   const double* in = nullptr;
@@ -130,7 +135,15 @@ struct submat_plan_s {
   double* d_cg = nullptr;          // submat_pcg work vectors (allocated by the first call)
   double* d_ref = nullptr;         // submat_refine work arrays (allocated by the first call)
   std::vector<GraphEntry> graphs;
-  std::vector<EngineRun> runs;        // mixed path: engine launches by size bucket
+  std::vector<EngineRun> runs;        // engine launches by size bucket
+  std::vector<EngineRun> runs_stall;  // the same while submat_test_stall is on
+  bool stalled = false;
+  bool use_krylov = false;            // some run is the Krylov engine's
+  kry::Nodes nodes{};
+  int32_t* d_redo = nullptr;          // rows the Krylov engine left to the general path
+  char* d_kry = nullptr;              // its scratch
+  std::vector<cudaStream_t> side;     // runs after the first execute beside it
+  std::vector<cudaEvent_t> side_ev;   // fork, then one join per side stream
 };
 
 namespace {
@@ -145,6 +158,10 @@ void release(submat_plan_t P) {
   if (P->cap_stream) cudaStreamDestroy(P->cap_stream);
   for (auto& e : P->ev)
     if (e) cudaEventDestroy(e);
+  for (auto& x : P->side) cudaStreamDestroy(x);
+  for (auto& x : P->side_ev) cudaEventDestroy(x);
+  cudaFree(P->d_redo);
+  cudaFree(P->d_kry);
   cudaFree(P->d_host_in);
   cudaFree(P->d_host_out);
   cudaFree(P->d_tpos);
@@ -175,6 +192,34 @@ cudaError_t ensure_tpos(submat_plan_t P, cudaStream_t s) {
   cudaError_t e = cudaMalloc(&P->d_tpos, (size_t)P->nnz * sizeof(int32_t));
   if (e != cudaSuccess) return e;
   return launch_transposed_positions(P->d_rowptr, P->d_colind, P->n, P->d_tpos, s);
+}
+
+// The Krylov engine's arguments for one run.
+kry::Args krylov_args(submat_plan_t P, const EngineRun& run, const double* in, double* out, int r) {
+  kry::Args k{};
+  k.rowptr = P->d_rowptr;
+  k.colind = P->d_colind;
+  k.m = P->d_m;
+  k.pos = P->d_pos;
+  k.order = P->d_order + run.begin;
+  k.n = run.count;
+  k.p = P->p;
+  k.sign = P->opts.root_sign;
+  k.vals = in;
+  k.out = out;
+  k.ctr = P->d_ctr;
+  k.queue = &P->d_ctr->run_queue[r];
+  k.redo_list = P->d_redo;
+  k.scratch = P->d_kry + run.scratch_off;
+  k.stride = run.stride;
+  k.nb = run.cls.nb;
+  k.ns = run.cls.ns;
+  k.part_smem = run.cls.part_smem ? 1 : 0;
+  k.resid_tol = P->opts.resid_tol;
+  k.kappa_max = P->opts.kappa_max;
+  k.fp64 = P->opts.precision == SUBMAT_PREC_FP64 ? 1 : 0;
+  k.nodes = P->nodes;
+  return k;
 }
 
 // Queue the forward of plan P on stream s.
@@ -211,19 +256,41 @@ submat_status enqueue_forward(submat_plan_t P, const double* in, double* out, cu
                            cudaMemcpyDeviceToDevice, s));
   CUDA_TRY(cudaMemsetAsync(P->d_ctr, 0, sizeof(DevCounters), s));
   CUDA_TRY(cudaEventRecordWithFlags(P->ev[0], s, evf));
-  if (P->opts.precision == SUBMAT_PREC_FP64) {
-    CUDA_TRY(launch_fwd_fp64(a, P->grid, s));
-  } else {
-    for (size_t r = 0; r < P->runs.size(); ++r) {    // longest rows first, one engine per run
-      const EngineRun& run = P->runs[r];
+  const std::vector<EngineRun>& runs = P->stalled ? P->runs_stall : P->runs;
+  const bool fp64 = P->opts.precision == SUBMAT_PREC_FP64;
+  // longest rows first, one engine per run.  The runs write disjoint rows; the Krylov runs have
+  // scratch of their own, so they execute beside the first run (and each other), and the last
+  // CTAs of one overlap the next; the coupled iteration's engines share the plan's scratch and
+  // follow each other on s
+  for (size_t r = 0; r < runs.size(); ++r) {
+    const EngineRun& run = runs[r];
+    const bool beside = r > 0 && run.engine == kEngineKrylov;
+    cudaStream_t q = beside ? P->side[r - 1] : s;
+    if (r == 0 && runs.size() > 1) CUDA_TRY(cudaEventRecord(P->side_ev[0], s));
+    if (beside) CUDA_TRY(cudaStreamWaitEvent(q, P->side_ev[0], 0));
+    if (run.engine == kEngineKrylov) {
+      CUDA_TRY(kry::launch_fwd(krylov_args(P, run, in, out, (int)r), run.cls, run.grid, q));
+    } else if (fp64) {
+      CUDA_TRY(launch_fwd_fp64(a, run.grid, q));
+    } else {
       FwdArgs b = a;
       b.engine = run.engine;
       b.order = P->d_order + run.begin;
       b.n = run.count;
       b.queue = &P->d_ctr->run_queue[r];
       b.scratch_stride = run.engine == kEngineSmall ? scratch_small() : P->stride;
-      CUDA_TRY(launch_fwd_mixed(b, run.grid, s));
+      CUDA_TRY(launch_fwd_mixed(b, run.grid, q));
     }
+    if (beside) CUDA_TRY(cudaEventRecord(P->side_ev[r], q));
+  }
+  for (size_t r = 1; r < runs.size(); ++r)
+    if (runs[r].engine == kEngineKrylov) CUDA_TRY(cudaStreamWaitEvent(s, P->side_ev[r], 0));
+  if (P->use_krylov) {                  // the rows it left to the coupled iteration
+    FwdArgs b = a;
+    b.order = P->d_redo;
+    b.n_dev = &P->d_ctr->n_redo;
+    if (fp64) CUDA_TRY(launch_fwd_fp64(b, P->grid, s));
+    else CUDA_TRY(launch_fwd_mixed(b, P->grid, s));
   }
   CUDA_TRY(cudaEventRecordWithFlags(P->ev[1], s, evf));
   CUDA_TRY(launch_fallback(a, P->grid, s));
@@ -299,6 +366,60 @@ const char* submat_status_string(submat_status s) {
 }
 
 const char* submat_last_error(void) { return g_last_error.c_str(); }
+
+// Largest order the Krylov engine takes.  FP64: every order.  Mixed p = 1 keeps the iteration
+// with its FP64 refinement.  Mixed p >= 2: the orders up to kKrylovMixedMax whose slice
+// arithmetic has no exponent bias; there the tcgen05 engine's result is within 1e-9 of the exact
+// one, so the two engines agree to that; beyond, its rounding grows to 7e-9 (order 240) and
+// 3e-8 (order 800) and the rows keep it.
+constexpr int kKrylovMixedMax = 192;
+static int krylov_max_m(int precision, int p) {
+  if (precision == SUBMAT_PREC_MIXED_F16_SYNC || p > SUBMAT_MIXED_MAX_P) return 0;
+  if (precision == SUBMAT_PREC_FP64) return SUBMAT_MAX_M;
+  if (p == 1) return 0;
+  return std::min(kKrylovMixedMax, mixed_unbiased_max_m(p));
+}
+
+// Engine launches over the plan's rows (sizes: their orders, decreasing).
+static std::vector<EngineRun> plan_runs(submat_plan_t P, const std::vector<int32_t>& sizes, int kry_max,
+                                        size_t* scratch_bytes, size_t* kry_bytes) {
+  std::vector<EngineRun> runs;
+  const submat_opts& o = P->opts;
+  const bool fp64 = o.precision == SUBMAT_PREC_FP64;
+  size_t off = 0;
+  auto bucket = [&](int32_t m) -> int {          // Krylov classes: kEngineKrylov + index
+    if (m <= kry_max) return kEngineKrylov + kry::class_of(m);
+    if (fp64) return kEngineTc;                  // (one kernel for every order)
+    if (o.precision == SUBMAT_PREC_MIXED_F16_SYNC) return kEngineSync;
+    if (m <= o.small_max_m) return kEngineSmall;
+    return m <= o.sync_max_m ? kEngineSync : kEngineTc;
+  };
+  for (int32_t i = 0; i < P->n_jobs;) {
+    const int b = bucket(sizes[i]);
+    int32_t e = i + 1;
+    while (e < P->n_jobs && bucket(sizes[e]) == b) ++e;
+    EngineRun run;
+    run.engine = std::min(b, kEngineKrylov);
+    run.begin = i;
+    run.count = e - i;
+    if (run.engine == kEngineKrylov) {
+      run.cls = kry::make_class(b - kEngineKrylov, sizes[i], false);
+      run.grid = std::min(P->n_sm * run.cls.ctas, run.count);
+      run.stride = kry::layout(run.cls.nb, run.cls.ns, run.cls.nw, run.cls.part_smem, false).g_total;
+      run.scratch_off = off;
+      off += run.stride * run.grid;
+    } else {
+      const int per_sm = fp64 ? 1 : mixed_ctas_per_sm(run.engine);
+      run.grid = std::max(1, std::min(P->n_sm * per_sm, run.count));
+      if (run.engine == kEngineSmall)
+        *scratch_bytes = std::max(*scratch_bytes, scratch_small() * (size_t)run.grid);
+    }
+    runs.push_back(run);
+    i = e;
+  }
+  *kry_bytes = std::max(*kry_bytes, off);
+  return runs;
+}
 
 static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_opts* opts,
                                submat_plan_t* out) {
@@ -463,32 +584,37 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
   stride = (stride + 1023) / 1024 * 1024;
   P->stride = stride;
   P->grid = std::max(1, std::min(P->n_sm, P->n_jobs));
-  // the mixed path's engine runs: the plan's rows are ordered by decreasing m, so each size
-  // bucket is one contiguous run of the order (tcgen05, then mma.sync, then small)
+  // engine runs: the plan's rows are ordered by decreasing m, so each size bucket is one
+  // contiguous run of the order
   size_t scratch_bytes = stride * (size_t)P->grid;
-  if (mixed) {
-    int32_t cnt[3] = {0, 0, 0};
-    for (int32_t j = P->row_begin; j < P->row_end; ++j) {
-      const int32_t mj = h_m[j];
-      int e = kEngineTc;
-      if (o.precision == SUBMAT_PREC_MIXED_F16_SYNC) e = kEngineSync;
-      else if (mj <= o.small_max_m) e = kEngineSmall;
-      else if (mj <= o.sync_max_m) e = kEngineSync;
-      cnt[e]++;
-    }
-    int32_t begin = 0;
-    for (int e : {kEngineTc, kEngineSync, kEngineSmall}) {
-      if (cnt[e] == 0) continue;
-      EngineRun run;
-      run.engine = e;
-      run.begin = begin;
-      run.count = cnt[e];
-      run.grid = std::max(1, std::min(P->n_sm * mixed_ctas_per_sm(e), cnt[e]));
-      if (e == kEngineSmall)
-        scratch_bytes = std::max(scratch_bytes, scratch_small() * (size_t)run.grid);
-      P->runs.push_back(run);
-      begin += cnt[e];
-    }
+  const bool steered = opts && (opts->k_max >= 1 && opts->k_max != 40 || opts->tol > 0.0 ||
+                                opts->refine_steps >= 0 || o.small_max_m != kTunedSmallMaxM ||
+                                o.sync_max_m != kTunedSyncMaxM);
+  const int kry_max = steered ? 0 : krylov_max_m(o.precision, p);
+  if (kry_max > 0 && !kry::cached_nodes(p, o.root_sign, &P->nodes)) {
+    fail(SUBMAT_EINVAL, "quadrature nodes");
+    return bail(SUBMAT_EINVAL);
+  }
+  std::vector<int32_t> sizes(P->n_jobs);
+  for (int32_t i = 0; i < P->n_jobs; ++i) sizes[i] = h_m[order[i]];
+  size_t kry_bytes = 0;
+  P->runs = plan_runs(P, sizes, kry_max, &scratch_bytes, &kry_bytes);
+  if (mixed) P->runs_stall = plan_runs(P, sizes, std::min(kry_max, (int)o.small_max_m), &scratch_bytes, &kry_bytes);
+  for (const EngineRun& run : P->runs) P->use_krylov |= run.engine == kEngineKrylov;
+  if (P->use_krylov) {
+    PLAN_TRY(kry::set_attr_fwd());
+    PLAN_TRY(cudaMalloc(&P->d_redo, nb * sizeof(int32_t)));
+    PLAN_TRY(cudaMalloc(&P->d_kry, kry_bytes));
+  }
+  const size_t n_runs = std::max(P->runs.size(), P->runs_stall.size());
+  for (size_t r = 0; r < n_runs && n_runs > 1; ++r) {
+    cudaEvent_t e = nullptr;
+    PLAN_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    P->side_ev.push_back(e);
+    if (r == 0) continue;
+    cudaStream_t q = nullptr;
+    PLAN_TRY(cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking));
+    P->side.push_back(q);
   }
   PLAN_TRY(cudaMalloc(&P->d_scratch, scratch_bytes));
   if (mixed && o.precision == SUBMAT_PREC_MIXED_F16) {
@@ -856,6 +982,11 @@ submat_status submat_test_stall(submat_plan_t P, int32_t on) {
   CUDA_TRY(dev.enter(P->device));
   const int32_t v = on != 0 ? 1 : 0;
   CUDA_TRY(cudaDeviceSynchronize());          // no forward of this plan reads the flag now
+  if (P->stalled != (v != 0)) {               // other launches: captured graphs are stale
+    for (auto& g : P->graphs) cudaGraphExecDestroy(g.exec);
+    P->graphs.clear();
+    P->stalled = v != 0;
+  }
   CUDA_TRY(cudaMemcpy(P->d_stall, &v, sizeof(v), cudaMemcpyHostToDevice));
   return SUBMAT_OK;
 }

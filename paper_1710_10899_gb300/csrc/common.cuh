@@ -30,7 +30,8 @@ struct DevCounters {
   double flops_tensor;
   unsigned long long n_illcond;        // rows sent to the fallback by the condition estimate
   int32_t error;                       // a device pipeline wait timed out
-  int32_t run_queue[4];                // work-queue heads of the mixed path's engine launches
+  int32_t run_queue[12];               // work-queue heads of the forward's engine launches
+  int32_t n_redo;                      // rows the Krylov engine left to the general path
   double flops_alg;                    // sum over rows of k_j (p+1) 2 m_j^3 (+ 2 m_j^3 for
                                        // p = 1's final X product): executed iterations k_j,
                                        // true orders m_j, every product counted as a dense GEMM
@@ -49,6 +50,8 @@ struct FwdArgs {
   const int32_t* pos;        // [n] position of the diagonal inside the row
   const int32_t* order;      // [n] rows by decreasing size
   int32_t n;
+  const int32_t* n_dev;      // number of rows on the device (the Krylov engine's left-over rows);
+                             // null: n
   int32_t p;
   const double* vals_in;
   double* vals_out;
@@ -88,6 +91,7 @@ struct BwdArgs {
   double* gbuf;
   const int64_t* gofs;       // [n+1] exclusive prefix sums of m_j^2
   int32_t j0, j1;
+  const int32_t* n_dev;      // number of rows on the device; null: n
 };
 
 // Launchers (return cudaGetLastError() of the launch).
@@ -132,7 +136,10 @@ cudaError_t refine_axpby(double c1, const double* x, double c2, const double* y,
 
 // Mixed-path engines (FwdArgs::engine) and their limits.
 constexpr int kEngineTc = 0, kEngineSync = 1, kEngineSmall = 2;
+constexpr int kEngineKrylov = 3;      // krylov.cuh (both precisions)
+constexpr int kMaxSmem = 232448;      // dynamic shared memory a CTA may ask for
 int mixed_ctas_per_sm(int engine);    // CTAs per SM of a mixed-path engine
+int mixed_unbiased_max_m(int p);      // largest order whose slices have no exponent bias
 int small_engine_max_m();             // largest order the small engine takes
 size_t scratch_small();               // small engine: global scratch bytes per CTA
 

@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(BwdArgs a) {
     __syncthreads();
     const int idx = job_s;
     __syncthreads();
-    if (idx >= a.n) break;
+    if (idx >= (a.n_dev ? *a.n_dev : a.n)) break;
     const int j = a.order[idx];
     if (a.gbuf && (j < a.j0 || j >= a.j1)) continue;     // another wave's row
     const int m = a.m[j], pos = a.pos[j], p = a.p;

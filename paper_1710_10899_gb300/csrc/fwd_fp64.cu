@@ -24,6 +24,7 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_fp64_kernel(FwdArgs a) {
   double* norm2_s = red_s + kRedDoubles;
   int32_t* R_s = reinterpret_cast<int32_t*>(norm2_s + 2);
   __shared__ int job_s;
+  const int n_rows = a.n_dev ? *a.n_dev : a.n;
 
   char* scr = a.scratch + (size_t)blockIdx.x * a.scratch_stride;
   const int tid = threadIdx.x;
@@ -32,7 +33,7 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_fp64_kernel(FwdArgs a) {
     __syncthreads();
     const int idx = job_s;
     __syncthreads();
-    if (idx >= a.n) break;
+    if (idx >= n_rows) break;
     const int j = a.order[idx];
     const int m = a.m[j];
     const int pos = a.pos[j];

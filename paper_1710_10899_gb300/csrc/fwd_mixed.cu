@@ -109,7 +109,7 @@ __device__ __forceinline__ int exp_of(float b) { return exp_bound(b * (1.f + 1e-
 // scale to |q0| <= 2^(9-b)): the smallest b for which alpha' = alpha 2^(9-b) stays an FP16
 // integer next to q0 (alpha <= p + 1) and the level-0 / level-1 partial sums of every
 // product stay integers below 2^24 (the bounds of the file header).
-__device__ __forceinline__ int slice_bias(int mp, int p) {
+__host__ __device__ __forceinline__ int slice_bias(int mp, int p) {
   const float rk = sqrtf((float)mp);
   for (int b = 0; b < 3; ++b) {
     const float s0 = ldexpf(1.f, Q0B - b);
@@ -1247,6 +1247,8 @@ __global__ void __launch_bounds__(ENG == ENG_TC ? TC_THREADS : kThreads,
   constexpr bool TC = ENG == ENG_TC, SMALL = ENG == ENG_SMALL;
   constexpr int VMAX = SMALL ? kSmallVmax : SUBMAT_MAX_M;
   extern __shared__ unsigned char smem_raw[];
+  const int n_rows = a.n_dev ? *a.n_dev : a.n;
+  if (a.n_dev && n_rows == 0) return;                  // nothing was left over
   unsigned char* sm = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   double* y_s = reinterpret_cast<double*>(sm);
@@ -1318,7 +1320,7 @@ __global__ void __launch_bounds__(ENG == ENG_TC ? TC_THREADS : kThreads,
     __syncthreads();
     const int idx = job_s;
     __syncthreads();
-    if (idx >= a.n) break;
+    if (idx >= n_rows) break;
     if (*abort_s) {
       pending = a.order[idx];
       break;
@@ -1672,7 +1674,7 @@ __global__ void __launch_bounds__(ENG == ENG_TC ? TC_THREADS : kThreads,
       __syncthreads();
       const int idx = job_s;
       __syncthreads();
-      if (idx >= a.n) break;
+      if (idx >= n_rows) break;
       j = a.order[idx];
     }
   }
@@ -1706,6 +1708,12 @@ cudaError_t launch_fwd_mixed(const FwdArgs& a, int grid, cudaStream_t s) {
   else
     fwd_mixed_kernel<ENG_TC><<<grid, TC_THREADS, smem_bytes<ENG_TC>(), s>>>(a);
   return cudaGetLastError();
+}
+
+int mixed_unbiased_max_m(int p) {
+  int mp = 0;
+  while (mp < SUBMAT_MAX_M && slice_bias(mp + 16, p) == 0) mp += 16;
+  return mp;
 }
 
 int mixed_ctas_per_sm(int engine) { return engine == ENG_SMALL ? kSmallCtasPerSm : 1; }

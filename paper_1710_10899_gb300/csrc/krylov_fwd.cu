@@ -1,0 +1,231 @@
+// Forward by the Krylov engine (krylov.cuh): one persistent launch per size class, one CTA per
+// submatrix, FP64 or double-float arithmetic.
+#include <algorithm>
+#include <cmath>
+#include <mutex>
+
+#include "krylov.cuh"
+
+namespace submat {
+namespace kry {
+namespace {
+
+// Relative bound at which the recurrence stops: double-float rounding leaves ~1e-13 of the
+// column, FP64 ~1e-15.
+template <class T> struct Tol;
+template <> struct Tol<df> { static constexpr float value = 1e-12f; };
+template <> struct Tol<double> { static constexpr float value = 2e-16f; };
+
+template <class T, int NW, bool GP, bool ALL, int NE, int MINB>
+__global__ void __launch_bounds__(threads_of<NW>(), MINB) fwd_kernel(const __grid_constant__ Args a) {
+  constexpr int NT = threads_of<NW>();
+  constexpr int NM = NW * 32;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool mat = warp < NW, node = NW == 1 || warp == NW;
+  Row<T, NW, GP, ALL> r;
+  bind(r, a, false);
+  double* scale_s = reinterpret_cast<double*>(r.flag() + 4);
+  for (;;) {
+    if (tid == 0) {
+      r.flag()[2] = atomicAdd(a.queue, 1);
+      r.flag()[1] = 0;
+    }
+    sync_all<NW>();
+    const int idx = r.flag()[2];
+    if (idx >= a.n) break;
+    r.j = a.order[idx];
+    r.m = a.m[r.j];
+    r.pos = a.pos[r.j];
+    r.nb = (r.m + kB - 1) / kB;
+    r.mp = r.nb * kB;
+    const int p = a.p;
+    const bool direct = p == 1 && a.sign > 0;        // A itself, once it is found definite
+    bool ok = gather(r, a);
+    int K = 0, nc = 0;
+    float est = 0.f, lo = 1.f;
+    if (ok) {
+      stats(r, a.fp64 ? 0.0 : a.kappa_max);
+      if (!direct) {
+        for (int i = tid; i < r.mp; i += NT) r.set_v(i, i == r.pos ? one<T>() : zero<T>());
+        sync_all<NW>();
+        K = lanczos<T, NW, GP, ALL, NE>(r, p, a.sign, Tol<T>::value, &est, &lo);
+      }
+      if (node) {
+        const float tau_f = tau_of(r.lam, lo);
+        if (!direct) nc = root_coefs(r, K, p, lo, a.sign > 0, lane);
+        if (lane == 0) {
+          const double E = (double)(r.e0 - 1023), ex = (double)a.sign / (double)p;
+          const double tau = (double)tau_f;
+          const double al = a.sign < 0 ? 1.0 / (double)p : 1.0 - 1.0 / (double)p;
+          *scale_s = exp2(E * ex) * (p > 1 ? pow(tau, -al) : 1.0);
+          // accepted only with the recurrence's bound met (NaN is not)
+          r.flag()[3] = direct || (lo > 0.f && est <= Tol<T>::value && (double)est <= a.resid_tol) ? nc + 1 : 0;
+        }
+      }
+      if (mat) cholesky(r);
+      sync_all<NW>();
+      nc = r.flag()[3] - 1;
+      ok = nc >= 0 && r.flag()[1] == 0;
+    }
+    if (ok) {
+      const double scale = *scale_s;
+      double* out = a.out + a.rowptr[r.j];
+      if (direct) {
+        for (int i = tid; i < r.m; i += NT) out[i] = a.vals[a.rowptr[r.j] + i];
+      } else if (mat) {
+        for (int i = tid; i < r.m; i += NM) {
+          T s = zero<T>();
+          for (int k = 0; k < nc; ++k) s = add(s, mul(r.coef()[k], r.V[(size_t)k * r.mp + i]));
+          out[i] = join(s) * scale;
+        }
+      }
+    }
+    if (node && lane == 0) {
+      if (!ok) {
+        a.redo_list[atomicAdd(&a.ctr->n_redo, 1)] = r.j;
+      } else {
+        const int iters = coupled_steps(lo, p, r.m, a.fp64 != 0);
+        const double m2 = (double)r.m * r.m;
+        atomicMax(&a.ctr->iters_max, iters);
+        atomicAdd(&a.ctr->iters_sum, (unsigned long long)iters);
+        atomic_max_nonneg(&a.ctr->resid_max_bits, (double)est);
+        if (a.fp64) atomicAdd(&a.ctr->flops_fp64, 2.0 * m2 * (double)K);
+        atomicAdd(&a.ctr->flops_alg, ((double)iters * (p + 1) + (p == 1 ? 1.0 : 0.0)) * 2.0 * m2 * r.m);
+      }
+    }
+    sync_all<NW>();
+  }
+}
+
+template <class T, int NW, bool GP, bool ALL, int NE, int MINB>
+cudaError_t run(const Args& a, int grid, cudaStream_t s) {
+  const Layout L = layout(a.nb, a.ns, NW, !GP, false);
+  fwd_kernel<T, NW, GP, ALL, NE, MINB><<<grid, threads_of<NW>(), L.total, s>>>(a);
+  return cudaGetLastError();
+}
+template <class T, int NW, bool GP, bool ALL, int NE, int MINB>
+cudaError_t attr() {
+  return cudaFuncSetAttribute(fwd_kernel<T, NW, GP, ALL, NE, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              kMaxSmem);
+}
+
+template <class T>
+cudaError_t dispatch(const Args& a, const Class& c, int grid, cudaStream_t s) {
+  switch (c.nw) {
+    case 1: return run<T, 1, false, true, 1, 16>(a, grid, s);
+    case 3: return run<T, 3, false, true, 1, 4>(a, grid, s);
+    case 5: return run<T, 5, false, true, 1, 2>(a, grid, s);
+  }
+  if (c.ns >= nblocks(c.nb)) return run<T, 15, false, true, 1, 1>(a, grid, s);
+  return c.part_smem ? run<T, 15, false, false, 1, 1>(a, grid, s) : run<T, 15, true, false, 4, 1>(a, grid, s);
+}
+
+template <class T>
+cudaError_t attrs() {
+  cudaError_t e;
+  if ((e = attr<T, 1, false, true, 1, 16>()) != cudaSuccess) return e;
+  if ((e = attr<T, 3, false, true, 1, 4>()) != cudaSuccess) return e;
+  if ((e = attr<T, 5, false, true, 1, 2>()) != cudaSuccess) return e;
+  if ((e = attr<T, 15, false, true, 1, 1>()) != cudaSuccess) return e;
+  if ((e = attr<T, 15, false, false, 1, 1>()) != cudaSuccess) return e;
+  return attr<T, 15, true, false, 4, 1>();
+}
+
+}  // namespace
+
+cudaError_t launch_fwd(const Args& a, const Class& c, int grid, cudaStream_t s) {
+  return a.fp64 ? dispatch<double>(a, c, grid, s) : dispatch<df>(a, c, grid, s);
+}
+
+cudaError_t set_attr_fwd() {
+  const cudaError_t e = attrs<df>();
+  return e != cudaSuccess ? e : attrs<double>();
+}
+
+// Gauss-Jacobi nodes for the weight (1-s)^(-a) (1+s)^(a-1): Newton's method on the Jacobi
+// polynomial P_N^(-a, a-1) from the asymptotic zeros; a weight is proportional to
+// 1 / ((1 - s^2) P'(s)^2), and the weights are scaled to the sum 1, which makes the rule
+// exact at x = tau.
+static bool gauss_jacobi(int N, double al, double* theta, double* weight) {
+  typedef long double ld;
+  const ld a = -(ld)al, b = (ld)al - 1.0L, ab = a + b;      // ab = -1
+  ld sum = 0.0L, s[kNodesWide], w[kNodesWide];
+  for (int q = 0; q < N; ++q) {
+    ld x = cosl(3.14159265358979323846264338327950288L * ((ld)q + 0.75L + a / 2) / ((ld)N + (ab + 1) / 2));
+    ld dp = 0.0L;
+    for (int it = 0; it < 30; ++it) {
+      ld p0 = 1.0L, p1 = ((a - b) + (ab + 2) * x) / 2;      // P_0, P_1
+      for (int k = 2; k <= N; ++k) {
+        const ld c = 2 * k + ab;
+        const ld p2 = ((c - 1) * (c * (c - 2) * x + a * a - b * b) * p1 -
+                       2 * (k + a - 1) * (k + b - 1) * c * p0) /
+                      (2 * k * (k + ab) * (c - 2));
+        p0 = p1;
+        p1 = p2;
+      }
+      const ld c = 2 * N + ab;
+      dp = (N * (a - b - c * x) * p1 + 2 * (N + a) * (N + b) * p0) / (c * (1 - x * x));
+      const ld dx = p1 / dp;
+      x -= dx;
+      if (!(fabsl(dx) > 1e-18L)) break;
+    }
+    if (!(x > -1.0L && x < 1.0L)) return false;
+    s[q] = x;
+    w[q] = 1.0L / ((1 - x * x) * dp * dp);
+    sum += w[q];
+  }
+  for (int q = 0; q < N; ++q) {
+    if (q > 0 && !(s[q] < s[q - 1])) return false;          // two starts met in one zero
+    theta[q] = (double)((1 - s[q]) / (1 + s[q]));
+    weight[q] = (double)(w[q] / sum * 2 / (1 + s[q]));
+  }
+  return true;
+}
+
+static bool make_nodes(int p, int sign, Nodes* out) {
+  *out = Nodes{};
+  if (p == 1) return true;                                  // x^(-1) needs no quadrature
+  const double al = sign < 0 ? 1.0 / p : 1.0 - 1.0 / p;
+  return gauss_jacobi(kNodes, al, out->theta, out->w) &&
+         gauss_jacobi(kNodesWide, al, out->theta + kNodes, out->w + kNodes);
+}
+
+bool cached_nodes(int p, int sign, Nodes* out) {     // a constant table per (p, sign)
+  static std::mutex lock;
+  static Nodes table[2][SUBMAT_MIXED_MAX_P + 1];
+  static bool have[2][SUBMAT_MIXED_MAX_P + 1] = {};
+  if (p < 1 || p > SUBMAT_MIXED_MAX_P) return false;
+  const int s = sign < 0 ? 0 : 1;
+  std::lock_guard<std::mutex> hold(lock);
+  if (!have[s][p]) have[s][p] = make_nodes(p, sign, &table[s][p]);
+  *out = table[s][p];
+  return have[s][p];
+}
+
+// Classes by order: warps per CTA and CTAs per SM.  S's blocks fill what shared memory the
+// CTAs per SM leave; a class whose blocks do not all fit streams the rest from scratch (L2).
+constexpr int kClassMax[] = {32, 64, 96, 128, 192, SUBMAT_MAX_M};
+constexpr int kClassWarps[] = {1, 3, 3, 5, 15, 15};    // matrix warps (and one for the nodes)
+constexpr int kClassCtas[] = {16, 4, 3, 2, 1, 1};
+
+int class_of(int m) {
+  int i = 0;
+  while (m > kClassMax[i]) ++i;
+  return i;
+}
+
+Class make_class(int index, int m_max, bool bwd) {
+  Class c;
+  c.max_m = std::min(kClassMax[index], (m_max + kB - 1) / kB * kB);
+  c.nw = kClassWarps[index];
+  c.nb = c.max_m / kB;
+  c.ctas = kClassCtas[index];
+  const size_t room = 233472 / c.ctas - 1024;        // 228 KB an SM, 1 KB reserved per CTA
+  c.part_smem = c.max_m <= 480;
+  const size_t rest = layout(c.nb, 0, c.nw, c.part_smem, bwd).total;
+  c.ns = std::min(nblocks(c.nb), (int)((room - rest) / kBlkBytes));
+  return c;
+}
+
+}  // namespace kry
+}  // namespace submat

@@ -1,0 +1,116 @@
+"""The Krylov engine (one column of the root by Lanczos) against the oracle and against the
+coupled iteration, at the edges of its size classes, and the rows it has to leave to others.
+
+Bars.  FP64: p kappa m eps = 3 * 9 * 250 * 2.2e-16 < 2e-12.  Double-float: products carry an
+error near 2^-45 of a row's norm, so m kappa 2^-45 = 192 * 9 * 2.8e-14 < 1e-10.
+"""
+import numpy as np
+import pytest
+import scipy.linalg as sl
+
+import oracle
+import workloads as wl
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+# one below, at and above each class edge, and the orders around a 32-entry block edge
+ORDERS = [1, 2, 5, 31, 32, 33, 63, 64, 65, 96, 97, 127, 128, 129, 160, 191, 192, 193, 225, 250]
+
+
+@pytest.fixture(scope="module")
+def sm():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_1710_10899_gb300 as pkg
+    pkg.load_library()
+    return pkg
+
+
+def blocks(orders, seed):
+    rng = np.random.default_rng(seed)
+    mats = []
+    for n in orders:
+        q = rng.standard_normal((n, n))
+        mats.append(q @ q.T / n + 0.5 * np.eye(n))
+    return wl.dense_to_csr(sl.block_diag(*mats),
+                           keep=sl.block_diag(*[np.ones((n, n), bool) for n in orders]))
+
+
+def row_err(a, y, ref, rows):
+    return max(float(np.linalg.norm(y[a.rowptr[j]:a.rowptr[j + 1]] - ref[a.rowptr[j]:a.rowptr[j + 1]]) /
+                     np.linalg.norm(ref[a.rowptr[j]:a.rowptr[j + 1]])) for j in rows)
+
+
+def forward(sm, a, p, **kw):
+    plan = sm.submat_plan(a.rowptr, a.colind, p, **kw)
+    y = sm.submat_invroot(plan, torch.tensor(a.vals, device="cuda"), sync=True)
+    return y.cpu().numpy(), plan.report()
+
+
+@pytest.mark.parametrize("p,sign", [(1, -1), (2, -1), (3, -1), (1, 1), (2, 1), (3, 1), (7, -1)])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_orders(sm, precision, p, sign):
+    orders = ORDERS if precision == "fp64" else [n for n in ORDERS if n <= 192]
+    a = blocks(orders, seed=p)
+    rows = sorted({int(r) for s, n in zip(np.cumsum([0] + orders), orders)
+                   for r in (s, s + n // 2, s + n - 1)})
+    y, rep = forward(sm, a, p, precision=precision, root_sign=sign)
+    ref = oracle.invroot(a.rowptr, a.colind, a.vals, p, rows=rows, sign=sign)
+    # the mixed path's largest order on this engine falls with p (the slices' exponent bias);
+    # the tcgen05 engine's rows keep its own bar
+    top = 250 if precision == "fp64" else {1: 192, 2: 192, 3: 144}.get(p, 1)
+    m = a.row_sizes()
+    bar = 2e-12 if precision == "fp64" else 1e-10
+    assert row_err(a, y, ref, [j for j in rows if m[j] <= top]) <= bar
+    assert row_err(a, y, ref, rows) <= (bar if precision == "fp64" else 1e-6)
+    assert rep["n_notspd"] == 0 and rep["n_fallback"] == 0 and rep["n_rows"] == a.n
+    # an explicit step limit keeps the coupled iteration: the two paths agree
+    z, _ = forward(sm, a, p, precision=precision, root_sign=sign, k_max=39)
+    assert row_err(a, z, y, range(a.n)) <= (1e-10 if precision == "fp64" else 1e-6)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("p,sign", [(2, -1), (1, 1)])
+def test_indefinite_part_out_of_reach(sm, precision, p, sign):
+    """A negative eigenvalue in a part of the submatrix that e_pos is not coupled to (stored
+    zeros) is found all the same: every row of that pattern is refused."""
+    n = 40
+    dense = np.eye(n) * 2.0 + np.diag(np.full(n - 1, 0.3), 1) + np.diag(np.full(n - 1, 0.3), -1)
+    dense[25, 25] = -1.0
+    dense[25, :25] = dense[:25, 25] = dense[25, 26:] = dense[26:, 25] = 0.0
+    dense[24, 26] = dense[26, 24] = 0.0
+    a = wl.dense_to_csr(dense, keep=np.ones((n, n), bool))
+    plan = sm.submat_plan(a.rowptr, a.colind, p, precision=precision, root_sign=sign)
+    out = torch.zeros(a.nnz, dtype=torch.float64, device="cuda")
+    with pytest.raises(sm.SubmatError) as ei:
+        sm.submat_invroot(plan, torch.tensor(a.vals, device="cuda"), out, sync=True)
+    assert ei.value.name == "SUBMAT_ENOTSPD"
+    assert torch.isnan(out).all()
+
+
+@pytest.mark.parametrize("kappa", [300.0, 1e5])
+def test_wide_spectra(sm, kappa):
+    """Condition numbers of the wide quadrature rule (300) and beyond the engine's limit (1e5,
+    left to the coupled iteration).  The submatrix is well scaled, so FP64 keeps
+    m kappa eps = 60 * 1e5 * 2.2e-16 < 2e-9 of the column."""
+    rng = np.random.default_rng(3)
+    q, _ = np.linalg.qr(rng.standard_normal((60, 60)))
+    s = (q * np.geomspace(1.0 / kappa, 1.0, 60)) @ q.T
+    a = wl.dense_to_csr(0.5 * (s + s.T), keep=np.ones((60, 60), bool))
+    y, rep = forward(sm, a, 2, precision="fp64")
+    ref = oracle.invroot(a.rowptr, a.colind, a.vals, 2)
+    assert row_err(a, y, ref, range(a.n)) <= (1e-11 if kappa < 1e3 else 2e-9)
+    assert rep["n_notspd"] == 0
+
+
+def test_extreme_scales(sm):
+    """Powers of two on the values scale the result exactly: the engine works on the
+    submatrix over its largest diagonal entry."""
+    a = blocks([20, 70, 150], seed=9)
+    y, _ = forward(sm, a, 2, precision="fp64")
+    for e in (-200, 200):
+        b = wl.CSR(a.n, a.rowptr, a.colind, a.vals * 2.0 ** e)
+        z, rep = forward(sm, b, 2, precision="fp64")
+        np.testing.assert_allclose(z * 2.0 ** (e // 2), y, rtol=1e-15)
+        assert rep["n_fallback"] == 0
