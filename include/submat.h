@@ -243,8 +243,13 @@ SUBMAT_API submat_status submat_invroot_host(submat_plan_t plan, const double* v
  * f(x) = x^(root_sign/p)):
  * grad_in = dL/dvals for L = sum(grad_out * vals_out) of the last forward, with respect to
  * A's stored values, the (r,c)/(c,r) pair sharing one symmetric perturbation.  For each row
- * j the submatrix is regathered from the saved vals_in and decomposed again (recomputation,
- * no stored iterates) by a cyclic Jacobi with the matrix and eigenvectors held as
+ * j the submatrix is regathered from the saved vals_in (recomputation, no stored iterates).
+ * With f as a sum of simple fractions the Daleckii-Krein form is a sum of rank-two terms in
+ * (S + t_q)^(-1) g and (S + t_q)^(-1) e_pos, which two Lanczos processes in double-float
+ * arithmetic give; rows that this refuses (as in the forward), the inverse (p = 1,
+ * root_sign = -1), p above SUBMAT_MIXED_MAX_P, and a first backward inside a stream capture
+ * (its storage is allocated by the first backward) are decomposed instead: a cyclic Jacobi with
+ * the matrix and eigenvectors held as
  * double-floats (FP32 pairs, ~44 significant bits; the rotation angles, the divided
  * differences and the products with the eigenvectors in FP64).  grad_out and grad_in are
  * device arrays of nnz doubles that must not overlap; grad_in is overwritten.  Returns

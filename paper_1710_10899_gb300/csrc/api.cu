@@ -137,6 +137,10 @@ struct submat_plan_s {
   std::vector<GraphEntry> graphs;
   std::vector<EngineRun> runs;        // engine launches by size bucket
   std::vector<EngineRun> runs_stall;  // the same while submat_test_stall is on
+  std::vector<EngineRun> runs_bwd;    // Krylov adjoint (empty: the Jacobi kernel takes every row)
+  size_t bwd_bytes = 0;               // its scratch, allocated by the first backward
+  char* d_kry_bwd = nullptr;
+  int32_t* d_redo_bwd = nullptr;
   bool stalled = false;
   bool use_krylov = false;            // some run is the Krylov engine's
   kry::Nodes nodes{};
@@ -162,6 +166,8 @@ void release(submat_plan_t P) {
   for (auto& x : P->side_ev) cudaEventDestroy(x);
   cudaFree(P->d_redo);
   cudaFree(P->d_kry);
+  cudaFree(P->d_kry_bwd);
+  cudaFree(P->d_redo_bwd);
   cudaFree(P->d_host_in);
   cudaFree(P->d_host_out);
   cudaFree(P->d_tpos);
@@ -214,7 +220,6 @@ kry::Args krylov_args(submat_plan_t P, const EngineRun& run, const double* in, d
   k.stride = run.stride;
   k.nb = run.cls.nb;
   k.ns = run.cls.ns;
-  k.part_smem = run.cls.part_smem ? 1 : 0;
   k.resid_tol = P->opts.resid_tol;
   k.kappa_max = P->opts.kappa_max;
   k.fp64 = P->opts.precision == SUBMAT_PREC_FP64 ? 1 : 0;
@@ -591,7 +596,9 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
                                 opts->refine_steps >= 0 || o.small_max_m != kTunedSmallMaxM ||
                                 o.sync_max_m != kTunedSyncMaxM);
   const int kry_max = steered ? 0 : krylov_max_m(o.precision, p);
-  if (kry_max > 0 && !kry::cached_nodes(p, o.root_sign, &P->nodes)) {
+  // (the inverse's adjoint stays with the Jacobi kernel, whose error there is the smaller one)
+  const bool kry_bwd = p <= SUBMAT_MIXED_MAX_P && (p > 1 || o.root_sign > 0);
+  if ((kry_bwd || kry_max > 0) && !kry::cached_nodes(p, o.root_sign, &P->nodes)) {
     fail(SUBMAT_EINVAL, "quadrature nodes");
     return bail(SUBMAT_EINVAL);
   }
@@ -606,7 +613,26 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
     PLAN_TRY(cudaMalloc(&P->d_redo, nb * sizeof(int32_t)));
     PLAN_TRY(cudaMalloc(&P->d_kry, kry_bytes));
   }
-  const size_t n_runs = std::max(P->runs.size(), P->runs_stall.size());
+  if (kry_bwd) {
+    PLAN_TRY(kry::set_attr_bwd());
+    for (int32_t i = 0; i < P->n_jobs;) {
+      const int b = kry::class_of(sizes[i]);
+      int32_t e = i + 1;
+      while (e < P->n_jobs && kry::class_of(sizes[e]) == b) ++e;
+      EngineRun run;
+      run.engine = kEngineKrylov;
+      run.begin = i;
+      run.count = e - i;
+      run.cls = kry::make_class(b, sizes[i], true);
+      run.grid = std::min(P->n_sm * run.cls.ctas, run.count);
+      run.stride = kry::layout(run.cls.nb, run.cls.ns, run.cls.nw, run.cls.part_smem, true).g_total;
+      run.scratch_off = P->bwd_bytes;
+      P->bwd_bytes += run.stride * run.grid;
+      P->runs_bwd.push_back(run);
+      i = e;
+    }
+  }
+  const size_t n_runs = std::max({P->runs.size(), P->runs_stall.size(), P->runs_bwd.size()});
   for (size_t r = 0; r < n_runs && n_runs > 1; ++r) {
     cudaEvent_t e = nullptr;
     PLAN_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -740,6 +766,63 @@ static submat_status invroot_host_impl(submat_plan_t P, const double* in, double
   return SUBMAT_OK;
 }
 
+// The Krylov adjoint's storage, allocated by the first backward.  False: not to be had (no
+// memory, or the stream is being captured, where nothing can be allocated), and the Jacobi
+// kernel, which needs none, takes every row.
+static bool ready_bwd(submat_plan_t P, cudaStream_t s) {
+  if (P->runs_bwd.empty()) return false;
+  if (P->d_kry_bwd && P->d_redo_bwd && (P->d_tpos || P->nnz == 0)) return true;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
+  if ((!P->d_kry_bwd && cudaMalloc(&P->d_kry_bwd, P->bwd_bytes) != cudaSuccess) ||
+      (!P->d_redo_bwd && cudaMalloc(&P->d_redo_bwd, (size_t)P->n * sizeof(int32_t)) != cudaSuccess) ||
+      ensure_tpos(P, s) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return true;
+}
+
+// The adjoint of the rows of a's wave (all rows without waves): the Krylov runs side by side,
+// then the rows they left in the Jacobi kernel.
+static submat_status enqueue_backward(submat_plan_t P, const BwdArgs& a, bool krylov, cudaStream_t s) {
+  CUDA_TRY(cudaMemsetAsync(P->d_ctr_bwd, 0, sizeof(DevCounters), s));
+  if (!krylov) {
+    CUDA_TRY(launch_backward(a, P->grid, s));
+    return SUBMAT_OK;
+  }
+  const std::vector<EngineRun>& runs = P->runs_bwd;
+  if (runs.size() > 1) CUDA_TRY(cudaEventRecord(P->side_ev[0], s));
+  for (size_t r = 0; r < runs.size(); ++r) {
+    const EngineRun& run = runs[r];
+    cudaStream_t q = r > 0 ? P->side[r - 1] : s;
+    if (r > 0) CUDA_TRY(cudaStreamWaitEvent(q, P->side_ev[0], 0));
+    kry::Args k = krylov_args(P, run, a.vals, a.grad_in, (int)r);
+    k.ctr = P->d_ctr_bwd;
+    k.queue = &P->d_ctr_bwd->run_queue[r];
+    k.redo_list = P->d_redo_bwd;
+    k.scratch = P->d_kry_bwd + run.scratch_off;
+    k.fp64 = 0;
+    k.grad_out = a.grad_out;
+    k.tpos = P->d_tpos;
+    k.gbuf = a.gbuf;
+    k.gofs = a.gofs;
+    k.j0 = a.j0;
+    k.j1 = a.j1;
+    CUDA_TRY(kry::launch_bwd(k, run.cls, run.grid, q));
+    if (r > 0) CUDA_TRY(cudaEventRecord(P->side_ev[r], q));
+  }
+  for (size_t r = 1; r < runs.size(); ++r) CUDA_TRY(cudaStreamWaitEvent(s, P->side_ev[r], 0));
+  BwdArgs b = a;
+  b.order = P->d_redo_bwd;
+  b.n_dev = &P->d_ctr_bwd->n_redo;
+  CUDA_TRY(launch_backward(b, P->grid, s));
+  return SUBMAT_OK;
+}
+
 static submat_status backward_impl(submat_plan_t P, const double* grad_out, double* grad_in,
                                    void* stream) {
   g_last_error.clear();
@@ -773,9 +856,10 @@ static submat_status backward_impl(submat_plan_t P, const double* grad_out, doub
   a.scratch_stride = P->stride;
   a.sign = P->opts.root_sign;
   CUDA_TRY(cudaMemsetAsync(grad_in, 0, (size_t)P->nnz * sizeof(double), s));
-  CUDA_TRY(cudaMemsetAsync(P->d_ctr_bwd, 0, sizeof(DevCounters), s));
+  const bool krylov = ready_bwd(P, s);
   if (!P->opts.grad_deterministic) {
-    CUDA_TRY(launch_backward(a, P->grid, s));
+    const submat_status st = enqueue_backward(P, a, krylov, s);
+    if (st != SUBMAT_OK) return st;
   } else {
     if (!P->d_gbuf) {
       // G_j offsets and waves of at most grad_wave_mib MiB
@@ -804,8 +888,8 @@ static submat_status backward_impl(submat_plan_t P, const double* grad_out, doub
     for (const auto& w : P->waves) {
       a.j0 = w.first;
       a.j1 = w.second;
-      CUDA_TRY(cudaMemsetAsync(&P->d_ctr_bwd->queue, 0, sizeof(int32_t), s));   // job queue
-      CUDA_TRY(launch_backward(a, P->grid, s));
+      const submat_status st = enqueue_backward(P, a, krylov, s);
+      if (st != SUBMAT_OK) return st;
       CUDA_TRY(launch_grad_gather(P->d_rowptr, P->d_colind, P->d_tpos, P->d_m, P->d_gofs,
                                   P->d_gbuf, P->n, w.first, w.second, grad_in, s));
     }

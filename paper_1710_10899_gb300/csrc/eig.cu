@@ -4,7 +4,8 @@
 //   fallback: rows whose mixed/FP64 Newton result failed its residual test are recomputed
 //             from S = V diag(lambda) V^T as column pos of V diag(lambda^(-1/p)) V^T;
 //             a non-positive (or non-finite) eigenvalue marks the row NaN (not SPD).
-//   backward: the Daleckii-Krein adjoint (Higham, Functions of Matrices, Thm. 3.11):
+//   backward: (rows that the Krylov adjoint, krylov_bwd.cu, leaves, and the inverse)
+//             the Daleckii-Krein adjoint (Higham, Functions of Matrices, Thm. 3.11):
 //             for L = <g, column pos of f(S)>, f(x) = x^(-1/p), and the symmetrised
 //             cotangent Gbar = (g e_pos^T + e_pos g^T)/2,
 //             dL/dS = V (Gamma o (V^T Gbar V)) V^T,  Gamma_ab = divided difference of f,
@@ -98,12 +99,13 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(BwdArgs a) {
   __shared__ int bad_s;
   char* scr = a.scratch + (size_t)blockIdx.x * a.scratch_stride;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n_rows = a.n_dev ? *a.n_dev : a.n;
   for (;;) {
     if (tid == 0) job_s = atomicAdd(&a.ctr->queue, 1);
     __syncthreads();
     const int idx = job_s;
     __syncthreads();
-    if (idx >= (a.n_dev ? *a.n_dev : a.n)) break;
+    if (idx >= n_rows) break;
     const int j = a.order[idx];
     if (a.gbuf && (j < a.j0 || j >= a.j1)) continue;     // another wave's row
     const int m = a.m[j], pos = a.pos[j], p = a.p;

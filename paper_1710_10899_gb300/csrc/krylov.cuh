@@ -55,7 +55,8 @@ constexpr int kBlkBytes = kB * kB * 8;
 constexpr int kBuckets = 256;              // column buckets of the gather
 constexpr int kNodes = 32;                 // quadrature nodes (one per lane)
 constexpr int kNodesWide = 64;             // nodes for spectra wider than [lam / 100, lam]
-constexpr int kNodesAll = kNodes + kNodesWide;
+constexpr int kNodesGrad = 20;             // nodes of the adjoint for spectra within [lam / 50, lam]
+constexpr int kNodesAll = kNodes + kNodesWide + kNodesGrad;
 constexpr float kKappa = 2000.f;           // largest lam / lambda_min taken here
 constexpr float kTau = 0.1f;               // tau / lam for spectra in [lam / 100, lam]
 constexpr float kLoWide = 0.01f;            // lo / lam from which kNodes nodes do
@@ -67,7 +68,7 @@ __host__ __device__ inline int nblocks(int nb) { return nb * (nb + 1) / 2; }
 // Quadrature of one exponent a: nodes theta = (1-s)/(1+s), weights omega 2/(1+s) (sum of omega
 // 1), so x^(-a) = tau^(-a) sum_q w_q tau / (x + tau theta_q).
 struct Nodes {
-  double theta[kNodesAll], w[kNodesAll];   // kNodes of one rule, then kNodesWide of the other
+  double theta[kNodesAll], w[kNodesAll];   // the rules of kNodes, kNodesWide and kNodesGrad nodes
 };
 
 // One size class: a persistent launch over rows of order <= 32 nb.
@@ -88,7 +89,6 @@ struct Args {
   size_t stride;                           // bytes per CTA
   int32_t nb;                              // blocks per edge of the class
   int32_t ns;                              // blocks of S held in shared memory
-  int32_t part_smem;                       // partial sums in shared memory
   double resid_tol, kappa_max;
   int32_t fp64;
   Nodes nodes;
@@ -102,32 +102,40 @@ struct Args {
 
 // Shared-memory and scratch layout of a class (bytes), host and device.
 struct Layout {
-  size_t blocks, v, part, al, be, coef, red, nodes, ext, R, bk, total;
+  size_t blocks, v, part, al, be, coef, red, nodes, ext, R, bk, start, total;
   size_t g_blocks, g_v, g_x, g_part, g_ab, g_total;
+  size_t v_bytes, x_bytes, t_bytes;        // one process's share of g_v, g_x, al and be
 };
 __host__ __device__ inline Layout layout(int nb, int ns, int nw, bool part_smem, bool bwd) {
   Layout L{};
   const size_t mp = (size_t)nb * kB, cap = cap_of(nw);
   size_t o = 0;
   auto take = [&](size_t b) { const size_t at = o; o += (b + 15) / 16 * 16; return at; };
-  L.blocks = take((size_t)ns * kBlkBytes);
+  const size_t proc = bwd ? 2 : 1;         // Lanczos processes (the adjoint runs two)
+  L.v_bytes = (cap + 2) * mp * 8;
+  L.x_bytes = (cap + 1) * (size_t)kNodes * 8;
+  L.t_bytes = (cap + 1) * 8 + 8;
+  // the adjoint's factors take S's place when they fit
+  const size_t ab = bwd && nblocks(nb) <= ns ? (size_t)kNodes * mp * 16 : 0;
+  L.blocks = take((size_t)ns * kBlkBytes > ab ? (size_t)ns * kBlkBytes : ab);
   L.v = take(mp * 8);
   L.part = take(part_smem ? (size_t)nb * mp * 8 : 0);
-  L.al = take((cap + 1) * 8);
-  L.be = take((cap + 1) * 8);
+  L.al = take(proc * L.t_bytes);
+  L.be = take(proc * L.t_bytes);
   L.coef = take((cap + 2) * 8);
-  L.red = take(4 * 16 * 8 + 64);
+  L.red = take(32 * 8 + 64);            // two sums of 16 warps, then flags
   L.nodes = take(2 * kNodesAll * 8);
   L.ext = take(mp * 8);
   L.R = take(mp * 4);
   L.bk = take((kBuckets + 2) * 2);
+  L.start = take(bwd ? mp * 4 : 0);
   L.total = o;
   o = 0;
   L.g_blocks = take((size_t)(nblocks(nb) - ns) * kBlkBytes);
-  L.g_v = take((cap + 2) * mp * 8);
-  L.g_x = take((cap + 1) * (size_t)kNodes * 8);
+  L.g_v = take(proc * L.v_bytes);
+  L.g_x = take(proc * L.x_bytes);
   L.g_part = take(part_smem ? 0 : (size_t)nb * mp * 8);
-  L.g_ab = take(bwd ? 2 * (size_t)kNodes * mp * 8 : 0);
+  L.g_ab = take(bwd && !ab ? (size_t)kNodes * mp * 16 : 0);
   L.g_total = (o + 1023) / 1024 * 1024;
   return L;
 }
@@ -342,9 +350,10 @@ __device__ __forceinline__ float hi32(f2 a) { return __uint_as_float((unsigned)(
 __device__ __forceinline__ void madd2(f2 sh, f2 sl, f2 vh, f2 vl, f2 minus1, f2& s, f2& c) {
   const f2 s1 = fma2(sh, vh, s);
   const f2 nz = fma2(s1, minus1, s);                 // s - s1, exact
-  c = add2(c, fma2(sh, vh, nz));
-  c = fma2(sh, vl, c);
-  c = fma2(sl, vh, c);
+  f2 t = fma2(sh, vh, nz);                           // exact; the small terms meet before c
+  t = fma2(sl, vh, t);
+  t = fma2(sh, vl, t);
+  c = add2(c, t);
   s = s1;
 }
 
@@ -485,7 +494,7 @@ struct Row {
   float4* gblk;                 // blocks t >= ns, in scratch
   T* gpart;                     // partial sums (GP)
   T *V, *X;                     // scratch: Lanczos vectors [k][mp], node solutions [k][32]
-  T* AB;                        // scratch: backward factors
+  float4* AB;                   // adjoint: factors (a, b) per node and row
   int e0;                       // exponent field of the largest diagonal entry
   float lam, C, sigma;          // of the scaled submatrix: Gershgorin bound, accumulator start,
                                 // certified lower end
@@ -507,6 +516,24 @@ struct Row {
       h[mp + i] = x.l;
     }
   }
+  // node solution k of node q (a double-float row: 32 leading, then 32 trailing parts)
+  __device__ __forceinline__ T x_at(int k, int q) const {
+    if constexpr (__is_same(T, double)) {
+      return X[(size_t)k * kNodes + q];
+    } else {
+      const float* h = reinterpret_cast<const float*>(X + (size_t)k * kNodes);
+      return df{h[q], h[kNodes + q]};
+    }
+  }
+  __device__ __forceinline__ void set_x(int k, int q, T x) const {
+    if constexpr (__is_same(T, double)) {
+      X[(size_t)k * kNodes + q] = x;
+    } else {
+      float* h = reinterpret_cast<float*>(X + (size_t)k * kNodes);
+      h[q] = x.h;
+      h[kNodes + q] = x.l;
+    }
+  }
   __device__ __forceinline__ T* part() const {
     if constexpr (GP) return gpart; else return reinterpret_cast<T*>(kry_smem + o_part);
   }
@@ -514,7 +541,7 @@ struct Row {
   __device__ __forceinline__ T* be() const { return reinterpret_cast<T*>(kry_smem + o_be); }
   __device__ __forceinline__ T* coef() const { return reinterpret_cast<T*>(kry_smem + o_coef); }
   __device__ __forceinline__ T* red() const { return reinterpret_cast<T*>(kry_smem + o_red); }
-  __device__ __forceinline__ int* flag() const { return reinterpret_cast<int*>(kry_smem + o_red + 512); }
+  __device__ __forceinline__ int* flag() const { return reinterpret_cast<int*>(kry_smem + o_red + 256); }
   __device__ __forceinline__ double* nodes() const { return reinterpret_cast<double*>(kry_smem + o_nodes); }
   __device__ __forceinline__ int2* ext() const { return reinterpret_cast<int2*>(kry_smem + o_ext); }
   __device__ __forceinline__ int32_t* R() const { return reinterpret_cast<int32_t*>(kry_smem + o_R); }
@@ -549,7 +576,7 @@ __device__ __forceinline__ void bind(Row<T, NW, GP, ALL>& r, const Args& a, bool
   r.gpart = reinterpret_cast<T*>(scr + L.g_part);
   r.V = reinterpret_cast<T*>(scr + L.g_v);
   r.X = reinterpret_cast<T*>(scr + L.g_x);
-  r.AB = reinterpret_cast<T*>(scr + L.g_ab);
+  r.AB = ALL ? r.sblk() : reinterpret_cast<float4*>(scr + L.g_ab);
   for (int q = threadIdx.x; q < kNodesAll; q += threads_of<NW>()) {
     r.nodes()[q] = a.nodes.theta[q];
     r.nodes()[kNodesAll + q] = a.nodes.w[q];
@@ -613,7 +640,7 @@ __device__ __forceinline__ void find_cols(const Row<T, NW, GP, ALL>& r, const Bu
 // first entries already requested.  Returns false (to every thread) when some diagonal entry
 // is not a positive normal number.
 template <class T, int NW, bool GP, bool ALL>
-__device__ bool gather(Row<T, NW, GP, ALL>& r, const Args& a) {
+__device__ bool gather(Row<T, NW, GP, ALL>& r, const Args& a, int32_t* start = nullptr) {
   constexpr int NT = threads_of<NW>();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int base = a.rowptr[r.j], m = r.m;
@@ -621,8 +648,10 @@ __device__ bool gather(Row<T, NW, GP, ALL>& r, const Args& a) {
   for (int k = tid; k < m; k += NT) {
     const int c = a.colind[base + k];
     r.R()[k] = c;
-    const int2 x = make_int2(a.rowptr[c] + a.pos[c], a.rowptr[c + 1]);
+    const int first = a.rowptr[c];
+    const int2 x = make_int2(first + a.pos[c], a.rowptr[c + 1]);
     r.ext()[k] = x;
+    if (start) start[k] = first;
     const int h = __double2hiint(a.vals[x.x]);
     mx = max(mx, h);
     mn = min(mn, h);
@@ -932,28 +961,33 @@ __device__ __forceinline__ float tau_of(float lam, float lo) {
 // Node solutions x = (T + t)^(-1) e_1 (node q of the lane, the whole warp calls it), times the
 // node's weight, in r.X[k][lane]; a bottom-up elimination leaves the right-hand side e_1 alone,
 // so one sweep up for the pivots and one down for x.
+// The weight is tau w_q times `extra` (times t for x^(1/p), whose adjoint weighs
+// t (x + t)^(-1)); wt0 multiplies every weight.
 template <class T, int NW, bool GP, bool ALL>
-__device__ void node_solve(const Row<T, NW, GP, ALL>& r, int K, int p, float tau_f, int q, bool weighted) {
+__device__ void node_solve(const Row<T, NW, GP, ALL>& r, int K, int p, float tau_f, int q, bool weighted,
+                           bool times_t, T wt0) {
   const int lane = threadIdx.x & 31;
   const T tau = as(tau_f, (T*)nullptr);
   T t = zero<T>(), wt = one<T>();
   if (p > 1) {
     t = mul(tau, as(r.nodes()[q], (T*)nullptr));
     wt = mul(tau, as(r.nodes()[kNodesAll + q], (T*)nullptr));
+    if (times_t) wt = mul(wt, t);
   } else if (lane > 0) {
     wt = zero<T>();
   }
+  wt = mul(wt, wt0);
   T x = rcp(add(r.al()[K - 1], t));
   for (int k = K - 2; k >= 0; --k) {
     const T g = mul(r.be()[k], x);
-    r.X[(size_t)k * kNodes + lane] = g;
+    r.set_x(k, lane, g);
     x = rcp(sub(add(r.al()[k], t), mul(r.be()[k], g)));
   }
   if (weighted) x = mul(x, wt);
   for (int k = 0; k < K; ++k) {
     T g = zero<T>();
-    if (k + 1 < K) g = r.X[(size_t)k * kNodes + lane];
-    r.X[(size_t)k * kNodes + lane] = x;
+    if (k + 1 < K) g = r.x_at(k, lane);
+    r.set_x(k, lane, x);
     x = neg(mul(g, x));
   }
   __syncwarp();
@@ -963,8 +997,8 @@ __device__ void node_solve(const Row<T, NW, GP, ALL>& r, int K, int p, float tau
 template <class T, int NW, bool GP, bool ALL>
 __device__ void sum_nodes(const Row<T, NW, GP, ALL>& r, int K, bool more) {
   for (int k = threadIdx.x & 31; k < K; k += 32) {
-    T s = r.X[(size_t)k * kNodes];
-    for (int q = 1; q < kNodes; ++q) s = add(s, r.X[(size_t)k * kNodes + q]);
+    T s = r.x_at(k, 0);
+    for (int q = 1; q < kNodes; ++q) s = add(s, r.x_at(k, q));
     r.coef()[k] = more ? add(r.coef()[k], s) : s;
   }
   __syncwarp();
@@ -976,12 +1010,12 @@ template <class T, int NW, bool GP, bool ALL>
 __device__ int root_coefs(const Row<T, NW, GP, ALL>& r, int K, int p, float lo, bool times_t, int lane) {
   const float tau = tau_of(r.lam, lo);
   if (p == 1 || lo >= kLoWide) {
-    node_solve(r, K, p, tau, lane, true);
+    node_solve(r, K, p, tau, lane, true, false, one<T>());
     sum_nodes(r, K, false);
   } else {
 #pragma unroll 1
     for (int h = 0; h < kNodesWide / 32; ++h) {
-      node_solve(r, K, p, tau, kNodes + 32 * h + lane, true);
+      node_solve(r, K, p, tau, kNodes + 32 * h + lane, true, false, one<T>());
       sum_nodes(r, K, h > 0);
     }
   }

@@ -100,6 +100,7 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) fwd_kernel(const __gri
 template <class T, int NW, bool GP, bool ALL, int NE, int MINB>
 cudaError_t run(const Args& a, int grid, cudaStream_t s) {
   const Layout L = layout(a.nb, a.ns, NW, !GP, false);
+  if ((ALL && a.ns < nblocks(a.nb)) || L.total > kMaxSmem) return cudaErrorInvalidValue;
   fwd_kernel<T, NW, GP, ALL, NE, MINB><<<grid, threads_of<NW>(), L.total, s>>>(a);
   return cudaGetLastError();
 }
@@ -146,29 +147,36 @@ cudaError_t set_attr_fwd() {
 // polynomial P_N^(-a, a-1) from the asymptotic zeros; a weight is proportional to
 // 1 / ((1 - s^2) P'(s)^2), and the weights are scaled to the sum 1, which makes the rule
 // exact at x = tau.
+template <class F>
+static F jacobi_step(int N, F a, F b, F x, F* dp) {         // P_N(x) / P_N'(x)
+  const F ab = a + b;
+  F p0 = 1, p1 = ((a - b) + (ab + 2) * x) / 2;              // P_0, P_1
+  for (int k = 2; k <= N; ++k) {
+    const F c = 2 * k + ab;
+    const F p2 = ((c - 1) * (c * (c - 2) * x + a * a - b * b) * p1 -
+                  2 * (k + a - 1) * (k + b - 1) * c * p0) /
+                 (2 * k * (k + ab) * (c - 2));
+    p0 = p1;
+    p1 = p2;
+  }
+  const F c = 2 * N + ab;
+  *dp = (N * (a - b - c * x) * p1 + 2 * (N + a) * (N + b) * p0) / (c * (1 - x * x));
+  return p1 / *dp;
+}
 static bool gauss_jacobi(int N, double al, double* theta, double* weight) {
   typedef long double ld;
-  const ld a = -(ld)al, b = (ld)al - 1.0L, ab = a + b;      // ab = -1
+  const ld a = -(ld)al, b = (ld)al - 1.0L;                  // a + b = -1
   ld sum = 0.0L, s[kNodesWide], w[kNodesWide];
   for (int q = 0; q < N; ++q) {
-    ld x = cosl(3.14159265358979323846264338327950288L * ((ld)q + 0.75L + a / 2) / ((ld)N + (ab + 1) / 2));
-    ld dp = 0.0L;
+    double xd = std::cos(3.14159265358979323846 * (q + 0.75 - al / 2) / N), dpd = 0.0;   // ab = -1
     for (int it = 0; it < 30; ++it) {
-      ld p0 = 1.0L, p1 = ((a - b) + (ab + 2) * x) / 2;      // P_0, P_1
-      for (int k = 2; k <= N; ++k) {
-        const ld c = 2 * k + ab;
-        const ld p2 = ((c - 1) * (c * (c - 2) * x + a * a - b * b) * p1 -
-                       2 * (k + a - 1) * (k + b - 1) * c * p0) /
-                      (2 * k * (k + ab) * (c - 2));
-        p0 = p1;
-        p1 = p2;
-      }
-      const ld c = 2 * N + ab;
-      dp = (N * (a - b - c * x) * p1 + 2 * (N + a) * (N + b) * p0) / (c * (1 - x * x));
-      const ld dx = p1 / dp;
-      x -= dx;
-      if (!(fabsl(dx) > 1e-18L)) break;
+      const double dx = jacobi_step<double>(N, -al, al - 1.0, xd, &dpd);
+      xd -= dx;
+      if (!(std::fabs(dx) > 1e-15)) break;
     }
+    ld x = xd, dp = 0.0L;                                   // polished in extended precision
+    x -= jacobi_step<ld>(N, a, b, x, &dp);
+    jacobi_step<ld>(N, a, b, x, &dp);
     if (!(x > -1.0L && x < 1.0L)) return false;
     s[q] = x;
     w[q] = 1.0L / ((1 - x * x) * dp * dp);
@@ -187,7 +195,8 @@ static bool make_nodes(int p, int sign, Nodes* out) {
   if (p == 1) return true;                                  // x^(-1) needs no quadrature
   const double al = sign < 0 ? 1.0 / p : 1.0 - 1.0 / p;
   return gauss_jacobi(kNodes, al, out->theta, out->w) &&
-         gauss_jacobi(kNodesWide, al, out->theta + kNodes, out->w + kNodes);
+         gauss_jacobi(kNodesWide, al, out->theta + kNodes, out->w + kNodes) &&
+         gauss_jacobi(kNodesGrad, al, out->theta + kNodes + kNodesWide, out->w + kNodes + kNodesWide);
 }
 
 bool cached_nodes(int p, int sign, Nodes* out) {     // a constant table per (p, sign)
@@ -220,10 +229,16 @@ Class make_class(int index, int m_max, bool bwd) {
   c.nw = kClassWarps[index];
   c.nb = c.max_m / kB;
   c.ctas = kClassCtas[index];
-  const size_t room = 233472 / c.ctas - 1024;        // 228 KB an SM, 1 KB reserved per CTA
+  if (bwd && index == 0) c.ctas = 8;                 // its factors need 16 KB a CTA
   c.part_smem = c.max_m <= 480;
-  const size_t rest = layout(c.nb, 0, c.nw, c.part_smem, bwd).total;
-  c.ns = std::min(nblocks(c.nb), (int)((room - rest) / kBlkBytes));
+  const bool all = index + 1 < (int)(sizeof(kClassMax) / sizeof(kClassMax[0]));   // holds every block
+  for (;; --c.ctas) {
+    const size_t room = 233472 / c.ctas - 1024;      // 228 KB an SM, 1 KB reserved per CTA
+    const size_t rest = layout(c.nb, 0, c.nw, c.part_smem, bwd).total;
+    c.ns = room > rest ? std::min(nblocks(c.nb), (int)((room - rest) / kBlkBytes)) : 0;
+    if (layout(c.nb, c.ns, c.nw, c.part_smem, bwd).total <= room && (!all || c.ns == nblocks(c.nb))) break;
+    if (c.ctas == 1) break;                          // refused by the launch
+  }
   return c;
 }
 

@@ -114,3 +114,61 @@ def test_extreme_scales(sm):
         z, rep = forward(sm, b, 2, precision="fp64")
         np.testing.assert_allclose(z * 2.0 ** (e // 2), y, rtol=1e-15)
         assert rep["n_fallback"] == 0
+
+
+@pytest.mark.parametrize("p,sign", [(1, -1), (2, -1), (3, -1), (1, 1), (2, 1), (3, 1)])
+@pytest.mark.parametrize("deterministic", [False, True])
+def test_adjoint_orders(sm, p, sign, deterministic):
+    """The Krylov adjoint at the class edges, with a zero cotangent on one block, against the
+    oracle gradient (bar as for the Jacobi adjoint)."""
+    orders = [1, 2, 31, 32, 33, 64, 65, 97, 129, 193, 250]
+    a = blocks(orders, seed=20 + p)
+    w = wl.random_on_pattern(a, seed=5)
+    lo = sum(n * n for n in orders[:4])
+    w[lo:lo + 33 * 33] = 0.0
+    plan = sm.submat_plan(a.rowptr, a.colind, p, root_sign=sign, grad_deterministic=deterministic)
+    sm.submat_invroot(plan, torch.tensor(a.vals, device="cuda"))
+    g = sm.submat_invroot_backward(plan, torch.tensor(w, device="cuda")).cpu().numpy()
+    gref = oracle.grad(a.rowptr, a.colind, a.vals, p, w, sign=sign)
+    assert np.linalg.norm(g - gref) / np.linalg.norm(gref) <= 1e-10
+    assert np.abs(g - gref).max() <= 1e-10 * np.abs(gref).max()
+    assert np.all(g[lo:lo + 33 * 33] == 0.0)
+
+
+@pytest.mark.parametrize("kappa,bar", [(300.0, 1e-10), (1e5, 1e-5)])
+def test_adjoint_wide_spectra(sm, kappa, bar):
+    """A spectrum of the wide quadrature rule (two passes over the entries) and one beyond the
+    engine (the Jacobi kernel).  f' ~ x^(-3/2) spans kappa^(3/2), so double-floats (2^-45)
+    keep 300^1.5 * 60 * 2.8e-14 < 1e-8 of the smallest and 1e-10 of the largest part; at 1e5
+    the divided differences themselves keep 1e-5."""
+    rng = np.random.default_rng(3)
+    q, _ = np.linalg.qr(rng.standard_normal((60, 60)))
+    s = (q * np.geomspace(1.0 / kappa, 1.0, 60)) @ q.T
+    a = wl.dense_to_csr(0.5 * (s + s.T), keep=np.ones((60, 60), bool))
+    w = wl.random_on_pattern(a, seed=6)
+    gref = oracle.grad(a.rowptr, a.colind, a.vals, 2, w)
+    for det in (False, True):
+        plan = sm.submat_plan(a.rowptr, a.colind, 2, precision="fp64", grad_deterministic=det)
+        sm.submat_invroot(plan, torch.tensor(a.vals, device="cuda"))
+        g = sm.submat_invroot_backward(plan, torch.tensor(w, device="cuda")).cpu().numpy()
+        assert np.abs(g - gref).max() <= bar * np.abs(gref).max()
+
+
+def test_first_backward_under_capture(sm):
+    """The first backward of a plan inside a stream capture, where the Krylov adjoint's storage
+    cannot be allocated: the Jacobi kernel takes every row, and the replay gives the gradient."""
+    a = blocks([20, 50], seed=11)
+    w = wl.random_on_pattern(a, seed=7)
+    plan = sm.submat_plan(a.rowptr, a.colind, 2, use_graph=False)
+    v, wd = torch.tensor(a.vals, device="cuda"), torch.tensor(w, device="cuda")
+    out, grad = torch.empty_like(v), torch.empty_like(v)
+    sm.submat_invroot(plan, v, out, sync=True)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        sm.submat_invroot(plan, v, out)
+        sm.submat_invroot_backward(plan, wd, grad)
+    grad.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    gref = oracle.grad(a.rowptr, a.colind, a.vals, 2, w)
+    assert np.abs(grad.cpu().numpy() - gref).max() <= 1e-10 * np.abs(gref).max()
