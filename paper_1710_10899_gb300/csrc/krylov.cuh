@@ -100,37 +100,56 @@ struct Args {
   int32_t j0, j1;
 };
 
-// Shared-memory and scratch layout of a class (bytes), host and device.
+// Shared-memory and scratch layout (bytes), host and device.  What a kernel instance needs is
+// sized for its largest order, so that the offsets are constants of the code (kept in
+// registers they cost ten of them); S's blocks follow, then the partial sums.
+struct Fixed {
+  int t_bytes;                             // one Lanczos process's share of al and be
+  int al, be, coef, red, nodes, bk, v, ext, R, start, blocks;
+};
+// Largest order of an instance in blocks: by its warps, or for kBigWarps by where S and the
+// partial sums lie.
+constexpr int kBigWarps = 15;
+__host__ __device__ constexpr int nb_cap(int nw, bool part_smem, bool all) {
+  return nw == 1 ? 1 : nw == 3 ? 3 : nw == 5 ? 4 : all ? 6 : part_smem ? 15 : SUBMAT_MAX_M / kB;
+}
+__host__ __device__ constexpr int up16(int b) { return (b + 15) / 16 * 16; }
+__host__ __device__ constexpr Fixed fixed(int nw, int nb, bool bwd) {
+  const int mp = nb * kB, cap = cap_of(nw), proc = bwd ? 2 : 1;
+  Fixed f{};
+  f.t_bytes = up16((cap + 1) * 8);
+  f.al = 0;
+  f.be = f.al + proc * f.t_bytes;
+  f.coef = f.be + proc * f.t_bytes;
+  f.red = f.coef + up16((cap + 2) * 8);
+  f.nodes = f.red + 32 * 8 + 64;           // two sums of 16 warps, then flags
+  f.bk = f.nodes + 2 * kNodesAll * 8;
+  f.v = f.bk + up16((kBuckets + 2) * 2);
+  f.ext = f.v + mp * 8;
+  f.R = f.ext + mp * 8;
+  f.start = f.R + mp * 4;
+  f.blocks = f.start + (bwd ? mp * 4 : 0);
+  return f;
+}
 struct Layout {
-  size_t blocks, v, part, al, be, coef, red, nodes, ext, R, bk, start, total;
+  size_t part, total;
   size_t g_blocks, g_v, g_x, g_part, g_ab, g_total;
-  size_t v_bytes, x_bytes, t_bytes;        // one process's share of g_v, g_x, al and be
+  size_t v_bytes, x_bytes;                 // one process's share of g_v and g_x
 };
 __host__ __device__ inline Layout layout(int nb, int ns, int nw, bool part_smem, bool bwd) {
   Layout L{};
   const size_t mp = (size_t)nb * kB, cap = cap_of(nw);
-  size_t o = 0;
-  auto take = [&](size_t b) { const size_t at = o; o += (b + 15) / 16 * 16; return at; };
+  const bool all = nw != kBigWarps || nb <= 6;
   const size_t proc = bwd ? 2 : 1;         // Lanczos processes (the adjoint runs two)
   L.v_bytes = (cap + 2) * mp * 8;
   L.x_bytes = (cap + 1) * (size_t)kNodes * 8;
-  L.t_bytes = (cap + 1) * 8 + 8;
-  // the adjoint's factors take S's place when they fit
-  const size_t ab = bwd && nblocks(nb) <= ns ? (size_t)kNodes * mp * 16 : 0;
-  L.blocks = take((size_t)ns * kBlkBytes > ab ? (size_t)ns * kBlkBytes : ab);
-  L.v = take(mp * 8);
-  L.part = take(part_smem ? (size_t)nb * mp * 8 : 0);
-  L.al = take(proc * L.t_bytes);
-  L.be = take(proc * L.t_bytes);
-  L.coef = take((cap + 2) * 8);
-  L.red = take(32 * 8 + 64);            // two sums of 16 warps, then flags
-  L.nodes = take(2 * kNodesAll * 8);
-  L.ext = take(mp * 8);
-  L.R = take(mp * 4);
-  L.bk = take((kBuckets + 2) * 2);
-  L.start = take(bwd ? mp * 4 : 0);
-  L.total = o;
-  o = 0;
+  // the adjoint's factors take S's place when all of S lies in shared memory
+  const size_t ab = bwd && all ? (size_t)kNodes * mp * 16 : 0;
+  const size_t blocks = (size_t)ns * kBlkBytes;
+  L.part = fixed(nw, nb_cap(nw, part_smem, all), bwd).blocks + (blocks > ab ? blocks : ab);
+  L.total = L.part + (part_smem ? (size_t)nb * mp * 8 : 0);
+  size_t o = 0;
+  auto take = [&](size_t b) { const size_t at = o; o += (b + 15) / 16 * 16; return at; };
   L.g_blocks = take((size_t)(nblocks(nb) - ns) * kBlkBytes);
   L.g_v = take(proc * L.v_bytes);
   L.g_x = take(proc * L.x_bytes);
@@ -487,10 +506,12 @@ __device__ __forceinline__ void block_stats(const float4* blk, int I, int J,
 extern __shared__ __align__(16) unsigned char kry_smem[];
 
 // GP: partial sums in scratch instead of shared memory; ALL: every block in shared memory
-template <class T, int NW, bool GP, bool ALL>
+template <class T, int NW, bool GP, bool ALL, bool BWD>
 struct Row {
+  static constexpr int kNb = nb_cap(NW, !GP, ALL);
+  static constexpr Fixed kF = fixed(NW, kNb, BWD);
   int m, nb, mp, ns, pos, j;
-  int o_v, o_part, o_al, o_be, o_coef, o_red, o_nodes, o_ext, o_R, o_bk;
+  int o_part, o_t;              // partial sums; current Lanczos process in al and be
   float4* gblk;                 // blocks t >= ns, in scratch
   T* gpart;                     // partial sums (GP)
   T *V, *X;                     // scratch: Lanczos vectors [k][mp], node solutions [k][32]
@@ -498,12 +519,12 @@ struct Row {
   int e0;                       // exponent field of the largest diagonal entry
   float lam, C, sigma;          // of the scaled submatrix: Gershgorin bound, accumulator start,
                                 // certified lower end
-  __device__ __forceinline__ T* v() const { return reinterpret_cast<T*>(kry_smem + o_v); }
+  __device__ __forceinline__ T* v() const { return reinterpret_cast<T*>(kry_smem + kF.v); }
   __device__ __forceinline__ T v_at(int i) const {
     if constexpr (__is_same(T, double)) {
       return v()[i];
     } else {
-      const float* h = reinterpret_cast<const float*>(kry_smem + o_v);
+      const float* h = reinterpret_cast<const float*>(kry_smem + kF.v);
       return df{h[i], h[mp + i]};
     }
   }
@@ -511,7 +532,7 @@ struct Row {
     if constexpr (__is_same(T, double)) {
       v()[i] = x;
     } else {
-      float* h = reinterpret_cast<float*>(kry_smem + o_v);
+      float* h = reinterpret_cast<float*>(kry_smem + kF.v);
       h[i] = x.h;
       h[mp + i] = x.l;
     }
@@ -537,17 +558,18 @@ struct Row {
   __device__ __forceinline__ T* part() const {
     if constexpr (GP) return gpart; else return reinterpret_cast<T*>(kry_smem + o_part);
   }
-  __device__ __forceinline__ T* al() const { return reinterpret_cast<T*>(kry_smem + o_al); }
-  __device__ __forceinline__ T* be() const { return reinterpret_cast<T*>(kry_smem + o_be); }
-  __device__ __forceinline__ T* coef() const { return reinterpret_cast<T*>(kry_smem + o_coef); }
-  __device__ __forceinline__ T* red() const { return reinterpret_cast<T*>(kry_smem + o_red); }
-  __device__ __forceinline__ int* flag() const { return reinterpret_cast<int*>(kry_smem + o_red + 256); }
-  __device__ __forceinline__ double* nodes() const { return reinterpret_cast<double*>(kry_smem + o_nodes); }
-  __device__ __forceinline__ int2* ext() const { return reinterpret_cast<int2*>(kry_smem + o_ext); }
-  __device__ __forceinline__ int32_t* R() const { return reinterpret_cast<int32_t*>(kry_smem + o_R); }
+  __device__ __forceinline__ T* al() const { return reinterpret_cast<T*>(kry_smem + kF.al + o_t); }
+  __device__ __forceinline__ T* be() const { return reinterpret_cast<T*>(kry_smem + kF.be + o_t); }
+  __device__ __forceinline__ T* coef() const { return reinterpret_cast<T*>(kry_smem + kF.coef); }
+  __device__ __forceinline__ T* red() const { return reinterpret_cast<T*>(kry_smem + kF.red); }
+  __device__ __forceinline__ int* flag() const { return reinterpret_cast<int*>(kry_smem + kF.red + 256); }
+  __device__ __forceinline__ double* nodes() const { return reinterpret_cast<double*>(kry_smem + kF.nodes); }
+  __device__ __forceinline__ int2* ext() const { return reinterpret_cast<int2*>(kry_smem + kF.ext); }
+  __device__ __forceinline__ int32_t* R() const { return reinterpret_cast<int32_t*>(kry_smem + kF.R); }
   // first position of each column bucket (kBuckets + 1 entries)
-  __device__ __forceinline__ uint16_t* bk() const { return reinterpret_cast<uint16_t*>(kry_smem + o_bk); }
-  __device__ __forceinline__ float4* sblk() const { return reinterpret_cast<float4*>(kry_smem); }
+  __device__ __forceinline__ uint16_t* bk() const { return reinterpret_cast<uint16_t*>(kry_smem + kF.bk); }
+  __device__ __forceinline__ int32_t* start() const { return reinterpret_cast<int32_t*>(kry_smem + kF.start); }
+  __device__ __forceinline__ float4* sblk() const { return reinterpret_cast<float4*>(kry_smem + kF.blocks); }
   __device__ __forceinline__ float4* sblk(int t) const { return sblk() + t * (kBlkBytes / 16); }
   __device__ __forceinline__ float4* gblk_at(int t) const { return gblk + (size_t)(t - ns) * (kBlkBytes / 16); }
   __device__ __forceinline__ float4* blk(int t) const {
@@ -557,20 +579,12 @@ struct Row {
   __device__ __forceinline__ int tri(int I, int J) const { return I * nb - I * (I - 1) / 2 + J - I; }
 };
 
-template <class T, int NW, bool GP, bool ALL>
-__device__ __forceinline__ void bind(Row<T, NW, GP, ALL>& r, const Args& a, bool bwd) {
-  const Layout L = layout(a.nb, a.ns, NW, !GP, bwd);
+template <class T, int NW, bool GP, bool ALL, bool BWD>
+__device__ __forceinline__ void bind(Row<T, NW, GP, ALL, BWD>& r, const Args& a) {
+  const Layout L = layout(a.nb, a.ns, NW, !GP, BWD);
   char* scr = a.scratch + (size_t)blockIdx.x * a.stride;
-  r.o_v = (int)L.v;
   r.o_part = (int)L.part;
-  r.o_al = (int)L.al;
-  r.o_be = (int)L.be;
-  r.o_coef = (int)L.coef;
-  r.o_red = (int)L.red;
-  r.o_nodes = (int)L.nodes;
-  r.o_ext = (int)L.ext;
-  r.o_R = (int)L.R;
-  r.o_bk = (int)L.bk;
+  r.o_t = 0;
   r.ns = a.ns;
   r.gblk = reinterpret_cast<float4*>(scr + L.g_blocks);
   r.gpart = reinterpret_cast<T*>(scr + L.g_part);
@@ -593,8 +607,8 @@ struct Buckets {
     return range <= (unsigned)kBuckets ? d : __umulhi(d, mul);
   }
 };
-template <class T, int NW, bool GP, bool ALL>
-__device__ __forceinline__ Buckets make_buckets(const Row<T, NW, GP, ALL>& r) {
+template <class T, int NW, bool GP, bool ALL, bool BWD>
+__device__ __forceinline__ Buckets make_buckets(const Row<T, NW, GP, ALL, BWD>& r) {
   Buckets k;
   k.first = (unsigned)r.R()[0];
   k.range = (unsigned)r.R()[r.m - 1] - k.first + 1;
@@ -602,8 +616,8 @@ __device__ __forceinline__ Buckets make_buckets(const Row<T, NW, GP, ALL>& r) {
   return k;
 }
 // r.bk()[b] = first position whose bucket is at least b (b <= kBuckets).
-template <class T, int NW, bool GP, bool ALL>
-__device__ __forceinline__ void fill_buckets(const Row<T, NW, GP, ALL>& r, const Buckets& k) {
+template <class T, int NW, bool GP, bool ALL, bool BWD>
+__device__ __forceinline__ void fill_buckets(const Row<T, NW, GP, ALL, BWD>& r, const Buckets& k) {
   for (int i = threadIdx.x; i <= r.m; i += threads_of<NW>()) {
     const int b0 = i == 0 ? 0 : (int)k.of(r.R()[i - 1]) + 1;
     const int b1 = i == r.m ? kBuckets : (int)k.of(r.R()[i]);
@@ -611,8 +625,8 @@ __device__ __forceinline__ void fill_buckets(const Row<T, NW, GP, ALL>& r, const
   }
 }
 // Positions of U columns in R (-1 where absent; col < 0 gives -1).
-template <int U, class T, int NW, bool GP, bool ALL>
-__device__ __forceinline__ void find_cols(const Row<T, NW, GP, ALL>& r, const Buckets& k, const int* col, int* pos) {
+template <int U, class T, int NW, bool GP, bool ALL, bool BWD>
+__device__ __forceinline__ void find_cols(const Row<T, NW, GP, ALL, BWD>& r, const Buckets& k, const int* col, int* pos) {
   int lo[U], n[U];
   int most = 0;
 #pragma unroll
@@ -639,8 +653,8 @@ __device__ __forceinline__ void find_cols(const Row<T, NW, GP, ALL>& r, const Bu
 // read from its diagonal on (plan's pos), so half of it; a warp takes one row, its next row's
 // first entries already requested.  Returns false (to every thread) when some diagonal entry
 // is not a positive normal number.
-template <class T, int NW, bool GP, bool ALL>
-__device__ bool gather(Row<T, NW, GP, ALL>& r, const Args& a, int32_t* start = nullptr) {
+template <class T, int NW, bool GP, bool ALL, bool BWD>
+__device__ bool gather(Row<T, NW, GP, ALL, BWD>& r, const Args& a) {
   constexpr int NT = threads_of<NW>();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int base = a.rowptr[r.j], m = r.m;
@@ -651,7 +665,7 @@ __device__ bool gather(Row<T, NW, GP, ALL>& r, const Args& a, int32_t* start = n
     const int first = a.rowptr[c];
     const int2 x = make_int2(first + a.pos[c], a.rowptr[c + 1]);
     r.ext()[k] = x;
-    if (start) start[k] = first;
+    if (BWD) r.start()[k] = first;
     const int h = __double2hiint(a.vals[x.x]);
     mx = max(mx, h);
     mn = min(mn, h);
@@ -720,8 +734,8 @@ __device__ bool gather(Row<T, NW, GP, ALL>& r, const Args& a, int32_t* start = n
   return true;
 }
 
-template <class T, int NW, bool GP, bool ALL, class F>
-__device__ __forceinline__ void for_blocks(const Row<T, NW, GP, ALL>& r, int warp, F f) {
+template <class T, int NW, bool GP, bool ALL, bool BWD, class F>
+__device__ __forceinline__ void for_blocks(const Row<T, NW, GP, ALL, BWD>& r, int warp, F f) {
   int I = 0, J = 0;
   auto step = [&](int s) {
     J += s;
@@ -735,8 +749,8 @@ __device__ __forceinline__ void for_blocks(const Row<T, NW, GP, ALL>& r, int war
 }
 
 // Gershgorin bound, accumulator start and certified lower end.
-template <class T, int NW, bool GP, bool ALL>
-__device__ void stats(Row<T, NW, GP, ALL>& r, double kappa_max) {
+template <class T, int NW, bool GP, bool ALL, bool BWD>
+__device__ void stats(Row<T, NW, GP, ALL, BWD>& r, double kappa_max) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float2* p2 = reinterpret_cast<float2*>(r.part());
   if (warp < NW)
@@ -866,8 +880,8 @@ template <int NW, class T> __device__ __forceinline__ T row_sum(const T* part, i
   return s;
 }
 
-template <class T, int NW, bool GP, bool ALL, int NE>
-__device__ int lanczos(const Row<T, NW, GP, ALL>& r, int p, int sign, float tol, float* est, float* lo) {
+template <int NE, class T, int NW, bool GP, bool ALL, bool BWD>
+__device__ int lanczos(const Row<T, NW, GP, ALL, BWD>& r, int p, int sign, float tol, float* est, float* lo) {
   constexpr int cap = cap_of(NW);
   constexpr int NM = NW * 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -885,11 +899,14 @@ __device__ int lanczos(const Row<T, NW, GP, ALL>& r, int p, int sign, float tol,
   T beta = zero<T>(), inv = one<T>();
   int k = 0;
   for (;; ++k) {
+    const int nv = NE > 1 ? NW : min(NW, r.nb);       // warps that hold elements
     if (k > 0) {
-      const T n2 = total_of<NW>(r.red() + 16, lane, NE > 1 ? NW : min(NW, r.nb));
-      const bool end = !(hi(n2) > 1e-34f);            // the space is exhausted
-      inv = end ? zero<T>() : inv_sqrt(n2);
-      beta = end ? zero<T>() : mul(n2, inv);
+      const T n2 = total_of<NW>(r.red() + 16, lane, nv);
+      if (warp < nv || node) {
+        const bool end = !(hi(n2) > 1e-34f);          // the space is exhausted
+        inv = end ? zero<T>() : inv_sqrt(n2);
+        beta = end ? zero<T>() : mul(n2, inv);
+      }
       const int ex = (int)((__float_as_uint(hi(n2)) >> 23) & 0xFF) - 127;
       C = r.C * __int_as_float((((ex + 2) >> 1) + 127) << 23);       // 2^((ex+2)/2) >= beta
     }
@@ -917,7 +934,6 @@ __device__ int lanczos(const Row<T, NW, GP, ALL>& r, int p, int sign, float tol,
     }
     sync_all<NW>();
     const bool stop = k > 0 && r.flag()[0];
-    const int nv = NE > 1 ? NW : min(NW, r.nb);       // warps that hold elements
     if (warp < nv) {
       const T al = mul(mul(total_of<NW>(r.red(), lane, NW), inv), inv);
       T n2 = zero<T>();
@@ -932,7 +948,7 @@ __device__ int lanczos(const Row<T, NW, GP, ALL>& r, int p, int sign, float tol,
             w[e] = sub(sub(sv, mul(beta, vp[e])), mul(al, v));
             vp[e] = v;
             r.set_v(i, w[e]);
-            n2 = add(n2, mul(w[e], w[e]));
+            n2 = NE > 1 ? add(n2, mul(w[e], w[e])) : mul(w[e], w[e]);
           }
         }
       }
@@ -963,8 +979,8 @@ __device__ __forceinline__ float tau_of(float lam, float lo) {
 // so one sweep up for the pivots and one down for x.
 // The weight is tau w_q times `extra` (times t for x^(1/p), whose adjoint weighs
 // t (x + t)^(-1)); wt0 multiplies every weight.
-template <class T, int NW, bool GP, bool ALL>
-__device__ void node_solve(const Row<T, NW, GP, ALL>& r, int K, int p, float tau_f, int q, bool weighted,
+template <class T, int NW, bool GP, bool ALL, bool BWD>
+__device__ void node_solve(const Row<T, NW, GP, ALL, BWD>& r, int K, int p, float tau_f, int q, bool weighted,
                            bool times_t, T wt0) {
   const int lane = threadIdx.x & 31;
   const T tau = as(tau_f, (T*)nullptr);
@@ -994,8 +1010,8 @@ __device__ void node_solve(const Row<T, NW, GP, ALL>& r, int K, int p, float tau
 }
 
 // coef[k] (+)= sum over the nodes of X[k][.].
-template <class T, int NW, bool GP, bool ALL>
-__device__ void sum_nodes(const Row<T, NW, GP, ALL>& r, int K, bool more) {
+template <class T, int NW, bool GP, bool ALL, bool BWD>
+__device__ void sum_nodes(const Row<T, NW, GP, ALL, BWD>& r, int K, bool more) {
   for (int k = threadIdx.x & 31; k < K; k += 32) {
     T s = r.x_at(k, 0);
     for (int q = 1; q < kNodes; ++q) s = add(s, r.x_at(k, q));
@@ -1006,8 +1022,8 @@ __device__ void sum_nodes(const Row<T, NW, GP, ALL>& r, int K, bool more) {
 
 // coef = f(T) e_1 up to the factor tau^(-a); f(x) = x x^(-a) (`times_t`) multiplies by T, which
 // adds the component K.  Returns the number of coefficients.  The whole (node) warp calls it.
-template <class T, int NW, bool GP, bool ALL>
-__device__ int root_coefs(const Row<T, NW, GP, ALL>& r, int K, int p, float lo, bool times_t, int lane) {
+template <class T, int NW, bool GP, bool ALL, bool BWD>
+__device__ int root_coefs(const Row<T, NW, GP, ALL, BWD>& r, int K, int p, float lo, bool times_t, int lane) {
   const float tau = tau_of(r.lam, lo);
   if (p == 1 || lo >= kLoWide) {
     node_solve(r, K, p, tau, lane, true, false, one<T>());
@@ -1045,8 +1061,8 @@ __device__ int root_coefs(const Row<T, NW, GP, ALL>& r, int K, int p, float lo, 
 // the others finish the update.  Called by the NW matrix warps; true when every pivot is
 // positive.  S's rounding to FP32 and the factorisation's own move eigenvalues by about
 // m 2^-24 lam, far below sigma = lam / kKappa.
-template <class T, int NW, bool GP, bool ALL>
-__device__ bool cholesky(const Row<T, NW, GP, ALL>& r) {
+template <class T, int NW, bool GP, bool ALL, bool BWD>
+__device__ bool cholesky(const Row<T, NW, GP, ALL, BWD>& r) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float* invd = reinterpret_cast<float*>(r.part());    // 32 reciprocal pivots' roots
   int* bad = r.flag() + 1;
@@ -1123,7 +1139,7 @@ __device__ bool cholesky(const Row<T, NW, GP, ALL>& r) {
       float4* d = r.blk(r.tri(J, Kb));
       const int a4 = lane >> 2, b8 = lane & 3;
       float acc[4][8] = {};
-#pragma unroll 8
+#pragma unroll 2
       for (int k = 0; k < 32; ++k) {
         const float4 x = p[k * 8 + a4], y0 = q[k * 8 + b8 * 2], y1 = q[k * 8 + b8 * 2 + 1];
         const float xs[4] = {x.x, x.y, x.z, x.w};

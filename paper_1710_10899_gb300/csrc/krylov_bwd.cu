@@ -36,7 +36,7 @@ __device__ __forceinline__ double widen(float f, int e) {
 // factor of the row goes into the weights, their power of two into flag 5.  r is bound to g's
 // process (al, be).
 template <int NW, bool GP, bool ALL>
-__device__ void solve_nodes(Row<df, NW, GP, ALL>& r, const Args& a, int K0, int K1, df* X0, df* X1, int t_bytes,
+__device__ void solve_nodes(Row<df, NW, GP, ALL, true>& r, const Args& a, int K0, int K1, df* X0, df* X1, int t_bytes,
                             df gnorm, int eg, int pass) {
   const int lane = threadIdx.x & 31, p = a.p, Q = r.flag()[3];
   const float lo = __int_as_float(r.flag()[4]);
@@ -55,11 +55,9 @@ __device__ void solve_nodes(Row<df, NW, GP, ALL>& r, const Args& a, int K0, int 
   r.X = X0;
   node_solve(r, K1, p, tau, q, false, false, one<df>());
   r.X = X1;
-  r.o_al -= t_bytes;
-  r.o_be -= t_bytes;
+  r.o_t -= t_bytes;
   node_solve(r, K0, p, tau, q, true, a.sign > 0, wt0);
-  r.o_al += t_bytes;
-  r.o_be += t_bytes;
+  r.o_t += t_bytes;
   r.X = X0;
   if (lane == 0) r.flag()[5] = ef + (int)fl + (eg - 1023);
 }
@@ -71,15 +69,14 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) bwd_kernel(const __gri
   constexpr int NM = NW * 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool mat = warp < NW, node = NW == 1 || warp == NW;
-  Row<T, NW, GP, ALL> r;
-  bind(r, a, true);
+  Row<T, NW, GP, ALL, true> r;
+  bind(r, a);
   const Layout L = layout(a.nb, a.ns, NW, !GP, true);
-  const int t_bytes = (int)L.t_bytes;
+  constexpr int t_bytes = decltype(r)::kF.t_bytes;
   T* const V0 = r.V;
   T* const X0 = r.X;
   T* const V1 = reinterpret_cast<T*>(reinterpret_cast<char*>(V0) + L.v_bytes);
   T* const X1 = reinterpret_cast<T*>(reinterpret_cast<char*>(X0) + L.x_bytes);
-  int32_t* start = reinterpret_cast<int32_t*>(kry_smem + L.start);
   const int p = a.p;
   const bool direct = p == 1 && a.sign > 0;          // f(x) = x: one term, x = g, y = e_pos
   for (;;) {
@@ -98,7 +95,7 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) bwd_kernel(const __gri
     r.nb = (r.m + kB - 1) / kB;
     r.mp = r.nb * kB;
     const int base = a.rowptr[r.j];
-    bool ok = gather(r, a, start);
+    bool ok = gather(r, a);
     // g 2^-eg, eg the exponent of its largest entry
     int eg = 0;
     for (int i = tid; i < r.m; i += NT)
@@ -123,7 +120,7 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) bwd_kernel(const __gri
         float est0 = 0.f, est1 = 0.f, lo0 = 0.f, lo1 = 0.f;
         for (int i = tid; i < r.mp; i += NT) r.set_v(i, i == r.pos ? one<T>() : zero<T>());
         sync_all<NW>();
-        K0 = lanczos<T, NW, GP, ALL, NE>(r, p, a.sign, kTolGrad, &est0, &lo0);
+        K0 = lanczos<NE>(r, p, a.sign, kTolGrad, &est0, &lo0);
         T n2 = zero<T>();
         for (int i = tid; i < r.mp; i += NT) {
           const T x = i < r.m ? scaled(a.grad_out[base + i], eg, (T*)nullptr) : zero<T>();
@@ -138,10 +135,9 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) bwd_kernel(const __gri
         gnorm = mul(n2, inv);
         for (int i = tid; i < r.mp; i += NT) r.set_v(i, mul(r.v_at(i), inv));
         r.V = V1;
-        r.o_al += t_bytes;
-        r.o_be += t_bytes;
+        r.o_t += t_bytes;
         sync_all<NW>();
-        K1 = lanczos<T, NW, GP, ALL, NE>(r, p, a.sign, kTolGrad, &est1, &lo1);
+        K1 = lanczos<NE>(r, p, a.sign, kTolGrad, &est1, &lo1);
         if (node) {
           lo = fminf(lo0, lo1);
           // the divided differences need the quadrature over both spectra
@@ -155,8 +151,7 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) bwd_kernel(const __gri
           if (good) solve_nodes(r, a, K0, K1, X0, X1, t_bytes, gnorm, eg, 0);
         }
         r.V = V0;
-        r.o_al -= t_bytes;
-        r.o_be -= t_bytes;
+        r.o_t -= t_bytes;
       } else if (tid == 0) {
         r.flag()[3] = 1;
         r.flag()[5] = eg - 1023;
@@ -188,12 +183,10 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) bwd_kernel(const __gri
     if (pass > 0) {                                  // the wide rule's next 32 nodes
       if (node) {
         r.V = V1;
-        r.o_al += t_bytes;
-        r.o_be += t_bytes;
+        r.o_t += t_bytes;
         solve_nodes(r, a, K0, K1, X0, X1, t_bytes, gnorm, eg, pass);
         r.V = V0;
-        r.o_al -= t_bytes;
-        r.o_be -= t_bytes;
+        r.o_t -= t_bytes;
       }
       sync_all<NW>();
     }
@@ -292,7 +285,7 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) bwd_kernel(const __gri
             gj[(size_t)li * r.m + k] = sum;
           } else {
             atomicAdd(a.out + e, val);
-            if (li != k) atomicAdd(a.out + start[li] + a.tpos[e], val);
+            if (li != k) atomicAdd(a.out + r.start()[li] + a.tpos[e], val);
           }
         }
       }
@@ -328,7 +321,7 @@ cudaError_t launch_bwd(const Args& a, const Class& c, int grid, cudaStream_t s) 
     case 3: return run<3, false, true, 1, 4>(a, grid, s);
     case 5: return run<5, false, true, 1, 2>(a, grid, s);
   }
-  if (c.ns >= nblocks(c.nb)) return run<15, false, true, 1, 1>(a, grid, s);
+  if (c.nb <= 6) return run<15, false, true, 1, 1>(a, grid, s);
   return c.part_smem ? run<15, false, false, 1, 1>(a, grid, s) : run<15, true, false, 4, 1>(a, grid, s);
 }
 
