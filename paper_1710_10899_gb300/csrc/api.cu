@@ -46,6 +46,7 @@ struct EngineRun {
   int engine = 0;
   int32_t begin = 0, count = 0;
   int grid = 0;
+  int32_t n_jobs = 0;                   // tcgen05: jobs (rows of one pattern form one)
   kry::Class cls;                       // Krylov engine: size class and its scratch
   size_t scratch_off = 0, stride = 0;
 };
@@ -141,6 +142,7 @@ struct submat_plan_s {
   size_t bwd_bytes = 0;               // its scratch, allocated by the first backward
   char* d_kry_bwd = nullptr;
   int32_t* d_redo_bwd = nullptr;
+  int2* d_jobs = nullptr;             // tcgen05 engine's jobs
   bool stalled = false;
   bool use_krylov = false;            // some run is the Krylov engine's
   kry::Nodes nodes{};
@@ -165,6 +167,7 @@ void release(submat_plan_t P) {
   for (auto& x : P->side) cudaStreamDestroy(x);
   for (auto& x : P->side_ev) cudaEventDestroy(x);
   cudaFree(P->d_redo);
+  cudaFree(P->d_jobs);
   cudaFree(P->d_kry);
   cudaFree(P->d_kry_bwd);
   cudaFree(P->d_redo_bwd);
@@ -282,6 +285,10 @@ submat_status enqueue_forward(submat_plan_t P, const double* in, double* out, cu
       b.engine = run.engine;
       b.order = P->d_order + run.begin;
       b.n = run.count;
+      if (run.engine == kEngineTc && P->d_jobs) {
+        b.jobs = P->d_jobs;
+        b.n = run.n_jobs;
+      }
       b.queue = &P->d_ctr->run_queue[r];
       b.scratch_stride = run.engine == kEngineSmall ? scratch_small() : P->stride;
       CUDA_TRY(launch_fwd_mixed(b, run.grid, q));
@@ -608,6 +615,40 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
   P->runs = plan_runs(P, sizes, kry_max, &scratch_bytes, &kry_bytes);
   if (mixed) P->runs_stall = plan_runs(P, sizes, std::min(kry_max, (int)o.small_max_m), &scratch_bytes, &kry_bytes);
   for (const EngineRun& run : P->runs) P->use_krylov |= run.engine == kEngineKrylov;
+  // rows of one pattern share their submatrix: the tcgen05 engine takes them as one job (the
+  // order keeps them together: equal m, ascending indices; its rows come first)
+  int32_t tc_rows = 0;
+  if (o.precision == SUBMAT_PREC_MIXED_F16)
+    for (const auto* rs : {&P->runs, &P->runs_stall})
+      for (const EngineRun& run : *rs)
+        if (run.engine == kEngineTc) tc_rows = std::max(tc_rows, run.count);
+  if (tc_rows > 0) {
+    std::vector<uint8_t> same((size_t)n);
+    uint8_t* d_same = nullptr;
+    PLAN_TRY(cudaMalloc(&d_same, (size_t)n));
+    std::unique_ptr<uint8_t, cudaError_t (*)(void*)> hold(d_same, [](void* q) { return cudaFree(q); });
+    PLAN_TRY(launch_same_pattern(P->d_rowptr, P->d_colind, n, d_same, 0));
+    PLAN_TRY(cudaMemcpy(same.data(), d_same, (size_t)n, cudaMemcpyDeviceToHost));
+    const int cap = mixed_group_max(P->ld, p);
+    std::vector<int2> jobs;
+    for (int32_t i = 0; i < tc_rows; ++i) {
+      const bool joins = i > 0 && jobs.back().y < cap && order[i] == order[i - 1] + 1 && same[order[i]];
+      if (joins) ++jobs.back().y;
+      else jobs.push_back(make_int2(i, 1));
+    }
+    if ((int32_t)jobs.size() < tc_rows) {
+      PLAN_TRY(cudaMalloc(&P->d_jobs, jobs.size() * sizeof(int2)));
+      PLAN_TRY(cudaMemcpy(P->d_jobs, jobs.data(), jobs.size() * sizeof(int2), cudaMemcpyHostToDevice));
+      for (auto* rs : {&P->runs, &P->runs_stall})
+        for (EngineRun& run : *rs)
+          if (run.engine == kEngineTc) {
+            int32_t k = 0;
+            while (k < (int32_t)jobs.size() && jobs[k].x < run.count) ++k;
+            run.n_jobs = k;
+            run.grid = std::min(run.grid, k);
+          }
+    }
+  }
   if (P->use_krylov) {
     PLAN_TRY(kry::set_attr_fwd());
     PLAN_TRY(cudaMalloc(&P->d_redo, nb * sizeof(int32_t)));

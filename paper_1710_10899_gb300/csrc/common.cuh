@@ -49,6 +49,7 @@ struct FwdArgs {
   const int32_t* m;          // [n] row sizes
   const int32_t* pos;        // [n] position of the diagonal inside the row
   const int32_t* order;      // [n] rows by decreasing size
+  const int2* jobs;          // tcgen05: job i = rows order[x, x + y), all of one pattern (null: row i)
   int32_t n;
   const int32_t* n_dev;      // number of rows on the device (the Krylov engine's left-over rows);
                              // null: n
@@ -97,6 +98,9 @@ struct BwdArgs {
 // Launchers (return cudaGetLastError() of the launch).
 cudaError_t launch_plan_rows(const int32_t* rowptr, const int32_t* colind, int32_t n,
                              int32_t* m, int32_t* pos, int32_t* flags, cudaStream_t s);
+// same[j] = 1 when row j's columns equal row j - 1's.
+cudaError_t launch_same_pattern(const int32_t* rowptr, const int32_t* colind, int32_t n, uint8_t* same,
+                                cudaStream_t s);
 cudaError_t launch_check_pattern(const int32_t* rowptr, const int32_t* colind, int32_t n,
                                  int32_t* flags, cudaStream_t s);
 cudaError_t launch_fwd_mixed(const FwdArgs& a, int grid, cudaStream_t s);
@@ -139,6 +143,7 @@ constexpr int kEngineTc = 0, kEngineSync = 1, kEngineSmall = 2;
 constexpr int kEngineKrylov = 3;      // krylov.cuh (both precisions)
 constexpr int kMaxSmem = 232448;      // dynamic shared memory a CTA may ask for
 int mixed_ctas_per_sm(int engine);    // CTAs per SM of a mixed-path engine
+int mixed_group_max(int ld, int p);   // rows of one pattern that a tcgen05 job may hold
 int mixed_unbiased_max_m(int p);      // largest order whose slices have no exponent bias
 int small_engine_max_m();             // largest order the small engine takes
 size_t scratch_small();               // small engine: global scratch bytes per CTA

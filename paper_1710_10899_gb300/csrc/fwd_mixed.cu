@@ -61,12 +61,14 @@
 // leading mp x mp block (mp = m padded to 16 for tcgen05, 64 for mma.sync); its padding
 // rows/columns stay exactly zero.  Rows of a tile beyond mp may hold older data: they only
 // reach output entries beyond mp, which are never stored.
+#include <algorithm>
 #include <cuda_fp16.h>
 #include "common.cuh"
 #include "refine.cuh"
 #include "slices.cuh"
 #include "scaled_step.cuh"
 #include "tc_prims.cuh"
+#include "krylov.cuh"
 
 namespace submat {
 namespace {
@@ -351,6 +353,151 @@ __device__ void vec_task(const VecTask& v) {
     }
     for (int i = gt; i < v.m; i += gn) v.u[i] = cf * (af * v.u[i] - v.t[i]);
     grp_sync<BAR>();
+  }
+}
+
+// W = M_k X for the nv <= kGroupVecs vectors x_v = X + v ld (FP64, zero-extended from m to mp) of
+// a group of rows with one pattern, all warps.  One pass over M_k's planes serves every vector:
+// the planes are decoded once (a = q0 2^10 + q1, b = q2 2^10 + q3) and two rows travel in packed
+// FP32 operations, the sums split into a part on the accumulator's grid and an exact rest, as in
+// krylov.cuh (6 operations a product, about 2^-44 of the row's norm).  sh: shared memory,
+// 8 nv mp bytes and 4 nv.
+constexpr int kGroupVecs = 12;
+__device__ __noinline__ void matvec_group(const __half* q, size_t plane, int ld, int e, const double* X, double* W,
+                             int nv, int m, int mp, float* sh) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = nwarps();
+  float* cv = sh + (size_t)2 * nv * mp;               // accumulator starts
+  for (int v = warp; v < nv; v += nw) {
+    float* xh = sh + (size_t)2 * v * mp;
+    float n2 = 0.f;
+    for (int i = lane; i < mp; i += 32) {
+      float h = 0.f, l = 0.f;
+      if (i < m) split_dbl(X[(size_t)v * ld + i], h, l);
+      xh[i] = h;
+      xh[mp + i] = l;
+      n2 = fmaf(h, h, n2);
+    }
+    n2 = warp_sum_f(n2);
+    // |sum| <= |row of a| |x|, the row's norm at most 2^(19 - e) (spectrum in (0, 1])
+    const int ex = (int)((__float_as_uint(n2) >> 23) & 0xFF) - 127;
+    if (lane == 0) cv[v] = 3.f * ldexpf(1.f, min(max(((ex + 2) >> 1) + 1 + Q0B + 10 - e, -100), 100));
+  }
+  __syncthreads();
+  const double sc = ldexp(1.0, e - Q0B - 10);
+  for (int i0 = warp * 2; i0 < m; i0 += nw * 2) {
+    kry::f2 s[kGroupVecs], c[kGroupVecs];
+#pragma unroll
+    for (int v = 0; v < kGroupVecs; ++v) {
+      const float C = v < nv ? cv[v] : 0.f;
+      s[v] = kry::pack(C, C);
+      c[v] = 0;
+    }
+    const kry::f2 minus1 = kry::pack(-1.f, -1.f);
+    const size_t r1 = (size_t)min(i0 + 1, m - 1) * ld;
+    for (int c0 = lane * 8; c0 < mp; c0 += 256) {
+      kry::f2 a[8], b[8];
+      {
+        uint4 raw[2][NSL];
+#pragma unroll
+        for (int k = 0; k < NSL; ++k) {
+          raw[0][k] = *reinterpret_cast<const uint4*>(q + k * plane + (size_t)i0 * ld + c0);
+          raw[1][k] = *reinterpret_cast<const uint4*>(q + k * plane + r1 + c0);
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          float av[2], bv[2];
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            float qq[NSL];
+#pragma unroll
+            for (int k = 0; k < NSL; ++k)
+              qq[k] = __half2float(reinterpret_cast<const __half*>(&raw[r][k])[j]);
+            av[r] = __fmaf_rn(qq[0], kRad, qq[1]);
+            bv[r] = __fmaf_rn(qq[2], kRad, qq[3]) * (kRadInv * kRadInv);
+          }
+          a[j] = kry::pack(av[0], av[1]);
+          b[j] = kry::pack(bv[0], bv[1]);
+        }
+      }
+#pragma unroll
+      for (int v = 0; v < kGroupVecs; ++v) {
+        if (v < nv) {
+          const float4* xh = reinterpret_cast<const float4*>(sh + (size_t)2 * v * mp + c0);
+          const float4* xl = reinterpret_cast<const float4*>(sh + (size_t)(2 * v + 1) * mp + c0);
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const float4 p = xh[h], t = xl[h];
+            kry::madd2(a[4 * h], b[4 * h], kry::pack(p.x, p.x), kry::pack(t.x, t.x), minus1, s[v], c[v]);
+            kry::madd2(a[4 * h + 1], b[4 * h + 1], kry::pack(p.y, p.y), kry::pack(t.y, t.y), minus1, s[v], c[v]);
+            kry::madd2(a[4 * h + 2], b[4 * h + 2], kry::pack(p.z, p.z), kry::pack(t.z, t.z), minus1, s[v], c[v]);
+            kry::madd2(a[4 * h + 3], b[4 * h + 3], kry::pack(p.w, p.w), kry::pack(t.w, t.w), minus1, s[v], c[v]);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < kGroupVecs; ++v) {
+      if (v < nv) {
+        const float C = cv[v];
+        float g0 = __fsub_rn(kry::lo32(s[v]), C), g1 = __fsub_rn(kry::hi32(s[v]), C);   // add exactly
+        float t0 = kry::lo32(c[v]), t1 = kry::hi32(c[v]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          g0 += __shfl_xor_sync(0xffffffffu, g0, o);
+          g1 += __shfl_xor_sync(0xffffffffu, g1, o);
+          t0 += __shfl_xor_sync(0xffffffffu, t0, o);
+          t1 += __shfl_xor_sync(0xffffffffu, t1, o);
+        }
+        if (lane == 0) {
+          W[(size_t)v * ld + i0] = ((double)g0 + (double)t0) * sc;
+          if (i0 + 1 < m) W[(size_t)v * ld + i0 + 1] = ((double)g1 + (double)t1) * sc;
+        }
+      }
+    }
+  }
+  __syncthreads();
+}
+
+// The carried columns of a group's other members (the first is carried as a VecTask): the step
+// T = c (alpha I - M_k), ny times, and the final Taylor polynomial (degree J), ny times.
+struct GroupVecs {
+  double *y, *a, *w;         // nv vectors each, stride ld
+  int nv, ld;
+  float* sh;
+};
+__device__ __noinline__ void group_step(const GroupVecs& g, const __half* q, size_t plane, int e, double c, double alpha,
+                           int ny, int m, int mp) {
+  for (int t = 0; t < ny; ++t) {
+    matvec_group(q, plane, g.ld, e, g.y, g.w, g.nv, m, mp, g.sh);
+    for (int v = 0; v < g.nv; ++v)
+      for (int i = threadIdx.x; i < m; i += blockDim.x) {
+        const size_t k = (size_t)v * g.ld + i;
+        g.y[k] = c * (alpha * g.y[k] - g.w[k]);
+      }
+    __syncthreads();
+  }
+}
+__device__ __noinline__ void group_final(const GroupVecs& g, const __half* q, size_t plane, int e, int J, int p, int ny,
+                            int m, int mp) {
+  for (int t = 0; t < ny; ++t) {
+    double cj[16];
+    cj[0] = 1.0;
+    for (int j = 1; j <= J; ++j) cj[j] = cj[j - 1] * (1.0 / (double)p + (double)(j - 1)) / (double)j;
+    for (int v = 0; v < g.nv; ++v)
+      for (int i = threadIdx.x; i < m; i += blockDim.x) g.a[(size_t)v * g.ld + i] = cj[J] * g.y[(size_t)v * g.ld + i];
+    __syncthreads();
+    for (int j = J - 1; j >= 0; --j) {
+      matvec_group(q, plane, g.ld, e, g.a, g.w, g.nv, m, mp, g.sh);
+      for (int v = 0; v < g.nv; ++v)
+        for (int i = threadIdx.x; i < m; i += blockDim.x) {
+          const size_t k = (size_t)v * g.ld + i;
+          g.a[k] = cj[j] * g.y[k] + (g.a[k] - g.w[k]);
+        }
+      __syncthreads();
+    }
+    for (int v = 0; v < g.nv; ++v)
+      for (int i = threadIdx.x; i < m; i += blockDim.x) g.y[(size_t)v * g.ld + i] = g.a[(size_t)v * g.ld + i];
+    __syncthreads();
   }
 }
 
@@ -1233,6 +1380,9 @@ static_assert(kVecBytes <= (size_t)SY_STAGE_AREA, "vector area must fit in the s
 // the Taylor finish's vectors follow it (3 doubles and 5 floats per entry)
 static_assert(kVecBytes + SUBMAT_MAX_M * sizeof(int2) <= (size_t)TC_STAGE_AREA,
               "the gather's row extents must fit in the idle stage area");
+static_assert(8 * (size_t)kGroupVecs * SUBMAT_MAX_M + 4 * kGroupVecs <=
+                  (size_t)TC_STAGE_AREA + TC_STAGING_BYTES - kVecBytes,
+              "a group's vectors fit in the idle stage area");
 static_assert(kVecBytes % 16 == 0, "16-byte aligned areas after the vectors");
 // tcgen05 engine: room for M_0 in FP32 after the vectors, in the idle stage and staging areas
 constexpr size_t kMfBytes = (size_t)TC_STAGE_AREA + TC_STAGING_BYTES - kVecBytes;
@@ -1240,7 +1390,9 @@ static_assert(kVecBytes + 44 * (size_t)SUBMAT_MAX_M <= (size_t)SY_STAGE_AREA &&
                   kVecBytes + 44 * (size_t)SUBMAT_MAX_M <= (size_t)TC_STAGE_AREA + TC_STAGING_BYTES,
               "finish vectors must fit in the idle stage area");
 
-template <int ENG>
+template <int ENG, bool GROUP = false>
+// GROUP: jobs of several rows of one pattern (an instance of its own: the vectors' registers
+// would spill in the GEMMs' loops of the other).
 __global__ void __launch_bounds__(ENG == ENG_TC ? TC_THREADS : kThreads,
                                   ENG == ENG_SMALL ? kSmallCtasPerSm : 1)
     fwd_mixed_kernel(const __grid_constant__ FwdArgs a) {
@@ -1314,18 +1466,26 @@ __global__ void __launch_bounds__(ENG == ENG_TC ? TC_THREADS : kThreads,
     __syncthreads();
   }
 
-  int pending = -1;          // a row taken from the queue and left unfinished by a time-out
+  // rows taken from the queue and left unfinished by a time-out: order[pending, + pending_n)
+  int pending = -1, pending_n = 0;
   for (;;) {
     if (tid == 0) job_s = atomicAdd(a.queue, 1);
     __syncthreads();
     const int idx = job_s;
     __syncthreads();
     if (idx >= n_rows) break;
+    // the job's rows (one submatrix, their own columns of its root)
+    int first = idx, members = 1;
+    if (GROUP) {
+      first = a.jobs[idx].x;
+      members = a.jobs[idx].y;
+    }
     if (*abort_s) {
-      pending = a.order[idx];
+      pending = first;
+      pending_n = members;
       break;
     }
-    const int j = a.order[idx];
+    const int j = a.order[first];
     const int m = a.m[j];
     const int pos = a.pos[j];
     const int p = a.p;
@@ -1441,6 +1601,20 @@ __global__ void __launch_bounds__(ENG == ENG_TC ? TC_THREADS : kThreads,
         yg[i] = a.sign < 0 ? ((i == pos) ? 1.0 : 0.0) : s0;
       }
     }
+    GroupVecs gv{};
+    if constexpr (GROUP) {
+      gv.nv = track ? members - 1 : 0;
+      gv.ld = LD;
+      gv.sh = reinterpret_cast<float*>(sm + kVecBytes);
+      gv.y = reinterpret_cast<double*>(reinterpret_cast<char*>(hb + vec_plane * plane) + (size_t)64 * LD);
+      gv.a = gv.y + (size_t)gv.nv * LD;
+      gv.w = gv.a + (size_t)gv.nv * LD;
+      for (int v = 0; v < gv.nv; ++v) {
+        const int pv = a.pos[a.order[first + 1 + v]];
+        for (int i = tid; i < m; i += blockDim.x)
+          gv.y[(size_t)v * LD + i] = a.sign < 0 ? (i == pv ? 1.0 : 0.0) : S[pv * m + i] * inv_lam;
+      }
+    }
     __threadfence();             // planes are read next through L2 (cp.async.cg / TMA)
     __syncthreads();
 
@@ -1531,6 +1705,8 @@ __global__ void __launch_bounds__(ENG == ENG_TC ? TC_THREADS : kThreads,
         dst = 3 - mi - dst;                     // the buffer that is neither M_k nor P_s
       }
       if (stop) break;
+      if (GROUP && gv.nv > 0)                   // M_k is still in place
+        group_step(gv, Mk.q, plane, Mk.e, (double)st.c, (double)st.alpha, ny, m, mp);
       mi = src;
       lo = st.lo_next;
       ++iters;
@@ -1543,7 +1719,8 @@ __global__ void __launch_bounds__(ENG == ENG_TC ? TC_THREADS : kThreads,
       prev2 = nrm2;
     }
     if (stop) {
-      pending = j;
+      pending = first;
+      pending_n = members;
       break;
     }
 
@@ -1609,6 +1786,16 @@ __global__ void __launch_bounds__(ENG == ENG_TC ? TC_THREADS : kThreads,
       __syncthreads();
       resid = sqrt((double)tot);
       kest = lo_raw > 0.f ? 1.f / lo_raw : 3.0e38f;
+      if (GROUP && gv.nv > 0) {
+        // the other members' columns of the same limit; the residual, a function of M_K
+        // alone but for the column, is the first member's
+        group_final(gv, B3[mi].q, plane, B3[mi].e, degree(1e-9f), p, ny, m, mp);
+        if (resid <= a.resid_tol && kest <= (float)a.kappa_max)
+          for (int v = 0; v < gv.nv; ++v) {
+            double* out = a.vals_out + a.rowptr[a.order[first + 1 + v]];
+            for (int k = tid; k < m; k += blockDim.x) out[k] = c_out * gv.y[(size_t)v * LD + k];
+          }
+      }
     } else if (!bad) {
       io.c = 1.f;                                // p = 1: X (2 I - M)
       io.alpha = 2.f;
@@ -1616,7 +1803,8 @@ __global__ void __launch_bounds__(ENG == ENG_TC ? TC_THREADS : kThreads,
       if (tid == 0) *amax_s = 0u;
       __syncthreads();
       if (!gemm(B3[mi], X[xc], X[xc ^ 1], X[xc], EPI_AMAX, nullptr)) {
-        pending = j;
+        pending = first;
+        pending_n = members;
         break;
       }
       ++n_gemm;
@@ -1640,20 +1828,20 @@ __global__ void __launch_bounds__(ENG == ENG_TC ? TC_THREADS : kThreads,
     }
     if (tid == 0) {
       if (!ok) {
-        const int slot = atomicAdd(&a.ctr->n_fallback, 1);
-        a.fallback_list[slot] = j;
+        const int slot = atomicAdd(&a.ctr->n_fallback, members);
+        for (int v = 0; v < members; ++v) a.fallback_list[slot + v] = a.order[first + v];
       }
-      if (illcond) atomicAdd(&a.ctr->n_illcond, 1ull);
+      if (illcond) atomicAdd(&a.ctr->n_illcond, (unsigned long long)members);
       atomicMax(&a.ctr->iters_max, iters);
-      atomicAdd(&a.ctr->iters_sum, (unsigned long long)iters);
+      atomicAdd(&a.ctr->iters_sum, (unsigned long long)iters * members);
       atomic_max_nonneg(&a.ctr->resid_max_bits, resid);
-      atomicAdd(&a.ctr->flops_fp64, refine_flops(m, p, a.refine_steps));
+      atomicAdd(&a.ctr->flops_fp64, members * refine_flops(m, p, a.refine_steps));
       // ten FP16 slice products per GEMM, counted with the true order m
       atomicAdd(&a.ctr->flops_tensor, (double)n_gemm * kSliceProducts * 2.0 * (double)m * m * m);
       // the method's own count: (p+1) dense products of order m per iteration (+ p = 1's
       // final X product), whatever this engine executes for them
-      atomicAdd(&a.ctr->flops_alg,
-                ((double)iters * (p + 1) + (p == 1 ? 1.0 : 0.0)) * 2.0 * (double)m * m * m);
+      atomicAdd(&a.ctr->flops_alg, members * ((double)iters * (p + 1) + (p == 1 ? 1.0 : 0.0)) *
+                                       2.0 * (double)m * m * m);
     }
     __syncthreads();
   }
@@ -1664,8 +1852,9 @@ __global__ void __launch_bounds__(ENG == ENG_TC ? TC_THREADS : kThreads,
     // the queue from now on are written as NaN (plain stores; nothing else is issued)
     if (tid == 0) atomicExch(&a.ctr->error, 1);
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
-    for (int j = pending;;) {
-      if (j >= 0) {
+    for (;;) {
+      for (int v = 0; v < pending_n; ++v) {
+        const int j = a.order[pending + v];
         double* out = a.vals_out + a.rowptr[j];
         for (int k = tid; k < a.m[j]; k += blockDim.x) out[k] = nan;
       }
@@ -1675,7 +1864,12 @@ __global__ void __launch_bounds__(ENG == ENG_TC ? TC_THREADS : kThreads,
       const int idx = job_s;
       __syncthreads();
       if (idx >= n_rows) break;
-      j = a.order[idx];
+      pending = idx;
+      pending_n = 1;
+      if (GROUP) {
+        pending = a.jobs[idx].x;
+        pending_n = a.jobs[idx].y;
+      }
     }
   }
   if (TC) {
@@ -1705,9 +1899,15 @@ cudaError_t launch_fwd_mixed(const FwdArgs& a, int grid, cudaStream_t s) {
     fwd_mixed_kernel<ENG_SYNC><<<grid, kThreads, smem_bytes<ENG_SYNC>(), s>>>(a);
   else if (a.engine == ENG_SMALL)
     fwd_mixed_kernel<ENG_SMALL><<<grid, kThreads, smem_bytes<ENG_SMALL>(), s>>>(a);
+  else if (a.jobs)
+    fwd_mixed_kernel<ENG_TC, true><<<grid, TC_THREADS, smem_bytes<ENG_TC>(), s>>>(a);
   else
     fwd_mixed_kernel<ENG_TC><<<grid, TC_THREADS, smem_bytes<ENG_TC>(), s>>>(a);
   return cudaGetLastError();
+}
+
+int mixed_group_max(int ld, int p) {   // rows that one tcgen05 job may hold (p = 1: its own only)
+  return p < 2 ? 1 : 1 + std::max(0, std::min(kGroupVecs, (2 * ld - 64) / 24));
 }
 
 int mixed_unbiased_max_m(int p) {
@@ -1722,6 +1922,9 @@ cudaError_t set_attr_mixed() {
   cudaError_t e = cudaFuncSetAttribute(fwd_mixed_kernel<ENG_TC>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem_bytes<ENG_TC>());
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(fwd_mixed_kernel<ENG_TC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)smem_bytes<ENG_TC>());
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(fwd_mixed_kernel<ENG_SMALL>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize,

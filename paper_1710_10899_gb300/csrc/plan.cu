@@ -52,7 +52,31 @@ __global__ void plan_rows_kernel(const int32_t* __restrict__ rowptr,
   if (hit < 0) atomicOr(flags, 8);
 }
 
+// same[j] = 1 when row j stores the columns of row j - 1: a warp per row.
+__global__ void same_pattern_kernel(const int32_t* __restrict__ rowptr,
+                                    const int32_t* __restrict__ colind, int32_t n,
+                                    uint8_t* __restrict__ same) {
+  const int warps = (gridDim.x * blockDim.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += warps) {
+    const int b = rowptr[r], m = rowptr[r + 1] - b;
+    bool eq = r > 0 && b - rowptr[r - 1] == m;
+    if (eq)
+      for (int k = lane; __any_sync(0xffffffffu, k < m) && eq; k += 32)
+        eq = __all_sync(0xffffffffu, k >= m || colind[b + k] == colind[b - m + k]);
+    if (lane == 0) same[r] = eq ? 1 : 0;
+  }
+}
+
 }  // namespace
+
+cudaError_t launch_same_pattern(const int32_t* rowptr, const int32_t* colind, int32_t n, uint8_t* same,
+                                cudaStream_t s) {
+  if (n == 0) return cudaSuccess;
+  const int blocks = (int)((n * 32LL + 255) / 256 < 65536 ? (n * 32LL + 255) / 256 : 65536);
+  same_pattern_kernel<<<blocks, 256, 0, s>>>(rowptr, colind, n, same);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_check_pattern(const int32_t* rowptr, const int32_t* colind, int32_t n,
                                  int32_t* flags, cudaStream_t s) {

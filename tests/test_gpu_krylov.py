@@ -172,3 +172,50 @@ def test_first_backward_under_capture(sm):
     torch.cuda.synchronize()
     gref = oracle.grad(a.rowptr, a.colind, a.vals, 2, w)
     assert np.abs(grad.cpu().numpy() - gref).max() <= 1e-10 * np.abs(gref).max()
+
+
+@pytest.mark.parametrize("p,sign", [(1, -1), (2, -1), (3, -1), (2, 1), (3, 1)])
+def test_rows_of_one_pattern(sm, p, sign):
+    """Rows that share their submatrix run as one job of the tcgen05 engine: blocks of orders
+    200..250 (every row of a block shares its pattern, so full jobs and a remainder), the mixed
+    bar on every row, and the same rows one by one (mma.sync engine) within the two bars."""
+    orders = [200, 224, 230, 250]
+    a = blocks(orders, seed=30 + p)
+    y, rep = forward(sm, a, p, precision="mixed", root_sign=sign)
+    ref = oracle.invroot(a.rowptr, a.colind, a.vals, p, sign=sign)
+    assert row_err(a, y, ref, range(a.n)) <= 1e-6
+    assert rep["n_fallback"] == 0 and rep["n_rows"] == a.n and rep["iters_sum"] >= a.n
+    z, _ = forward(sm, a, p, precision="mixed_sync", root_sign=sign)
+    assert row_err(a, y, z, range(a.n)) <= 2e-6
+
+
+def test_rows_of_one_pattern_time_out_together(sm):
+    """A pipeline wait that gives up leaves every row of its job NaN."""
+    a = blocks([200, 210], seed=41)
+    v = torch.tensor(a.vals, device="cuda")
+    plan = sm.submat_plan(a.rowptr, a.colind, 2)
+    ref = sm.submat_invroot(plan, v, sync=True).clone()
+    plan.test_stall(True)
+    out = torch.zeros_like(v)
+    with pytest.raises(sm.SubmatError) as ei:
+        sm.submat_invroot(plan, v, out, sync=True)
+    assert ei.value.name == "SUBMAT_ETIMEOUT"
+    assert torch.isnan(out).all()
+    plan.test_stall(False)
+    assert torch.equal(sm.submat_invroot(plan, v, out, sync=True), ref)
+
+
+def test_rows_of_one_pattern_not_spd(sm):
+    """A group whose submatrix is not positive definite: every member refused, others kept."""
+    a = blocks([200, 210], seed=42)
+    vals = a.vals.copy()
+    r = 200 + 17
+    d = a.rowptr[r] + int(np.nonzero(a.colind[a.rowptr[r]:a.rowptr[r + 1]] == r)[0][0])
+    vals[d] = -5.0
+    plan = sm.submat_plan(a.rowptr, a.colind, 2)
+    out = torch.zeros(a.nnz, dtype=torch.float64, device="cuda")
+    with pytest.raises(sm.SubmatError) as ei:
+        sm.submat_invroot(plan, torch.tensor(vals, device="cuda"), out, sync=True)
+    assert ei.value.name == "SUBMAT_ENOTSPD"
+    y = out.cpu().numpy()
+    assert np.isnan(y[200 * 200:]).all() and np.isfinite(y[:200 * 200]).all()
