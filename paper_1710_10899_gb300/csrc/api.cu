@@ -956,7 +956,7 @@ static submat_status pcg_impl(submat_plan_t P, const double* vals_a, const doubl
   const int32_t n = P->n;
   const size_t nd = (size_t)n;
   if (!P->d_cg) {
-    const size_t words = 6 * nd + (size_t)P->nnz + cg_dot_scratch() + 2;
+    const size_t words = 6 * nd + (size_t)P->nnz + cg_dot_scratch() + sizeof(CgResult) / sizeof(double);
     CUDA_TRY(cudaMalloc(&P->d_cg, words * sizeof(double)));
   }
   double* r = P->d_cg;
@@ -969,52 +969,37 @@ static submat_status pcg_impl(submat_plan_t P, const double* vals_a, const doubl
   double* part = kt + P->nnz;
   double* scal = part + cg_dot_scratch();
   const bool pre = vals_k != nullptr;
-  double* it_x = pre ? y : x;
   if (pre) {
     CUDA_TRY(ensure_tpos(P, s));
     CUDA_TRY(cg_transpose_vals(P->d_rowptr, P->d_colind, P->d_tpos, vals_k, kt, P->nnz, s));
-    CUDA_TRY(cg_spmv(P->d_rowptr, P->d_colind, kt, b, r, n, s));          // r = K^T b
-  } else {
-    CUDA_TRY(cudaMemcpyAsync(r, b, nd * sizeof(double), cudaMemcpyDeviceToDevice, s));
   }
-  CUDA_TRY(cudaMemsetAsync(it_x, 0, nd * sizeof(double), s));
-  CUDA_TRY(cudaMemcpyAsync(p, r, nd * sizeof(double), cudaMemcpyDeviceToDevice, s));
-  CUDA_TRY(cg_dot(r, r, n, part, scal, s));
-  double rr = 0.0;
-  CUDA_TRY(cudaMemcpyAsync(&rr, scal, sizeof(double), cudaMemcpyDeviceToHost, s));
+  CgArgs c{};
+  c.rowptr = P->d_rowptr;
+  c.colind = P->d_colind;
+  c.n = n;
+  c.max_iter = max_iter;
+  c.a = vals_a;
+  c.k = vals_k;
+  c.kt = pre ? kt : nullptr;
+  c.b = b;
+  c.x = x;
+  c.y = pre ? y : x;
+  c.r = r;
+  c.p = p;
+  c.q = q;
+  c.t1 = t1;
+  c.t2 = t2;
+  c.part = part;
+  c.tol = tol;
+  c.out = reinterpret_cast<CgResult*>(scal);
+  CUDA_TRY(cg_solve(c, P->m_max, P->n_sm, s));
+  CgResult res;
+  CUDA_TRY(cudaMemcpyAsync(&res, c.out, sizeof(res), cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaStreamSynchronize(s));
-  const double bnorm = std::sqrt(rr);
-  int32_t it = 0;
   submat_status st = SUBMAT_OK;
-  while (bnorm > 0.0 && std::sqrt(rr) > tol * bnorm && it < max_iter) {
-    if (pre) {                                                            // q = K^T A K p
-      CUDA_TRY(cg_spmv(P->d_rowptr, P->d_colind, vals_k, p, t1, n, s));
-      CUDA_TRY(cg_spmv(P->d_rowptr, P->d_colind, vals_a, t1, t2, n, s));
-      CUDA_TRY(cg_spmv(P->d_rowptr, P->d_colind, kt, t2, q, n, s));
-    } else {                                                              // q = A p
-      CUDA_TRY(cg_spmv(P->d_rowptr, P->d_colind, vals_a, p, q, n, s));
-    }
-    CUDA_TRY(cg_dot(p, q, n, part, scal, s));
-    double pq = 0.0;
-    CUDA_TRY(cudaMemcpyAsync(&pq, scal, sizeof(double), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaStreamSynchronize(s));
-    if (!(pq > 0.0) || !std::isfinite(pq)) {      // the operator is not positive definite
-      st = fail(SUBMAT_ENOTSPD, "CG: p^T A p <= 0");
-      break;
-    }
-    const double alpha = rr / pq;
-    CUDA_TRY(cg_update(alpha, it_x, r, p, q, n, part, scal + 1, s));
-    double rr_new = 0.0;
-    CUDA_TRY(cudaMemcpyAsync(&rr_new, scal + 1, sizeof(double), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaStreamSynchronize(s));
-    CUDA_TRY(cg_dir(rr_new / rr, r, p, n, s));
-    rr = rr_new;
-    ++it;
-  }
-  if (pre) CUDA_TRY(cg_spmv(P->d_rowptr, P->d_colind, vals_k, y, x, n, s));   // x = K y
-  CUDA_TRY(cudaStreamSynchronize(s));
-  if (iters) *iters = it;
-  if (rel_resid) *rel_resid = bnorm > 0.0 ? std::sqrt(rr) / bnorm : 0.0;
+  if (res.status != 0) st = fail(SUBMAT_ENOTSPD, "CG: p^T A p <= 0");
+  if (iters) *iters = res.iters;
+  if (rel_resid) *rel_resid = res.bnorm > 0.0 ? std::sqrt(res.rr) / res.bnorm : 0.0;
   P->last_stream = s;
   return st;
 }

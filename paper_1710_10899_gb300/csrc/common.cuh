@@ -118,17 +118,25 @@ cudaError_t launch_grad_gather(const int32_t* rowptr, const int32_t* colind, con
                                int32_t n, int32_t j0, int32_t j1, double* grad_in,
                                cudaStream_t s);
 
-// Conjugate-gradient pieces (cg.cu).  cg_dot / cg_update reduce in a fixed order through
-// cg_dot_scratch() doubles of part.
-cudaError_t cg_spmv(const int32_t* rowptr, const int32_t* colind, const double* vals,
-                    const double* x, double* y, int32_t n, cudaStream_t s);
+// Conjugate gradients (cg.cu) as one cooperative kernel; part: cg_dot_scratch() doubles.
+struct CgResult {
+  double rr, bnorm;          // r.r at the end, |b| (of the iterated system)
+  int32_t iters, status;     // status 1: p^T A p <= 0
+};
+struct CgArgs {
+  const int32_t* rowptr;
+  const int32_t* colind;
+  int32_t n, max_iter;
+  const double *a, *k, *kt;  // A; K and K^T (null: plain)
+  const double* b;
+  double *x, *y;             // solution; the iterate (x itself without K)
+  double *r, *p, *q, *t1, *t2, *part;
+  double tol;
+  CgResult* out;
+};
+cudaError_t cg_solve(const CgArgs& a, int m_max, int n_sm, cudaStream_t s);
 cudaError_t cg_transpose_vals(const int32_t* rowptr, const int32_t* colind, const int32_t* tpos,
                               const double* vals, double* kt, int64_t nnz, cudaStream_t s);
-cudaError_t cg_dot(const double* x, const double* y, int32_t n, double* part, double* out,
-                   cudaStream_t s);
-cudaError_t cg_update(double alpha, double* x, double* r, const double* p, const double* q,
-                      int32_t n, double* part, double* rr, cudaStream_t s);
-cudaError_t cg_dir(double beta, const double* r, double* p, int32_t n, cudaStream_t s);
 size_t cg_dot_scratch();
 
 // Global refinement pieces (refine_global.cu): C = (L R) restricted to the pattern, R given

@@ -75,3 +75,27 @@ def test_cg_not_positive_definite(sm):
     with pytest.raises(sm.SubmatError) as ei:
         sm.submat_pcg(plan, v)
     assert ei.value.name == "SUBMAT_ENOTSPD"
+
+
+@pytest.mark.parametrize("n,width", [(1, 0), (255, 1), (257, 3), (3000, 4), (70001, 1), (700, 5)])
+def test_cg_sizes_and_row_lengths(sm, n, width):
+    """One row, sizes around a reduction block and beyond one sweep of them (65536 elements), and
+    rows of at most 8 entries (a thread each) or more (a warp each), against the CG oracle."""
+    import scipy.sparse as sp
+    rng = np.random.default_rng(n)
+    m = sp.diags([np.full(n, 2.5)] + [np.full(n - k, -1.0 / width) for k in range(1, width + 1) if k < n]
+                 + [np.full(n - k, -1.0 / width) for k in range(1, width + 1) if k < n],
+                 [0] + [k for k in range(1, width + 1) if k < n] + [-k for k in range(1, width + 1) if k < n]).tocsr()
+    m.sort_indices()
+    rp, ci, vals = sm.csr_arrays(m)
+    b = rng.standard_normal(n)
+    plan = sm.submat_plan(rp, ci, 2, precision="fp64")
+    v = torch.tensor(vals, device="cuda")
+    k = sm.submat_invroot(plan, v)
+    for vk in (None, k):
+        x, it, rel = sm.submat_pcg(plan, v, torch.tensor(b, device="cuda"), vals_k=vk)
+        kk = vk.cpu().numpy() if vk is not None else None
+        xo, ito, relo, _ = oracle.cg.solve(rp, ci, vals, b, vals_k=kk)
+        assert _close_iters(it, ito) and rel <= 1e-6
+        # both stop at 1e-6 of the right-hand side; kappa <= (2.5 + 2) / 0.5 = 9
+        assert np.linalg.norm(x.cpu().numpy() - xo) <= 2e-5 * np.linalg.norm(xo)
