@@ -65,11 +65,12 @@ typedef enum {
  *
  * Only column pos of each root is kept, so rows whose spectrum allows it take a Krylov method
  * for that column (Lanczos and a quadrature of the root, O(k m^2) instead of O(m^3)): in FP64
- * mode every order, in FP64 arithmetic; in MIXED_F16 mode, p >= 2, orders up to 192 with
- * double-float arithmetic (FP32 pairs).  A row that it refuses (lambda_bar / lambda_min above
- * 2000, or above kappa_max in the mixed mode; not positive definite) and every row of a plan
- * whose options steer the coupled iteration (k_max, tol, refine_steps, size buckets) takes the
- * coupled iteration.
+ * mode every order, in FP64 arithmetic; in MIXED_F16 mode with double-float arithmetic (FP32
+ * pairs) orders up to 192 for p = 2 (up to 160 for p = 3, none beyond) and every order for p = 1,
+ * whose column is then refined in FP64.  A row that it refuses
+ * (lambda_bar / lambda_min above 2000; not positive definite) and every row of a plan whose
+ * options steer the coupled iteration (k_max, tol, refine_steps, kappa_max, size buckets) takes
+ * the coupled iteration.
  */
 enum {
   SUBMAT_PREC_FP64 = 0,       /* everything in FP64 (CUDA cores)                            */
@@ -107,7 +108,7 @@ typedef struct {
                               step amplifies the part of the error that does not commute
                               with S_j); < 0 selects the default                          */
   int32_t use_graph;       /* capture the forward launches into a CUDA graph; default 1  */
-  double kappa_max;        /* mixed path: a row whose condition estimate
+  double kappa_max;        /* coupled iteration, mixed path: a row whose condition estimate
                               lambda_bar / lambda_min (power iteration on the converged
                               iterate) exceeds this goes to the FP64 fallback; default 100 */
   int32_t root_sign;       /* -1 (default): the inverse p-th root A^(-1/p); +1: the positive

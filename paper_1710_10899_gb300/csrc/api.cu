@@ -224,7 +224,6 @@ kry::Args krylov_args(submat_plan_t P, const EngineRun& run, const double* in, d
   k.nb = run.cls.nb;
   k.ns = run.cls.ns;
   k.resid_tol = P->opts.resid_tol;
-  k.kappa_max = P->opts.kappa_max;
   k.fp64 = P->opts.precision == SUBMAT_PREC_FP64 ? 1 : 0;
   k.nodes = P->nodes;
   return k;
@@ -379,16 +378,15 @@ const char* submat_status_string(submat_status s) {
 
 const char* submat_last_error(void) { return g_last_error.c_str(); }
 
-// Largest order the Krylov engine takes.  FP64: every order.  Mixed p = 1 keeps the iteration
-// with its FP64 refinement.  Mixed p >= 2: the orders up to kKrylovMixedMax whose slice
+// Largest order the Krylov engine takes.  FP64, and mixed p = 1 (which it refines to FP64
+// accuracy): every order.  Mixed p >= 2: the orders up to kKrylovMixedMax whose slice
 // arithmetic has no exponent bias; there the tcgen05 engine's result is within 1e-9 of the exact
 // one, so the two engines agree to that; beyond, its rounding grows to 7e-9 (order 240) and
 // 3e-8 (order 800) and the rows keep it.
 constexpr int kKrylovMixedMax = 192;
 static int krylov_max_m(int precision, int p) {
   if (precision == SUBMAT_PREC_MIXED_F16_SYNC || p > SUBMAT_MIXED_MAX_P) return 0;
-  if (precision == SUBMAT_PREC_FP64) return SUBMAT_MAX_M;
-  if (p == 1) return 0;
+  if (precision == SUBMAT_PREC_FP64 || p == 1) return SUBMAT_MAX_M;
   return std::min(kKrylovMixedMax, mixed_unbiased_max_m(p));
 }
 
@@ -599,9 +597,10 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
   // engine runs: the plan's rows are ordered by decreasing m, so each size bucket is one
   // contiguous run of the order
   size_t scratch_bytes = stride * (size_t)P->grid;
-  const bool steered = opts && (opts->k_max >= 1 && opts->k_max != 40 || opts->tol > 0.0 ||
-                                opts->refine_steps >= 0 || o.small_max_m != kTunedSmallMaxM ||
-                                o.sync_max_m != kTunedSyncMaxM);
+  // options that steer the coupled iteration, its refinement or its fallback keep it
+  const bool steered = opts && ((opts->k_max >= 1 && opts->k_max != 40) || opts->tol > 0.0 ||
+                                opts->refine_steps >= 0 || o.kappa_max != 100.0 ||
+                                o.small_max_m != kTunedSmallMaxM || o.sync_max_m != kTunedSyncMaxM);
   const int kry_max = steered ? 0 : krylov_max_m(o.precision, p);
   // (the inverse's adjoint stays with the Jacobi kernel, whose error there is the smaller one)
   const bool kry_bwd = p <= SUBMAT_MIXED_MAX_P && (p > 1 || o.root_sign > 0);

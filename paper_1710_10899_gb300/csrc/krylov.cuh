@@ -89,7 +89,7 @@ struct Args {
   size_t stride;                           // bytes per CTA
   int32_t nb;                              // blocks per edge of the class
   int32_t ns;                              // blocks of S held in shared memory
-  double resid_tol, kappa_max;
+  double resid_tol;
   int32_t fp64;
   Nodes nodes;
   // backward
@@ -242,6 +242,22 @@ __device__ __forceinline__ double join(double a) { return a; }
 __device__ __forceinline__ double as(float x, double*) { return (double)x; }
 __device__ __forceinline__ double as(double x, double*) { return x; }
 
+// Single precision: the correction of a refined column.
+__device__ __forceinline__ float add(float a, float b) { return a + b; }
+__device__ __forceinline__ float sub(float a, float b) { return a - b; }
+__device__ __forceinline__ float neg(float a) { return -a; }
+__device__ __forceinline__ float mul(float a, float b) { return a * b; }
+__device__ __forceinline__ float rcp(float a) { return __frcp_rn(a); }
+__device__ __forceinline__ float inv_sqrt(float a) { return rsqrtf(a); }
+__device__ __forceinline__ float shfl_xor(float a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ float hi(float a) { return a; }
+__device__ __forceinline__ double join(float a) { return (double)a; }
+__device__ __forceinline__ float as(float x, float*) { return x; }
+__device__ __forceinline__ float as(double x, float*) { return (float)x; }
+
+template <class T> constexpr bool kDf = false;
+template <> constexpr bool kDf<df> = true;
+
 template <class T> __device__ __forceinline__ T zero() { return as(0.f, (T*)nullptr); }
 template <class T> __device__ __forceinline__ T one() { return as(1.f, (T*)nullptr); }
 
@@ -292,6 +308,7 @@ __device__ __forceinline__ df warp_total(df a) {
   return a;
 }
 __device__ __forceinline__ double warp_total(double a) { return warp_sum(a); }
+__device__ __forceinline__ float warp_total(float a) { return warp_sum_f(a); }
 
 // Sum of the first n warps' totals in red, the same on every thread (lane w reads warp w's).
 template <int NW, class T> __device__ __forceinline__ T total_of(const T* red, int lane, int n) {
@@ -465,6 +482,41 @@ __device__ __forceinline__ void block_mul(const float4* blk4, const double* v, i
   }
 }
 
+// Single precision, from the leading parts of a double-float block.
+template <bool OFF>
+__device__ __forceinline__ void block_mul(const float4* blk, const float* v, int I, int J, float, float* part,
+                                          int mp, int lane, float& dot) {
+  const int a = lane >> 2, b = lane & 3;
+  const ulonglong2* ch = reinterpret_cast<const ulonglong2*>(v + J * kB + b * 8);
+  const ulonglong2 h0 = ch[0], h1 = ch[1];
+  const f2 vc[4] = {h0.x, h0.y, h1.x, h1.y};
+  f2 rs[4] = {}, cs[4] = {}, vr[4];
+  const float4 xr = *reinterpret_cast<const float4*>(v + I * kB + a * 4);
+  vr[0] = pack(xr.x, xr.x), vr[1] = pack(xr.y, xr.y), vr[2] = pack(xr.z, xr.z), vr[3] = pack(xr.w, xr.w);
+  const ulonglong2* e = reinterpret_cast<const ulonglong2*>(blk) + lane;
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const f2 x = e[(i * 4 + j) * 32].x;
+      rs[i] = fma2(x, vc[j], rs[i]);
+      if (OFF) cs[j] = fma2(x, vr[i], cs[j]);
+    }
+  float s4[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) s4[i] = lo32(rs[i]) + hi32(rs[i]);
+  const float s = lane_rows(s4, lane);
+  part[J * mp + I * kB + lane] = s;
+  dot = fmaf(OFF ? 2.f * s : s, v[I * kB + lane], dot);
+  if (OFF) {
+    float s8[8];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) s8[2 * j] = lo32(cs[j]), s8[2 * j + 1] = hi32(cs[j]);
+    const float t = lane_cols(s8, lane);
+    part[I * mp + J * kB + b * 8 + a] = t;
+  }
+}
+
 __device__ __forceinline__ void elem_hi(const float4& x, float& a, float& b, df*) { a = x.x; b = x.y; }
 __device__ __forceinline__ void elem_hi(const float4& x, float& a, float& b, double*) {
   const double2 d = *reinterpret_cast<const double2*>(&x);
@@ -521,7 +573,7 @@ struct Row {
                                 // certified lower end
   __device__ __forceinline__ T* v() const { return reinterpret_cast<T*>(kry_smem + kF.v); }
   __device__ __forceinline__ T v_at(int i) const {
-    if constexpr (__is_same(T, double)) {
+    if constexpr (!kDf<T>) {
       return v()[i];
     } else {
       const float* h = reinterpret_cast<const float*>(kry_smem + kF.v);
@@ -529,7 +581,7 @@ struct Row {
     }
   }
   __device__ __forceinline__ void set_v(int i, T x) const {
-    if constexpr (__is_same(T, double)) {
+    if constexpr (!kDf<T>) {
       v()[i] = x;
     } else {
       float* h = reinterpret_cast<float*>(kry_smem + kF.v);
@@ -539,7 +591,7 @@ struct Row {
   }
   // node solution k of node q (a double-float row: 32 leading, then 32 trailing parts)
   __device__ __forceinline__ T x_at(int k, int q) const {
-    if constexpr (__is_same(T, double)) {
+    if constexpr (!kDf<T>) {
       return X[(size_t)k * kNodes + q];
     } else {
       const float* h = reinterpret_cast<const float*>(X + (size_t)k * kNodes);
@@ -547,7 +599,7 @@ struct Row {
     }
   }
   __device__ __forceinline__ void set_x(int k, int q, T x) const {
-    if constexpr (__is_same(T, double)) {
+    if constexpr (!kDf<T>) {
       X[(size_t)k * kNodes + q] = x;
     } else {
       float* h = reinterpret_cast<float*>(X + (size_t)k * kNodes);
@@ -750,7 +802,7 @@ __device__ __forceinline__ void for_blocks(const Row<T, NW, GP, ALL, BWD>& r, in
 
 // Gershgorin bound, accumulator start and certified lower end.
 template <class T, int NW, bool GP, bool ALL, bool BWD>
-__device__ void stats(Row<T, NW, GP, ALL, BWD>& r, double kappa_max) {
+__device__ void stats(Row<T, NW, GP, ALL, BWD>& r) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float2* p2 = reinterpret_cast<float2*>(r.part());
   if (warp < NW)
@@ -795,7 +847,7 @@ __device__ void stats(Row<T, NW, GP, ALL, BWD>& r, double kappa_max) {
   int ex = ((__float_as_int(norm) >> 23) & 0xFF) + 1;      // 2^(ex - 127) > norm
   ex = min(max(ex, 1), 250);
   r.C = 3.f * __int_as_float(ex << 23);
-  r.sigma = r.lam / (kappa_max > 0.0 ? fminf(kKappa, (float)kappa_max) : kKappa);
+  r.sigma = r.lam / kKappa;
   sync_all<NW>();
 }
 
@@ -869,14 +921,14 @@ template <int NW, class T> __device__ __forceinline__ T row_sum(const T* part, i
   T s = part[i];
   for (int x = 1; x < nb; ++x) {
     const T q = part[x * mp + i];
-    if constexpr (__is_same(T, double)) {
+    if constexpr (!kDf<T>) {
       s += q;
     } else {                                          // grid parts add exactly
       s.h += q.h;
       s.l += q.l;
     }
   }
-  if constexpr (!__is_same(T, double)) s = quick(s.h, s.l);
+  if constexpr (kDf<T>) s = quick(s.h, s.l);
   return s;
 }
 
@@ -1179,6 +1231,36 @@ __device__ bool cholesky(const Row<T, NW, GP, ALL, BWD>& r) {
     sync_mat<NW>();
   }
   return *bad == 0;
+}
+
+// r = e_pos - S x in FP64 for x (FP64, r.m entries, in the units of the values): the pattern rows
+// are read again, in full, and their entries' columns found as in the gather.  All warps.
+template <class T, int NW, bool GP, bool ALL, bool BWD>
+__device__ void residual(const Row<T, NW, GP, ALL, BWD>& r, const Args& a, const double* x, double* out) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int NWALL = threads_of<NW>() / 32;
+  const Buckets bk = make_buckets(r);
+  constexpr int U = 4;
+  for (int k = warp; k < r.m; k += NWALL) {
+    const int e1 = r.ext()[k].y;
+    double s = 0.0;
+    for (int e0 = a.rowptr[r.R()[k]]; e0 < e1; e0 += 32 * U) {
+      int col[U], l[U];
+      double v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int e = e0 + u * 32 + lane;
+        col[u] = e < e1 ? a.colind[e] : -1;
+        v[u] = e < e1 ? a.vals[e] : 0.0;
+      }
+      find_cols<U>(r, bk, col, l);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (l[u] >= 0) s = fma(v[u], x[l[u]], s);
+    }
+    s = warp_sum(s);
+    if (lane == 0) out[k] = (k == r.pos ? 1.0 : 0.0) - s;
+  }
 }
 
 // Steps that the coupled iteration would take on spec(M) in [lo, 1] (reported as the row's

@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) bwd_kernel(const __gri
     float lo = 1.f;
     T gnorm = one<T>();
     if (ok) {
-      stats(r, 0.0);
+      stats(r);
       if (!direct && !none) {
         float est0 = 0.f, est1 = 0.f, lo0 = 0.f, lo1 = 0.f;
         for (int i = tid; i < r.mp; i += NT) r.set_v(i, i == r.pos ? one<T>() : zero<T>());
