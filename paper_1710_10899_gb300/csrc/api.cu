@@ -413,7 +413,7 @@ static std::vector<EngineRun> plan_runs(submat_plan_t P, const std::vector<int32
     run.begin = i;
     run.count = e - i;
     if (run.engine == kEngineKrylov) {
-      run.cls = kry::make_class(b - kEngineKrylov, sizes[i], false);
+      run.cls = kry::make_class(b - kEngineKrylov, sizes[i], run.count, P->n_sm, false);
       run.grid = std::min(P->n_sm * run.cls.ctas, run.count);
       run.stride = kry::layout(run.cls.nb, run.cls.ns, run.cls.nw, run.cls.part_smem, false).g_total;
       run.scratch_off = off;
@@ -663,7 +663,7 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
       run.engine = kEngineKrylov;
       run.begin = i;
       run.count = e - i;
-      run.cls = kry::make_class(b, sizes[i], true);
+      run.cls = kry::make_class(b, sizes[i], run.count, P->n_sm, true);
       run.grid = std::min(P->n_sm * run.cls.ctas, run.count);
       run.stride = kry::layout(run.cls.nb, run.cls.ns, run.cls.nw, run.cls.part_smem, true).g_total;
       run.scratch_off = P->bwd_bytes;

@@ -163,10 +163,10 @@ __host__ __device__ inline Layout layout(int nb, int ns, int nw, bool part_smem,
 bool cached_nodes(int p, int sign, Nodes* out);
 struct Class {
   int max_m = 0, nw = 0, nb = 0, ns = 0, ctas = 0;
-  bool part_smem = true;
+  bool part_smem = true, lone = false;     // lone: one warp in both roles
 };
 int class_of(int m);                       // class index of a row of order m
-Class make_class(int index, int m_max, bool bwd);
+Class make_class(int index, int m_max, int rows, int n_sm, bool bwd);
 cudaError_t launch_fwd(const Args& a, const Class& c, int grid, cudaStream_t s);
 cudaError_t launch_bwd(const Args& a, const Class& c, int grid, cudaStream_t s);
 cudaError_t set_attr_fwd();
@@ -287,14 +287,19 @@ __device__ __forceinline__ df scaled(double v, int e0, df*) {
 }
 
 // ---- barriers ---------------------------------------------------------------------------
-template <int NW> __device__ __forceinline__ void sync_all() {
-  if constexpr (NW == 1) __syncwarp(); else __syncthreads();
+// One matrix warp comes in two forms: with a node warp beside it (lower latency of a row), or, as
+// ALL = false, alone with both roles (more rows per SM).
+template <int NW, bool ALL> constexpr bool kLone = NW == 1 && !ALL;
+template <int NW, bool ALL> __device__ __forceinline__ void sync_all() {
+  if constexpr (kLone<NW, ALL>) __syncwarp(); else __syncthreads();
 }
 template <int NW> __device__ __forceinline__ void sync_mat() {   // the NW matrix warps only
   if constexpr (NW == 1) __syncwarp();
   else asm volatile("bar.sync 1, %0;" ::"n"(NW * 32) : "memory");
 }
-template <int NW> __host__ __device__ constexpr int threads_of() { return NW == 1 ? 32 : NW * 32 + 32; }
+template <int NW, bool ALL> __host__ __device__ constexpr int threads_of() {
+  return NW * 32 + (NW == 1 && !ALL ? 0 : 32);
+}
 
 // Sum over a warp (every lane gets it); double-floats as unnormalised pairs between levels.
 __device__ __forceinline__ df warp_total(df a) {
@@ -642,8 +647,8 @@ __device__ __forceinline__ void bind(Row<T, NW, GP, ALL, BWD>& r, const Args& a)
   r.gpart = reinterpret_cast<T*>(scr + L.g_part);
   r.V = reinterpret_cast<T*>(scr + L.g_v);
   r.X = reinterpret_cast<T*>(scr + L.g_x);
-  r.AB = ALL ? r.sblk() : reinterpret_cast<float4*>(scr + L.g_ab);
-  for (int q = threadIdx.x; q < kNodesAll; q += threads_of<NW>()) {
+  r.AB = ALL || NW == 1 ? r.sblk() : reinterpret_cast<float4*>(scr + L.g_ab);
+  for (int q = threadIdx.x; q < kNodesAll; q += threads_of<NW, ALL>()) {
     r.nodes()[q] = a.nodes.theta[q];
     r.nodes()[kNodesAll + q] = a.nodes.w[q];
   }
@@ -670,7 +675,7 @@ __device__ __forceinline__ Buckets make_buckets(const Row<T, NW, GP, ALL, BWD>& 
 // r.bk()[b] = first position whose bucket is at least b (b <= kBuckets).
 template <class T, int NW, bool GP, bool ALL, bool BWD>
 __device__ __forceinline__ void fill_buckets(const Row<T, NW, GP, ALL, BWD>& r, const Buckets& k) {
-  for (int i = threadIdx.x; i <= r.m; i += threads_of<NW>()) {
+  for (int i = threadIdx.x; i <= r.m; i += threads_of<NW, ALL>()) {
     const int b0 = i == 0 ? 0 : (int)k.of(r.R()[i - 1]) + 1;
     const int b1 = i == r.m ? kBuckets : (int)k.of(r.R()[i]);
     for (int b = b0; b <= b1; ++b) r.bk()[b] = (uint16_t)i;
@@ -707,7 +712,7 @@ __device__ __forceinline__ void find_cols(const Row<T, NW, GP, ALL, BWD>& r, con
 // is not a positive normal number.
 template <class T, int NW, bool GP, bool ALL, bool BWD>
 __device__ bool gather(Row<T, NW, GP, ALL, BWD>& r, const Args& a) {
-  constexpr int NT = threads_of<NW>();
+  constexpr int NT = threads_of<NW, ALL>();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int base = a.rowptr[r.j], m = r.m;
   int mx = 0, mn = 0x7fffffff;                       // high words of the diagonal entries
@@ -732,7 +737,7 @@ __device__ bool gather(Row<T, NW, GP, ALL, BWD>& r, const Args& a) {
     ired[2 * warp] = mx;
     ired[2 * warp + 1] = mn;
   }
-  sync_all<NW>();
+  sync_all<NW, ALL>();
   const Buckets bk = make_buckets(r);
   fill_buckets(r, bk);
 #pragma unroll
@@ -741,7 +746,7 @@ __device__ bool gather(Row<T, NW, GP, ALL, BWD>& r, const Args& a) {
     mn = min(mn, ired[2 * w + 1]);
   }
   r.e0 = mx >> 20;
-  sync_all<NW>();
+  sync_all<NW, ALL>();
   if (mn <= 0x00100000 || r.e0 < 64 || r.e0 >= 0x7FF - 64) return false;
   constexpr int U = 4;                               // 128 entries of a pattern row in flight
   int ncol[U];
@@ -782,7 +787,7 @@ __device__ bool gather(Row<T, NW, GP, ALL, BWD>& r, const Args& a) {
       load(e0, e1, col, v);
     }
   }
-  sync_all<NW>();
+  sync_all<NW, ALL>();
   return true;
 }
 
@@ -810,7 +815,7 @@ __device__ void stats(Row<T, NW, GP, ALL, BWD>& r) {
       if (ALL || t < r.ns) block_stats<T>(r.sblk(t), I, J, p2, r.mp, lane);
       else block_stats<T>(r.gblk_at(t), I, J, p2, r.mp, lane);
     });
-  sync_all<NW>();
+  sync_all<NW, ALL>();
   float lam = 0.f, nu = 0.f;
   if (warp < NW)
     for (int i = tid; i < r.mp; i += NW * 32) {
@@ -834,8 +839,8 @@ __device__ void stats(Row<T, NW, GP, ALL, BWD>& r) {
     fred[2 * warp] = lam;
     fred[2 * warp + 1] = nu;
   }
-  sync_all<NW>();
-  constexpr int NWALL = threads_of<NW>() / 32;
+  sync_all<NW, ALL>();
+  constexpr int NWALL = threads_of<NW, ALL>() / 32;
 #pragma unroll
   for (int w = 0; w < NWALL; ++w) {
     const float s = fred[2 * w];
@@ -848,7 +853,7 @@ __device__ void stats(Row<T, NW, GP, ALL, BWD>& r) {
   ex = min(max(ex, 1), 250);
   r.C = 3.f * __int_as_float(ex << 23);
   r.sigma = r.lam / kKappa;
-  sync_all<NW>();
+  sync_all<NW, ALL>();
 }
 
 // Node state of the stopping bound (node warp: lane = node) and a Sturm sequence at the
@@ -937,7 +942,7 @@ __device__ int lanczos(const Row<T, NW, GP, ALL, BWD>& r, int p, int sign, float
   constexpr int cap = cap_of(NW);
   constexpr int NM = NW * 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const bool mat = warp < NW, node = NW == 1 || warp == NW;
+  const bool mat = warp < NW, node = kLone<NW, ALL> || warp == NW;
   T w[NE], vp[NE];
 #pragma unroll
   for (int e = 0; e < NE; ++e) {
@@ -984,7 +989,7 @@ __device__ int lanczos(const Row<T, NW, GP, ALL, BWD>& r, int p, int sign, float
         r.flag()[0] = !(bound > tol) || k >= cap;
       }
     }
-    sync_all<NW>();
+    sync_all<NW, ALL>();
     const bool stop = k > 0 && r.flag()[0];
     if (warp < nv) {
       const T al = mul(mul(total_of<NW>(r.red(), lane, NW), inv), inv);
@@ -1011,9 +1016,9 @@ __device__ int lanczos(const Row<T, NW, GP, ALL, BWD>& r, int p, int sign, float
       }
     }
     if (stop) break;
-    sync_all<NW>();
+    sync_all<NW, ALL>();
   }
-  sync_all<NW>();
+  sync_all<NW, ALL>();
   if (node) {
     *est = bound;
     *lo = node_lo(ns);
@@ -1238,7 +1243,7 @@ __device__ bool cholesky(const Row<T, NW, GP, ALL, BWD>& r) {
 template <class T, int NW, bool GP, bool ALL, bool BWD>
 __device__ void residual(const Row<T, NW, GP, ALL, BWD>& r, const Args& a, const double* x, double* out) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int NWALL = threads_of<NW>() / 32;
+  constexpr int NWALL = threads_of<NW, ALL>() / 32;
   const Buckets bk = make_buckets(r);
   constexpr int U = 4;
   for (int k = warp; k < r.m; k += NWALL) {

@@ -63,12 +63,12 @@ __device__ void solve_nodes(Row<df, NW, GP, ALL, true>& r, const Args& a, int K0
 }
 
 template <int NW, bool GP, bool ALL, int NE, int MINB>
-__global__ void __launch_bounds__(threads_of<NW>(), MINB) bwd_kernel(const __grid_constant__ Args a) {
+__global__ void __launch_bounds__(threads_of<NW, ALL>(), MINB) bwd_kernel(const __grid_constant__ Args a) {
   typedef df T;
-  constexpr int NT = threads_of<NW>();
+  constexpr int NT = threads_of<NW, ALL>();
   constexpr int NM = NW * 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const bool mat = warp < NW, node = NW == 1 || warp == NW;
+  const bool mat = warp < NW, node = kLone<NW, ALL> || warp == NW;
   Row<T, NW, GP, ALL, true> r;
   bind(r, a);
   const Layout L = layout(a.nb, a.ns, NW, !GP, true);
@@ -84,9 +84,9 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) bwd_kernel(const __gri
       r.flag()[2] = atomicAdd(a.queue, 1);
       r.flag()[1] = 0;
     }
-    sync_all<NW>();
+    sync_all<NW, ALL>();
     const int idx = r.flag()[2];
-    sync_all<NW>();
+    sync_all<NW, ALL>();
     if (idx >= a.n) break;
     r.j = a.order[idx];
     if (a.gbuf && (r.j < a.j0 || r.j >= a.j1)) continue;     // another wave's row
@@ -102,13 +102,13 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) bwd_kernel(const __gri
       eg = max(eg, __double2hiint(a.grad_out[base + i]) & 0x7FFFFFFF);
     eg = __reduce_max_sync(0xffffffffu, eg);
     int* ired = reinterpret_cast<int*>(r.red());
-    sync_all<NW>();
+    sync_all<NW, ALL>();
     if (lane == 0) ired[warp] = eg;
-    sync_all<NW>();
+    sync_all<NW, ALL>();
 #pragma unroll
     for (int w = 0; w < NT / 32; ++w) eg = max(eg, ired[w]);
     eg >>= 20;
-    sync_all<NW>();
+    sync_all<NW, ALL>();
     const bool none = eg == 0;                       // g = 0: no contribution
     ok = ok && eg < 0x7FF - 64 && (none || eg >= 64);
     int K0 = 0, K1 = 0, Q = 1, passes = 1;
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) bwd_kernel(const __gri
       if (!direct && !none) {
         float est0 = 0.f, est1 = 0.f, lo0 = 0.f, lo1 = 0.f;
         for (int i = tid; i < r.mp; i += NT) r.set_v(i, i == r.pos ? one<T>() : zero<T>());
-        sync_all<NW>();
+        sync_all<NW, ALL>();
         K0 = lanczos<NE>(r, p, a.sign, kTolGrad, &est0, &lo0);
         T n2 = zero<T>();
         for (int i = tid; i < r.mp; i += NT) {
@@ -129,14 +129,14 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) bwd_kernel(const __gri
         }
         n2 = warp_total(n2);
         if (lane == 0) r.red()[warp] = n2;
-        sync_all<NW>();
+        sync_all<NW, ALL>();
         n2 = total_of<NT / 32>(r.red(), lane, NT / 32);
         const T inv = inv_sqrt(n2);
         gnorm = mul(n2, inv);
         for (int i = tid; i < r.mp; i += NT) r.set_v(i, mul(r.v_at(i), inv));
         r.V = V1;
         r.o_t += t_bytes;
-        sync_all<NW>();
+        sync_all<NW, ALL>();
         K1 = lanczos<NE>(r, p, a.sign, kTolGrad, &est1, &lo1);
         if (node) {
           lo = fminf(lo0, lo1);
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) bwd_kernel(const __gri
         r.flag()[6] = 1;
       }
       if (mat) cholesky(r);
-      sync_all<NW>();
+      sync_all<NW, ALL>();
       Q = r.flag()[3];
       lo = __int_as_float(r.flag()[4]);
       passes = r.flag()[6];
@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) bwd_kernel(const __gri
     }
     if (!ok) {
       if (tid == 0) a.redo_list[atomicAdd(&a.ctr->n_redo, 1)] = r.j;
-      sync_all<NW>();
+      sync_all<NW, ALL>();
       continue;
     }
     if (none) {
@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) bwd_kernel(const __gri
         double* gj = a.gbuf + (a.gofs[r.j] - a.gofs[a.j0]);
         for (int e = tid; e < r.m * r.m; e += NT) gj[e] = 0.0;
       }
-      sync_all<NW>();
+      sync_all<NW, ALL>();
       continue;
     }
     const Buckets bk = make_buckets(r);
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) bwd_kernel(const __gri
         r.V = V0;
         r.o_t -= t_bytes;
       }
-      sync_all<NW>();
+      sync_all<NW, ALL>();
     }
     const int shift = r.flag()[5];
     float* AB = reinterpret_cast<float*>(r.AB);
@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) bwd_kernel(const __gri
         }
       }
     }
-    sync_all<NW>();
+    sync_all<NW, ALL>();
     // G(k, l) over the stored entries of the upper triangle
     for (int k = warp; k < r.m; k += NT / 32) {
       const int e1 = r.ext()[k].y;
@@ -290,21 +290,21 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) bwd_kernel(const __gri
         }
       }
     }
-    sync_all<NW>();
+    sync_all<NW, ALL>();
     }
     if (tid == 0) {
       const double m2 = (double)r.m * r.m;
       atomicAdd(&a.ctr->flops_fp64, 2.0 * m2 * (double)(K0 + K1) + 4.0 * m2 * Q * passes);
     }
-    sync_all<NW>();
+    sync_all<NW, ALL>();
   }
 }
 
 template <int NW, bool GP, bool ALL, int NE, int MINB>
 cudaError_t run(const Args& a, int grid, cudaStream_t s) {
   const Layout L = layout(a.nb, a.ns, NW, !GP, true);
-  if ((ALL && a.ns < nblocks(a.nb)) || L.total > kMaxSmem) return cudaErrorInvalidValue;
-  bwd_kernel<NW, GP, ALL, NE, MINB><<<grid, threads_of<NW>(), L.total, s>>>(a);
+  if (((ALL || NW == 1) && a.ns < nblocks(a.nb)) || L.total > kMaxSmem) return cudaErrorInvalidValue;
+  bwd_kernel<NW, GP, ALL, NE, MINB><<<grid, threads_of<NW, ALL>(), L.total, s>>>(a);
   return cudaGetLastError();
 }
 template <int NW, bool GP, bool ALL, int NE, int MINB>
@@ -317,7 +317,7 @@ cudaError_t attr() {
 
 cudaError_t launch_bwd(const Args& a, const Class& c, int grid, cudaStream_t s) {
   switch (c.nw) {
-    case 1: return run<1, false, true, 1, 8>(a, grid, s);
+    case 1: return c.lone ? run<1, false, false, 1, 8>(a, grid, s) : run<1, false, true, 1, 8>(a, grid, s);
     case 3: return run<3, false, true, 1, 4>(a, grid, s);
     case 5: return run<5, false, true, 1, 2>(a, grid, s);
   }
@@ -328,6 +328,7 @@ cudaError_t launch_bwd(const Args& a, const Class& c, int grid, cudaStream_t s) 
 cudaError_t set_attr_bwd() {
   cudaError_t e;
   if ((e = attr<1, false, true, 1, 8>()) != cudaSuccess) return e;
+  if ((e = attr<1, false, false, 1, 8>()) != cudaSuccess) return e;
   if ((e = attr<3, false, true, 1, 4>()) != cudaSuccess) return e;
   if ((e = attr<5, false, true, 1, 2>()) != cudaSuccess) return e;
   if ((e = attr<15, false, true, 1, 1>()) != cudaSuccess) return e;

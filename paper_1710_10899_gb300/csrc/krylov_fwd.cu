@@ -22,11 +22,11 @@ template <> struct Tol<double> { static constexpr float value = 2e-16f; };
 constexpr float kTolFix = 3e-4f;
 
 template <class T, int NW, bool GP, bool ALL, int NE, int MINB>
-__global__ void __launch_bounds__(threads_of<NW>(), MINB) fwd_kernel(const __grid_constant__ Args a) {
-  constexpr int NT = threads_of<NW>();
+__global__ void __launch_bounds__(threads_of<NW, ALL>(), MINB) fwd_kernel(const __grid_constant__ Args a) {
+  constexpr int NT = threads_of<NW, ALL>();
   constexpr int NM = NW * 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const bool mat = warp < NW, node = NW == 1 || warp == NW;
+  const bool mat = warp < NW, node = kLone<NW, ALL> || warp == NW;
   Row<T, NW, GP, ALL, false> r;
   bind(r, a);
   double* scale_s = reinterpret_cast<double*>(r.flag() + 4);
@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) fwd_kernel(const __gri
       r.flag()[2] = atomicAdd(a.queue, 1);
       r.flag()[1] = 0;
     }
-    sync_all<NW>();
+    sync_all<NW, ALL>();
     const int idx = r.flag()[2];
     if (idx >= a.n) break;
     r.j = a.order[idx];
@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) fwd_kernel(const __gri
       stats(r);
       if (!direct) {
         for (int i = tid; i < r.mp; i += NT) r.set_v(i, i == r.pos ? one<T>() : zero<T>());
-        sync_all<NW>();
+        sync_all<NW, ALL>();
         K = lanczos<NE>(r, p, a.sign, Tol<T>::value, &est, &lo);
       }
       if constexpr (kDf<T>) {
@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) fwd_kernel(const __gri
             nc = root_coefs(r, K, p, lo, false, lane);
             if (lane == 0) r.flag()[3] = lo > 0.f && est <= Tol<T>::value ? K + 1 : 0;
           }
-          sync_all<NW>();
+          sync_all<NW, ALL>();
           nc = r.flag()[3] - 1;
           const double unit = exp2((double)(1023 - r.e0));
           double* xd = reinterpret_cast<double*>(r.part());
@@ -82,9 +82,9 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) fwd_kernel(const __gri
                 xd[i] = fix[e];
               }
             }
-          sync_all<NW>();
+          sync_all<NW, ALL>();
           residual(r, a, xd, rd);
-          sync_all<NW>();
+          sync_all<NW, ALL>();
           Row<float, NW, GP, ALL, false> q;
           q.m = r.m, q.nb = r.nb, q.mp = r.mp, q.ns = r.ns, q.pos = r.pos, q.j = r.j;
           q.o_part = r.o_part, q.o_t = 0;
@@ -102,11 +102,11 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) fwd_kernel(const __gri
           }
           n2 = warp_total(n2);
           if (lane == 0) q.red()[warp] = n2;
-          sync_all<NW>();
+          sync_all<NW, ALL>();
           n2 = total_of<NT / 32>(q.red(), lane, NT / 32);
           const float inv = n2 > 1e-36f ? rsqrtf(n2) : 0.f;
           for (int i = tid; i < r.mp; i += NT) q.set_v(i, q.v_at(i) * inv);
-          sync_all<NW>();
+          sync_all<NW, ALL>();
           if (inv > 0.f) {                            // (the residual may vanish: m = 1)
             float est2 = 0.f, lo2 = 0.f;
             const int K2 = lanczos<NE>(q, 1, -1, kTolFix, &est2, &lo2);
@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) fwd_kernel(const __gri
               root_coefs(q, K2, 1, lo2, false, lane);
               if (lane == 0 && !(lo2 > 0.f && est2 <= kTolFix)) r.flag()[3] = 0;
             }
-            sync_all<NW>();
+            sync_all<NW, ALL>();
             if (mat)
 #pragma unroll
               for (int e = 0; e < NE; ++e) {
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) fwd_kernel(const __gri
                   for (int k = 0; k < K2; ++k) s = fmaf(q.coef()[k], q.V[(size_t)k * r.mp + i], s);
                 fix[e] = fma((double)(s * (n2 * inv)), unit, fix[e]);
               }
-            sync_all<NW>();
+            sync_all<NW, ALL>();
           }
         }
       }
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) fwd_kernel(const __gri
         }
       }
       if (mat) cholesky(r);
-      sync_all<NW>();
+      sync_all<NW, ALL>();
       nc = r.flag()[3] - 1;
       ok = nc >= 0 && r.flag()[1] == 0;
     }
@@ -181,15 +181,15 @@ __global__ void __launch_bounds__(threads_of<NW>(), MINB) fwd_kernel(const __gri
         atomicAdd(&a.ctr->flops_alg, ((double)iters * (p + 1) + (p == 1 ? 1.0 : 0.0)) * 2.0 * m2 * r.m);
       }
     }
-    sync_all<NW>();
+    sync_all<NW, ALL>();
   }
 }
 
 template <class T, int NW, bool GP, bool ALL, int NE, int MINB>
 cudaError_t run(const Args& a, int grid, cudaStream_t s) {
   const Layout L = layout(a.nb, a.ns, NW, !GP, false);
-  if ((ALL && a.ns < nblocks(a.nb)) || L.total > kMaxSmem) return cudaErrorInvalidValue;
-  fwd_kernel<T, NW, GP, ALL, NE, MINB><<<grid, threads_of<NW>(), L.total, s>>>(a);
+  if (((ALL || NW == 1) && a.ns < nblocks(a.nb)) || L.total > kMaxSmem) return cudaErrorInvalidValue;
+  fwd_kernel<T, NW, GP, ALL, NE, MINB><<<grid, threads_of<NW, ALL>(), L.total, s>>>(a);
   return cudaGetLastError();
 }
 template <class T, int NW, bool GP, bool ALL, int NE, int MINB>
@@ -201,7 +201,7 @@ cudaError_t attr() {
 template <class T>
 cudaError_t dispatch(const Args& a, const Class& c, int grid, cudaStream_t s) {
   switch (c.nw) {
-    case 1: return run<T, 1, false, true, 1, 16>(a, grid, s);
+    case 1: return c.lone ? run<T, 1, false, false, 1, 16>(a, grid, s) : run<T, 1, false, true, 1, 8>(a, grid, s);
     case 3: return run<T, 3, false, true, 1, 4>(a, grid, s);
     case 5: return run<T, 5, false, true, 1, 2>(a, grid, s);
   }
@@ -212,7 +212,8 @@ cudaError_t dispatch(const Args& a, const Class& c, int grid, cudaStream_t s) {
 template <class T>
 cudaError_t attrs() {
   cudaError_t e;
-  if ((e = attr<T, 1, false, true, 1, 16>()) != cudaSuccess) return e;
+  if ((e = attr<T, 1, false, true, 1, 8>()) != cudaSuccess) return e;
+  if ((e = attr<T, 1, false, false, 1, 16>()) != cudaSuccess) return e;
   if ((e = attr<T, 3, false, true, 1, 4>()) != cudaSuccess) return e;
   if ((e = attr<T, 5, false, true, 1, 2>()) != cudaSuccess) return e;
   if ((e = attr<T, 15, false, true, 1, 1>()) != cudaSuccess) return e;
@@ -303,7 +304,7 @@ bool cached_nodes(int p, int sign, Nodes* out) {     // a constant table per (p,
 // CTAs per SM leave; a class whose blocks do not all fit streams the rest from scratch (L2).
 constexpr int kClassMax[] = {32, 64, 96, 128, 192, SUBMAT_MAX_M};
 constexpr int kClassWarps[] = {1, 3, 3, 5, 15, 15};    // matrix warps (and one for the nodes)
-constexpr int kClassCtas[] = {16, 4, 3, 2, 1, 1};
+constexpr int kClassCtas[] = {8, 4, 3, 2, 1, 1};
 
 int class_of(int m) {
   int i = 0;
@@ -311,13 +312,20 @@ int class_of(int m) {
   return i;
 }
 
-Class make_class(int index, int m_max, bool bwd) {
+Class make_class(int index, int m_max, int rows, int n_sm, bool bwd) {
   Class c;
   c.max_m = std::min(kClassMax[index], (m_max + kB - 1) / kB * kB);
   c.nw = kClassWarps[index];
   c.nb = c.max_m / kB;
   c.ctas = kClassCtas[index];
-  if (bwd && index == 0) c.ctas = 8;                 // its factors need 16 KB a CTA
+  if (index == 0) {
+    // Two warps a row while the rows are at most about two waves of them, then one warp and twice
+    // the rows per SM (as far as the adjoint's factors, 16 KB a CTA, leave room): n = 200, 98 -> 78 us with two;
+    // n = 2000, FP64, 343 -> 260; n = 4000, double-float, 263 -> 205 with one; adjoint n = 700, 351 -> 338
+    // with two, n = 2000, 430 -> 388 with one.
+    c.lone = rows > n_sm * (bwd ? 8 : 16);
+    if (c.lone && !bwd) c.ctas = 16;
+  }
   c.part_smem = c.max_m <= 480;
   const bool all = index + 1 < (int)(sizeof(kClassMax) / sizeof(kClassMax[0]));   // holds every block
   for (;; --c.ctas) {

@@ -219,3 +219,23 @@ def test_rows_of_one_pattern_not_spd(sm):
     assert ei.value.name == "SUBMAT_ENOTSPD"
     y = out.cpu().numpy()
     assert np.isnan(y[200 * 200:]).all() and np.isfinite(y[:200 * 200]).all()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_many_short_rows(sm, precision):
+    """More rows of order <= 32 than two waves (one warp per row in both roles), every fifth row
+    and the gradient against the oracle, same bits twice."""
+    a = wl.overlap_small(n=3000)
+    assert (a.row_sizes() <= 32).all()
+    plan = sm.submat_plan(a.rowptr, a.colind, 2, precision=precision)
+    v = torch.tensor(a.vals, device="cuda")
+    y = sm.submat_invroot(plan, v, sync=True)
+    assert torch.equal(y, sm.submat_invroot(plan, v))
+    rows = list(range(0, a.n, 5))
+    ref = oracle.invroot(a.rowptr, a.colind, a.vals, 2, rows=rows)
+    # m kappa eps = 32 * 250 * 2.2e-16 and, in double-float, 32 * 250 * 2^-45
+    assert row_err(a, y.cpu().numpy(), ref, rows) <= (2e-12 if precision == "fp64" else 3e-10)
+    w = wl.random_on_pattern(a, seed=8)
+    g = sm.submat_invroot_backward(plan, torch.tensor(w, device="cuda")).cpu().numpy()
+    gref = oracle.grad(a.rowptr, a.colind, a.vals, 2, w)
+    assert np.abs(g - gref).max() <= 1e-10 * np.abs(gref).max()
