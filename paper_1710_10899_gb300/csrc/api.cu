@@ -613,7 +613,19 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
   size_t kry_bytes = 0;
   P->runs = plan_runs(P, sizes, kry_max, &scratch_bytes, &kry_bytes);
   if (mixed) P->runs_stall = plan_runs(P, sizes, std::min(kry_max, (int)o.small_max_m), &scratch_bytes, &kry_bytes);
-  for (const EngineRun& run : P->runs) P->use_krylov |= run.engine == kEngineKrylov;
+  if (kry_bytes > 0) {
+    PLAN_TRY(kry::set_attr_fwd());
+    const cudaError_t e1 = cudaMalloc(&P->d_redo, nb * sizeof(int32_t));
+    const cudaError_t e2 = e1 == cudaSuccess ? cudaMalloc(&P->d_kry, kry_bytes) : e1;
+    if (e2 == cudaErrorMemoryAllocation) {     // no room: the coupled iteration takes every row
+      cudaGetLastError();
+      P->runs = plan_runs(P, sizes, 0, &scratch_bytes, &kry_bytes);
+      if (mixed) P->runs_stall = P->runs;
+    } else {
+      PLAN_TRY(e2);
+      P->use_krylov = true;
+    }
+  }
   // rows of one pattern share their submatrix: the tcgen05 engine takes them as one job (the
   // order keeps them together: equal m, ascending indices; its rows come first)
   int32_t tc_rows = 0;

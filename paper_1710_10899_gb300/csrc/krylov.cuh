@@ -39,9 +39,9 @@
 // Why: the coupled iteration spends p m^3 products (ten FP16 slice products each on the mixed
 // path, FP64 at 2 FMA per clock and SM on the FP64 path) per step for a matrix of which one
 // column is kept.  Measured on GB300, whole forward, coupled -> Krylov: FP64 n = 2048, orders
-// 28..239, 301 -> 6.5 ms (bound: the FP64 pipe, 30 products of m^2 a row); FP64 n = 2000,
-// orders 1..28, 11.6 -> 0.33 ms; double-float n = 8192, orders 19..119, 11.1 -> 2.9 ms and
-// n = 9973, orders 25..169, 23.0 -> 5.2 ms (bound: the latency of a step's two barriers and
+// 28..239, 301 -> 6.4 ms (bound: the FP64 pipe, 30 products of m^2 a row); FP64 n = 2000,
+// orders 1..28, 11.6 -> 0.26 ms; double-float n = 8192, orders 19..119, 11.1 -> 2.6 ms and
+// n = 9973, orders 25..169, 23.0 -> 4.7 ms (bound: the latency of a step's two barriers and
 // dependent reductions, half of the issue slots are empty).
 #pragma once
 #include "common.cuh"

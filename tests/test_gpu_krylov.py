@@ -239,3 +239,27 @@ def test_many_short_rows(sm, precision):
     g = sm.submat_invroot_backward(plan, torch.tensor(w, device="cuda")).cpu().numpy()
     gref = oracle.grad(a.rowptr, a.colind, a.vals, 2, w)
     assert np.abs(g - gref).max() <= 1e-10 * np.abs(gref).max()
+
+
+def test_long_row_forward_and_adjoint(sm):
+    """A row of 700 entries (partial sums and most blocks in global scratch) among short ones:
+    FP64 forward against the oracle (m kappa eps = 700 * 4 * 2.2e-16 < 2e-12) and the gradient."""
+    n = 700
+    rng = np.random.default_rng(12)
+    dense = np.eye(n) * 2.0
+    off = 0.15 * rng.uniform(0.5, 1.0, n - 1)
+    dense += np.diag(off, 1) + np.diag(off, -1)
+    dense[0, 1:] = dense[1:, 0] = 0.02 * rng.uniform(0.5, 1.0, n - 1)
+    a = wl.dense_to_csr(dense)
+    y, rep = forward(sm, a, 2, precision="fp64")
+    rows = [0, 1, 2, 350, n - 1]
+    ref = oracle.invroot(a.rowptr, a.colind, a.vals, 2, rows=rows)
+    assert row_err(a, y, ref, rows) <= 2e-12 and rep["n_fallback"] == 0
+    w = wl.random_on_pattern(a, seed=13)
+    for det in (False, True):
+        plan = sm.submat_plan(a.rowptr, a.colind, 2, precision="fp64", grad_deterministic=det)
+        sm.submat_invroot(plan, torch.tensor(a.vals, device="cuda"))
+        g = sm.submat_invroot_backward(plan, torch.tensor(w, device="cuda")).cpu().numpy()
+        gref = oracle.grad(a.rowptr, a.colind, a.vals, 2, w)
+        assert np.linalg.norm(g - gref) / np.linalg.norm(gref) <= 1e-10
+        assert np.abs(g - gref).max() <= 1e-10 * np.abs(gref).max()
