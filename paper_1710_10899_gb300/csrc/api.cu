@@ -611,18 +611,25 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
   std::vector<int32_t> sizes(P->n_jobs);
   for (int32_t i = 0; i < P->n_jobs; ++i) sizes[i] = h_m[order[i]];
   size_t kry_bytes = 0;
+  std::vector<EngineRun> coupled = plan_runs(P, sizes, 0, &scratch_bytes, &kry_bytes);
   P->runs = plan_runs(P, sizes, kry_max, &scratch_bytes, &kry_bytes);
   if (mixed) P->runs_stall = plan_runs(P, sizes, std::min(kry_max, (int)o.small_max_m), &scratch_bytes, &kry_bytes);
+  // what the plan cannot do without first; the Krylov engine's scratch (up to 12 MB a CTA) then
+  // takes what is left, and without room for it the coupled iteration takes every row
+  PLAN_TRY(cudaMalloc(&P->d_scratch, scratch_bytes));
+  PLAN_TRY(cudaMalloc(&P->d_saved, (nnz > 0 ? nnz : 1) * sizeof(double)));
   if (kry_bytes > 0) {
     PLAN_TRY(kry::set_attr_fwd());
-    const cudaError_t e1 = cudaMalloc(&P->d_redo, nb * sizeof(int32_t));
-    const cudaError_t e2 = e1 == cudaSuccess ? cudaMalloc(&P->d_kry, kry_bytes) : e1;
-    if (e2 == cudaErrorMemoryAllocation) {     // no room: the coupled iteration takes every row
+    cudaError_t e = cudaMalloc(&P->d_redo, nb * sizeof(int32_t));
+    if (e == cudaSuccess) e = cudaMalloc(&P->d_kry, kry_bytes);
+    if (e == cudaErrorMemoryAllocation) {
       cudaGetLastError();
-      P->runs = plan_runs(P, sizes, 0, &scratch_bytes, &kry_bytes);
+      cudaFree(P->d_redo);
+      P->d_redo = nullptr;
+      P->runs = std::move(coupled);
       if (mixed) P->runs_stall = P->runs;
     } else {
-      PLAN_TRY(e2);
+      PLAN_TRY(e);
       P->use_krylov = true;
     }
   }
@@ -660,11 +667,6 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
           }
     }
   }
-  if (P->use_krylov) {
-    PLAN_TRY(kry::set_attr_fwd());
-    PLAN_TRY(cudaMalloc(&P->d_redo, nb * sizeof(int32_t)));
-    PLAN_TRY(cudaMalloc(&P->d_kry, kry_bytes));
-  }
   if (kry_bwd) {
     PLAN_TRY(kry::set_attr_bwd());
     for (int32_t i = 0; i < P->n_jobs;) {
@@ -694,7 +696,6 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
     PLAN_TRY(cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking));
     P->side.push_back(q);
   }
-  PLAN_TRY(cudaMalloc(&P->d_scratch, scratch_bytes));
   if (mixed && o.precision == SUBMAT_PREC_MIXED_F16) {
     // TMA descriptors over all CTAs' planes: dims (LD cols, LD rows, planes), 32-byte swizzle
     PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
@@ -723,7 +724,6 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
       return bail(SUBMAT_ECUDA);
     }
   }
-  PLAN_TRY(cudaMalloc(&P->d_saved, (nnz > 0 ? nnz : 1) * sizeof(double)));
   PLAN_TRY(cudaStreamCreateWithFlags(&P->cap_stream, cudaStreamNonBlocking));
   for (auto& e : P->ev) PLAN_TRY(cudaEventCreate(&e));
   PLAN_TRY(cudaDeviceSynchronize());
