@@ -613,7 +613,10 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
   size_t kry_bytes = 0;
   std::vector<EngineRun> coupled = plan_runs(P, sizes, 0, &scratch_bytes, &kry_bytes);
   P->runs = plan_runs(P, sizes, kry_max, &scratch_bytes, &kry_bytes);
-  if (mixed) P->runs_stall = plan_runs(P, sizes, std::min(kry_max, (int)o.small_max_m), &scratch_bytes, &kry_bytes);
+  // (the stall flag concerns the tcgen05 engine alone: the other precisions' launches stay)
+  P->runs_stall = o.precision != SUBMAT_PREC_MIXED_F16
+                      ? P->runs
+                      : plan_runs(P, sizes, std::min(kry_max, (int)o.small_max_m), &scratch_bytes, &kry_bytes);
   // what the plan cannot do without first; the Krylov engine's scratch (up to 12 MB a CTA) then
   // takes what is left, and without room for it the coupled iteration takes every row
   PLAN_TRY(cudaMalloc(&P->d_scratch, scratch_bytes));
@@ -627,7 +630,7 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
       cudaFree(P->d_redo);
       P->d_redo = nullptr;
       P->runs = std::move(coupled);
-      if (mixed) P->runs_stall = P->runs;
+      P->runs_stall = P->runs;
     } else {
       PLAN_TRY(e);
       P->use_krylov = true;

@@ -263,3 +263,15 @@ def test_long_row_forward_and_adjoint(sm):
         gref = oracle.grad(a.rowptr, a.colind, a.vals, 2, w)
         assert np.linalg.norm(g - gref) / np.linalg.norm(gref) <= 1e-10
         assert np.abs(g - gref).max() <= 1e-10 * np.abs(gref).max()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed_sync"])
+def test_other_precisions_ignore_the_stall_flag(sm, precision):
+    """Only the tcgen05 engine reads the flag: the other precisions write every row, with the same bits."""
+    a = wl.overlap_small(n=300)
+    v = torch.tensor(a.vals, device="cuda")
+    plan = sm.submat_plan(a.rowptr, a.colind, 2, precision=precision)
+    ref = sm.submat_invroot(plan, v, sync=True).clone()
+    plan.test_stall(True)
+    out = torch.full_like(v, 7.0)
+    assert torch.equal(sm.submat_invroot(plan, v, out, sync=True), ref)
