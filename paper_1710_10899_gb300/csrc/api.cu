@@ -219,6 +219,7 @@ kry::Args krylov_args(submat_plan_t P, const EngineRun& run, const double* in, d
   k.ctr = P->d_ctr;
   k.queue = &P->d_ctr->run_queue[r];
   k.redo_list = P->d_redo;
+  k.nonfinite = &P->d_ctr->nonfinite;   // of the last forward's input (the backward's, too)
   k.scratch = P->d_kry + run.scratch_off;
   k.stride = run.stride;
   k.nb = run.cls.nb;
@@ -259,9 +260,8 @@ submat_status enqueue_forward(submat_plan_t P, const double* in, double* out, cu
   a.tm_a = P->tm_a;
   a.tm_b = P->tm_b;
   a.stall = P->d_stall;
-  CUDA_TRY(cudaMemcpyAsync(P->d_saved, in, (size_t)P->nnz * sizeof(double),
-                           cudaMemcpyDeviceToDevice, s));
   CUDA_TRY(cudaMemsetAsync(P->d_ctr, 0, sizeof(DevCounters), s));
+  CUDA_TRY(launch_save_vals(in, P->d_saved, P->nnz, &P->d_ctr->nonfinite, s));
   CUDA_TRY(cudaEventRecordWithFlags(P->ev[0], s, evf));
   const std::vector<EngineRun>& runs = P->stalled ? P->runs_stall : P->runs;
   const bool fp64 = P->opts.precision == SUBMAT_PREC_FP64;

@@ -32,6 +32,7 @@ struct DevCounters {
   int32_t error;                       // a device pipeline wait timed out
   int32_t run_queue[12];               // work-queue heads of the forward's engine launches
   int32_t n_redo;                      // rows the Krylov engine left to the general path
+  int32_t nonfinite;                   // some value of A is infinite or NaN
   double flops_alg;                    // sum over rows of k_j (p+1) 2 m_j^3 (+ 2 m_j^3 for
                                        // p = 1's final X product): executed iterations k_j,
                                        // true orders m_j, every product counted as a dense GEMM
@@ -98,6 +99,8 @@ struct BwdArgs {
 // Launchers (return cudaGetLastError() of the launch).
 cudaError_t launch_plan_rows(const int32_t* rowptr, const int32_t* colind, int32_t n,
                              int32_t* m, int32_t* pos, int32_t* flags, cudaStream_t s);
+// saved = vals, *nonfinite = 1 when some value is infinite or NaN (else unchanged).
+cudaError_t launch_save_vals(const double* vals, double* saved, int64_t nnz, int32_t* nonfinite, cudaStream_t s);
 // same[j] = 1 when row j's columns equal row j - 1's.
 cudaError_t launch_same_pattern(const int32_t* rowptr, const int32_t* colind, int32_t n, uint8_t* same,
                                 cudaStream_t s);

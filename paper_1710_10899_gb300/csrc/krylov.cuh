@@ -85,6 +85,7 @@ struct Args {
   DevCounters* ctr;
   int32_t* queue;
   int32_t* redo_list;                      // rows left to the general path
+  const int32_t* nonfinite;                // nonzero: some value is infinite or NaN
   char* scratch;
   size_t stride;                           // bytes per CTA
   int32_t nb;                              // blocks per edge of the class
@@ -709,12 +710,14 @@ __device__ __forceinline__ void find_cols(const Row<T, NW, GP, ALL, BWD>& r, con
 // Gather (Alg. 1): the stored entries (k, l), l >= k, of S into the blocks.  A pattern row is
 // read from its diagonal on (plan's pos), so half of it; a warp takes one row, its next row's
 // first entries already requested.  Returns false (to every thread) when some diagonal entry
-// is not a positive normal number.
+// is not a positive normal number, or an entry below the diagonal is not finite (those are looked
+// at only when A holds such a value at all; above it, they reach the row sums of stats()).
 template <class T, int NW, bool GP, bool ALL, bool BWD>
 __device__ bool gather(Row<T, NW, GP, ALL, BWD>& r, const Args& a) {
   constexpr int NT = threads_of<NW, ALL>();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int base = a.rowptr[r.j], m = r.m;
+  const bool look = *a.nonfinite != 0;
   int mx = 0, mn = 0x7fffffff;                       // high words of the diagonal entries
   for (int k = tid; k < m; k += NT) {
     const int c = a.colind[base + k];
@@ -787,8 +790,22 @@ __device__ bool gather(Row<T, NW, GP, ALL, BWD>& r, const Args& a) {
       load(e0, e1, col, v);
     }
   }
+  if (look) {
+    for (int k = warp; k < m; k += NWALL) {
+      const int e1 = r.ext()[k].x;
+      for (int e0 = a.rowptr[r.R()[k]]; e0 < e1; e0 += 32 * U) {
+        int col[U], l[U];
+        double v[U];
+        load(e0, e1, col, v);
+        find_cols<U>(r, bk, col, l);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (l[u] >= 0 && (__double2hiint(v[u]) & 0x7FF00000) == 0x7FF00000) r.flag()[1] = 1;
+      }
+    }
+  }
   sync_all<NW, ALL>();
-  return true;
+  return !look || r.flag()[1] == 0;
 }
 
 template <class T, int NW, bool GP, bool ALL, bool BWD, class F>

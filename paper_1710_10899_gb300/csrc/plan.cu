@@ -52,6 +52,27 @@ __global__ void plan_rows_kernel(const int32_t* __restrict__ rowptr,
   if (hit < 0) atomicOr(flags, 8);
 }
 
+// The copy of the forward's input for the backward, with a look at every value on its way: engines
+// that read one triangle of the submatrices only search the other one when this found something.
+// Bound by the memory (16 bytes a value), as the plain copy that it takes the place of.
+__global__ void save_vals_kernel(const double* __restrict__ vals, double* __restrict__ saved, int64_t nnz,
+                                 int32_t* __restrict__ nonfinite) {
+  constexpr int U = 4;
+  const int64_t nt = gridDim.x * (int64_t)blockDim.x;
+  bool bad = false;
+  for (int64_t e0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e0 < nnz; e0 += U * nt) {
+    double v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = e0 + u * nt < nnz ? vals[e0 + u * nt] : 0.0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      bad = bad || (__double2hiint(v[u]) & 0x7FF00000) == 0x7FF00000;
+      if (e0 + u * nt < nnz) saved[e0 + u * nt] = v[u];
+    }
+  }
+  if (bad) *nonfinite = 1;
+}
+
 // same[j] = 1 when row j stores the columns of row j - 1: a warp per row.
 __global__ void same_pattern_kernel(const int32_t* __restrict__ rowptr,
                                     const int32_t* __restrict__ colind, int32_t n,
@@ -69,6 +90,13 @@ __global__ void same_pattern_kernel(const int32_t* __restrict__ rowptr,
 }
 
 }  // namespace
+
+cudaError_t launch_save_vals(const double* vals, double* saved, int64_t nnz, int32_t* nonfinite, cudaStream_t s) {
+  if (nnz == 0) return cudaSuccess;
+  const int blocks = (int)((nnz + 1023) / 1024 < 152 * 8 ? (nnz + 1023) / 1024 : 152 * 8);
+  save_vals_kernel<<<blocks, 256, 0, s>>>(vals, saved, nnz, nonfinite);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_same_pattern(const int32_t* rowptr, const int32_t* colind, int32_t n, uint8_t* same,
                                 cudaStream_t s) {

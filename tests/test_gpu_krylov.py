@@ -275,3 +275,26 @@ def test_other_precisions_ignore_the_stall_flag(sm, precision):
     plan.test_stall(True)
     out = torch.full_like(v, 7.0)
     assert torch.equal(sm.submat_invroot(plan, v, out, sync=True), ref)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("p,sign", [(2, -1), (1, -1), (1, 1)])
+@pytest.mark.parametrize("bad", [np.nan, -np.inf])
+def test_non_finite_value_below_the_diagonal(sm, precision, p, sign, bad):
+    """A non-finite value stored at (r, c), r > c, only: the rows whose submatrix holds it are NaN and reported,
+    the others keep their bits."""
+    a = blocks([20, 40, 70], seed=51)
+    r, c = 20 + 33, 20 + 5
+    e = a.rowptr[r] + int(np.nonzero(a.colind[a.rowptr[r]:a.rowptr[r + 1]] == c)[0][0])
+    vals = a.vals.copy()
+    vals[e] = bad
+    plan = sm.submat_plan(a.rowptr, a.colind, p, precision=precision, root_sign=sign)
+    ref = sm.submat_invroot(plan, torch.tensor(a.vals, device="cuda"), sync=True).cpu().numpy()
+    out = torch.zeros(a.nnz, dtype=torch.float64, device="cuda")
+    with pytest.raises(sm.SubmatError) as ei:
+        sm.submat_invroot(plan, torch.tensor(vals, device="cuda"), out, sync=True)
+    assert ei.value.name == "SUBMAT_ENOTSPD" and plan.report()["n_notspd"] == 40
+    y = out.cpu().numpy()
+    hit = np.zeros(a.nnz, bool)
+    hit[a.rowptr[20]:a.rowptr[60]] = True
+    assert np.isnan(y[hit]).all() and np.array_equal(y[~hit], ref[~hit])
