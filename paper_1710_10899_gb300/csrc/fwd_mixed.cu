@@ -1787,9 +1787,13 @@ __global__ void __launch_bounds__(ENG == ENG_TC ? TC_THREADS : kThreads,
       resid = sqrt((double)tot);
       kest = lo_raw > 0.f ? 1.f / lo_raw : 3.0e38f;
       if (GROUP && gv.nv > 0) {
-        // the other members' columns of the same limit; the residual, a function of M_K
-        // alone but for the column, is the first member's
-        group_final(gv, B3[mi].q, plane, B3[mi].e, degree(1e-9f), p, ny, m, mp);
+        // the other members' columns of the same limit.  The residual above is the first member's
+        // column of P(E)^p M_K - I; M_K may be far from I in the others.  They are all bounded by
+        // that matrix's 2-norm, with P = M_K^(-1/p) + d, |d| <= the tail at ||E||_2 <= ||E||_F.
+        const int J = degree(1e-9f);
+        const double tail = eps < 1.f ? pow((double)eps, J + 1.0) / (1.0 - (double)eps) : 1e300;
+        resid = fmax(resid, pow(1.0 + tail * pow(1.0 + (double)eps, 1.0 / (double)p), (double)p) - 1.0);
+        group_final(gv, B3[mi].q, plane, B3[mi].e, J, p, ny, m, mp);
         if (resid <= a.resid_tol && kest <= (float)a.kappa_max)
           for (int v = 0; v < gv.nv; ++v) {
             double* out = a.vals_out + a.rowptr[a.order[first + 1 + v]];

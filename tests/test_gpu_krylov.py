@@ -298,3 +298,19 @@ def test_non_finite_value_below_the_diagonal(sm, precision, p, sign, bad):
     hit = np.zeros(a.nnz, bool)
     hit[a.rowptr[20]:a.rowptr[60]] = True
     assert np.isnan(y[hit]).all() and np.array_equal(y[~hit], ref[~hit])
+
+
+@pytest.mark.parametrize("p,sign", [(2, -1), (3, -1), (2, 1)])
+def test_group_not_converged_in_other_columns(sm, p, sign):
+    """A diagonal submatrix of order 200 (full pattern) after one step only: the first row of each job of 13
+    has a value that the step and the Taylor finish bring to the limit, the others the smallest one, which
+    they do not.  Every row is right to the residual threshold 1e-3: those that are not converged take the fallback."""
+    n = 200
+    d = np.full(n, 0.02)
+    d[::13] = np.linspace(0.2, 1.0, len(d[::13]))
+    a = wl.dense_to_csr(np.diag(d), keep=np.ones((n, n), bool))
+    y, rep = forward(sm, a, p, precision="mixed", root_sign=sign, k_max=1)
+    got = y.reshape(n, n)
+    ref = np.diag(d ** (sign / p))
+    assert (np.linalg.norm(got - ref, axis=1) <= 2e-3 * np.diag(ref)).all()
+    assert rep["n_fallback"] >= n - len(d[::13])
