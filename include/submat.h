@@ -77,7 +77,7 @@ enum {
   SUBMAT_PREC_MIXED_F16 = 1,  /* coupled Newton iteration on the tensor cores (tcgen05) with
                                  every matrix split into four FP16 planes of 10-bit integers,
                                  accumulated per level (10 FP16 products per product),
-                                 then the FP64 column residual check                       */
+                                 then the column residual check (see resid_tol)            */
   SUBMAT_PREC_MIXED_F16_SYNC = 2  /* the same arithmetic on the legacy mma.sync tensor path
                                  (kept as the baseline of the tcgen05 engine)               */
 };
@@ -99,9 +99,15 @@ typedef struct {
                               and finishes with a Taylor polynomial of M^(-1/p) on the
                               carried column instead; default 1e-4 (mixed) / 1e-7 (FP64);
                               <= 0 selects the default                                    */
-  double resid_tol;        /* a row whose FP64 column residual ||e_pos - F^p s_pos||_2
-                              exceeds this goes to the FP64 eigendecomposition fallback;
-                              default 1e-3                                                */
+  double resid_tol;        /* a row whose column residual ||e_pos - F^p s_pos||_2 exceeds
+                              this goes to the FP64 eigendecomposition fallback; default
+                              1e-3.  The inverse (p = 1): ||e_pos - S y||_2 of the column y
+                              before its refinement, in FP64.  p >= 2, coupled iteration: of
+                              the converged iterate M_K taken through the last step (a job of
+                              rows of one pattern: also a bound over every column).  p >= 2,
+                              Krylov engine: the bound on the column's relative error at
+                              which its recurrence stopped (such a row then takes the coupled
+                              iteration)                                                  */
   int32_t refine_steps;    /* FP64 column refinement: p = 1: iterative-refinement sweeps
                               (default 2); p >= 2: 1 = one Newton step on the column,
                               0 = none (default 0: once the iteration has converged the
@@ -158,8 +164,8 @@ typedef struct {
                               steps that the coupled iteration takes on its interval)     */
   int64_t n_fallback;      /* rows recomputed by the FP64 eigendecomposition fallback    */
   int64_t n_notspd;        /* rows with a non-positive eigenvalue or non-finite input    */
-  double max_resid;        /* largest FP64 column residual seen before the fallback (Krylov
-                              engine: the error bound at which its recurrence stopped)    */
+  double max_resid;        /* largest column residual seen before the fallback (as the one
+                              that resid_tol is compared with)                            */
   double sum_m3;           /* sum over rows of m^3 (true sizes)                           */
   double flops_tensor;     /* tensor-core flops executed by the last forward: sum over
                               rows of (GEMMs executed) * 10 FP16 slice products *

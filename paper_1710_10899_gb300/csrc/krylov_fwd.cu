@@ -48,6 +48,7 @@ __global__ void __launch_bounds__(threads_of<NW, ALL>(), MINB) fwd_kernel(const 
     bool ok = gather(r, a);
     int K = 0, nc = 0;
     double fix[NE];
+    double res1 = 0.0;                               // p = 1: the column's residual, in FP64
     float est = 0.f, lo = 1.f;
     if (ok) {
       stats(r);
@@ -104,6 +105,7 @@ __global__ void __launch_bounds__(threads_of<NW, ALL>(), MINB) fwd_kernel(const 
           if (lane == 0) q.red()[warp] = n2;
           sync_all<NW, ALL>();
           n2 = total_of<NT / 32>(q.red(), lane, NT / 32);
+          res1 = sqrt((double)n2);
           const float inv = n2 > 1e-36f ? rsqrtf(n2) : 0.f;
           for (int i = tid; i < r.mp; i += NT) q.set_v(i, q.v_at(i) * inv);
           sync_all<NW, ALL>();
@@ -137,21 +139,48 @@ __global__ void __launch_bounds__(threads_of<NW, ALL>(), MINB) fwd_kernel(const 
           const double tau = (double)tau_f;
           const double al = a.sign < 0 ? 1.0 / (double)p : 1.0 - 1.0 / (double)p;
           *scale_s = exp2(E * ex) * (p > 1 ? pow(tau, -al) : 1.0);
-          // accepted only with the recurrence's bound met (NaN is not)
+          // accepted only with the recurrence's bound met (NaN is not); for p = 1 the residual of
+          // the column (before its correction) is measured as well, as in refine_column
           if (!fixed_up) r.flag()[3] = direct || (lo > 0.f && est <= Tol<T>::value && (double)est <= a.resid_tol) ? nc + 1 : 0;
-          else if (!((double)est <= a.resid_tol)) r.flag()[3] = 0;
+          else if (!(res1 <= a.resid_tol)) r.flag()[3] = 0;
         }
       }
       if (mat) cholesky(r);
       sync_all<NW, ALL>();
       nc = r.flag()[3] - 1;
       ok = nc >= 0 && r.flag()[1] == 0;
+      if constexpr (!kDf<T>) {
+        if (ok && p == 1 && !direct) {                // the residual of the FP64 inverse's column
+          double* xd = r.part();
+          double* rd = r.X;
+          const double unit = exp2((double)(1023 - r.e0));
+          for (int i = tid; i < r.m; i += NT) {
+            double s = 0.0;
+            for (int k = 0; k < nc; ++k) s += r.coef()[k] * r.V[(size_t)k * r.mp + i];
+            xd[i] = s * unit;
+          }
+          sync_all<NW, ALL>();
+          residual(r, a, xd, rd);
+          sync_all<NW, ALL>();
+          double n2 = 0.0;
+          for (int i = tid; i < r.m; i += NT) n2 = fma(rd[i], rd[i], n2);
+          n2 = warp_total(n2);
+          if (lane == 0) r.red()[warp] = n2;
+          sync_all<NW, ALL>();
+          res1 = sqrt(total_of<NT / 32>(r.red(), lane, NT / 32));
+          ok = res1 <= a.resid_tol;
+          if (ok)
+            for (int i = tid; i < r.m; i += NT) a.out[a.rowptr[r.j] + i] = xd[i];
+        }
+      }
     }
     if (ok) {
       const double scale = *scale_s;
       double* out = a.out + a.rowptr[r.j];
       if (direct) {
         for (int i = tid; i < r.m; i += NT) out[i] = a.vals[a.rowptr[r.j] + i];
+      } else if (!kDf<T> && p == 1) {
+        // written above
       } else if (kDf<T> && p == 1) {
         if (mat)
 #pragma unroll
@@ -176,7 +205,7 @@ __global__ void __launch_bounds__(threads_of<NW, ALL>(), MINB) fwd_kernel(const 
         const double m2 = (double)r.m * r.m;
         atomicMax(&a.ctr->iters_max, iters);
         atomicAdd(&a.ctr->iters_sum, (unsigned long long)iters);
-        atomic_max_nonneg(&a.ctr->resid_max_bits, (double)est);
+        atomic_max_nonneg(&a.ctr->resid_max_bits, p == 1 && !direct ? res1 : (double)est);
         if (a.fp64) atomicAdd(&a.ctr->flops_fp64, 2.0 * m2 * (double)K);
         atomicAdd(&a.ctr->flops_alg, ((double)iters * (p + 1) + (p == 1 ? 1.0 : 0.0)) * 2.0 * m2 * r.m);
       }

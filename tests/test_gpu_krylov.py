@@ -314,3 +314,17 @@ def test_group_not_converged_in_other_columns(sm, p, sign):
     ref = np.diag(d ** (sign / p))
     assert (np.linalg.norm(got - ref, axis=1) <= 2e-3 * np.diag(ref)).all()
     assert rep["n_fallback"] >= n - len(d[::13])
+
+
+def test_inverse_column_residual_is_measured(sm):
+    """p = 1 in FP64: the residual that resid_tol is compared with is that of the column itself, rounding included
+    (about |y| eps; the recurrence alone always stops below 2e-16).  At resid_tol = 2e-16 rows of order 70 fail it
+    and end in the fallback; at the default nothing does, and the report holds the residual of the rows written."""
+    a = blocks([70], seed=61)
+    y, rep = forward(sm, a, 1, precision="fp64")
+    s = a.vals.reshape(70, 70).astype(np.longdouble)
+    r = np.linalg.norm((np.eye(70) - y.reshape(70, 70).astype(np.longdouble) @ s).astype(float), axis=1).max()
+    assert rep["n_fallback"] == 0 and 2e-16 < r < 1e-13 and r / 4 <= rep["max_resid"] <= 4 * r
+    z, rep = forward(sm, a, 1, precision="fp64", resid_tol=2e-16)
+    assert rep["n_fallback"] >= 1
+    assert row_err(a, z, y, range(a.n)) <= 2e-12
