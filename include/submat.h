@@ -69,8 +69,9 @@ typedef enum {
  * pairs) orders up to 192 for p = 2 (up to 160 for p = 3, none beyond) and every order for p = 1,
  * whose column is then refined in FP64.  A row that it refuses
  * (lambda_bar / lambda_min above 2000; not positive definite) and every row of a plan whose
- * options steer the coupled iteration (k_max, tol, refine_steps, kappa_max, size buckets) takes
- * the coupled iteration.
+ * options steer the coupled iteration (k_max, tol, refine_steps, kappa_max, small_max_m or
+ * sync_max_m other than its default; the default given explicitly is the default) takes the
+ * coupled iteration.
  */
 enum {
   SUBMAT_PREC_FP64 = 0,       /* everything in FP64 (CUDA cores)                            */
@@ -316,6 +317,12 @@ SUBMAT_API submat_status submat_get_report(submat_plan_t plan, submat_report* ou
  * pos[j] = R_j.indexof(j), copied into the caller's host arrays of n int32 each.
  */
 SUBMAT_API submat_status submat_plan_rows(submat_plan_t plan, int32_t* m, int32_t* pos);
+
+/*
+ * Kernel launches of one forward: the copy of the input, one per engine and Krylov size class that
+ * has rows, the coupled iteration over the rows that the Krylov engine left, and the fallback.
+ */
+SUBMAT_API submat_status submat_plan_launches(submat_plan_t plan, int32_t* launches);
 
 /*
  * Test aid for the bounded device waits (the paper has no counterpart).  While on != 0,

@@ -75,7 +75,7 @@ EXPORTS = ["submat_default_opts", "submat_plan", "submat_invroot", "submat_invro
            "submat_invroot_backward",
            "submat_get_report", "submat_plan_rows", "submat_plan_shape", "submat_plan_destroy",
            "submat_status_string", "submat_last_error", "submat_invroot_noalloc", "submat_pcg",
-           "submat_shard_rows", "submat_test_stall", "submat_refine"]
+           "submat_shard_rows", "submat_test_stall", "submat_refine", "submat_plan_launches"]
 
 _lib_handle = None
 
@@ -120,6 +120,8 @@ def load_library(path: str = LIB_PATH):
     lib.submat_shard_rows.restype = i32
     lib.submat_test_stall.argtypes = [vp, i32]
     lib.submat_test_stall.restype = i32
+    lib.submat_plan_launches.argtypes = [vp, ctypes.POINTER(i32)]
+    lib.submat_plan_launches.restype = i32
     lib.submat_refine.argtypes = [vp, vp, vp, i32, i32, vp, vp]
     lib.submat_refine.restype = i32
     _lib_handle = lib
@@ -200,9 +202,6 @@ class Plan:
         self.sync_max_m = int(o.sync_max_m)
         self.shard = (int(shard[0]), int(shard[1]))
         self.device = torch.device("cuda", torch.cuda.current_device())
-        # options that keep the coupled iteration (see include/submat.h)
-        self._steered = (k_max >= 1 and k_max != 40) or tol > 0.0 or refine_steps >= 0 or \
-            (kappa_max > 0.0 and kappa_max != 100.0) or self.small_max_m != 32 or self.sync_max_m != 0
         self._fwd_gen = 0              # forwards run on this plan (the backward's input)
 
     def __del__(self):
@@ -219,31 +218,10 @@ class Plan:
         return m, pos
 
     def engine_launches(self):
-        """Kernel launches of one forward: one per engine and Krylov size class that gets rows,
-        the coupled iteration over the rows the Krylov engine left, and the fallback kernel."""
-        m, _ = self.rows()
-        b, e = shard_rows(self.rowptr_host, self.shard[1], self.shard[0])
-        m = m[b:e]
-        # largest order of the Krylov engine (0: not used; its classes end at these orders)
-        top = 0
-        if not self._steered and self.p <= SUBMAT_MIXED_MAX_P:
-            if self.precision == "fp64" or (self.precision == "mixed" and self.p == 1):
-                top = 1536
-            elif self.precision == "mixed":
-                top = {2: 192, 3: 160}.get(self.p, 0)
-        edges = [0, 32, 64, 96, 128, 192, 1536]
-        kry = sum(int(((m > lo) & (m <= min(hi, top))).any())
-                  for lo, hi in zip(edges[:-1], edges[1:]) if lo < top)
-        left = 1 if kry else 0
-        rest = m[m > top]
-        if self.precision == "fp64":
-            return kry + left + int(len(rest) > 0) + 1
-        if self.precision == "mixed_sync":
-            return 1 + int(len(m) > 0)
-        small = rest <= self.small_max_m
-        sync = (~small) & (rest <= self.sync_max_m)
-        tc = ~(small | sync)
-        return kry + left + 1 + int(small.any()) + int(sync.any()) + int(tc.any())
+        """Kernel launches of one forward (``submat_plan_launches``)."""
+        k = ctypes.c_int32()
+        _check(self._lib, self._lib.submat_plan_launches(self._h, ctypes.byref(k)))
+        return int(k.value)
 
     def test_stall(self, on: bool):
         """``submat_test_stall``: make the tensor-core forward's first pipeline wait run out

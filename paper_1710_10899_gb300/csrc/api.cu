@@ -53,6 +53,12 @@ struct EngineRun {
 constexpr int kMaxRuns = 9;             // tcgen05, mma.sync, small and six Krylov classes
 static_assert(kMaxRuns <= (int)(sizeof(DevCounters::run_queue) / sizeof(int32_t)), "queue heads");
 
+// Defaults of the options that steer the coupled iteration (submat.h).
+constexpr int kDefaultKMax = 40;
+constexpr double kDefaultKappaMax = 100.0;
+double default_tol(int precision) { return precision == SUBMAT_PREC_FP64 ? 1e-7 : 1e-4; }
+int default_refine(int p) { return p == 1 ? 2 : 0; }
+
 struct GraphEntry {
   const double* in = nullptr;
   double* out = nullptr;
@@ -345,12 +351,12 @@ submat_status submat_shard_rows(int32_t n, const int32_t* rowptr, int32_t count,
 void submat_default_opts(submat_opts* o) {
   if (!o) return;
   o->precision = SUBMAT_PREC_MIXED_F16;
-  o->k_max = 40;
+  o->k_max = kDefaultKMax;
   o->tol = 0.0;
   o->resid_tol = 1e-3;
   o->refine_steps = -1;
   o->use_graph = 1;
-  o->kappa_max = 100.0;
+  o->kappa_max = kDefaultKappaMax;
   o->root_sign = -1;
   o->grad_deterministic = 0;
   o->grad_wave_mib = 0;
@@ -451,11 +457,11 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
   if (o.precision != SUBMAT_PREC_FP64 && o.precision != SUBMAT_PREC_MIXED_F16 &&
       o.precision != SUBMAT_PREC_MIXED_F16_SYNC)
     return fail(SUBMAT_EINVAL, "unknown precision");
-  if (o.k_max < 1) o.k_max = 40;
-  if (!(o.tol > 0.0)) o.tol = (o.precision == SUBMAT_PREC_FP64) ? 1e-7 : 1e-4;
+  if (o.k_max < 1) o.k_max = kDefaultKMax;
+  if (!(o.tol > 0.0)) o.tol = default_tol(o.precision);
   if (!(o.resid_tol > 0.0)) o.resid_tol = 1e-3;
-  if (o.refine_steps < 0) o.refine_steps = (p == 1) ? 2 : 0;
-  if (!(o.kappa_max > 0.0)) o.kappa_max = 100.0;
+  if (o.refine_steps < 0) o.refine_steps = default_refine(p);
+  if (!(o.kappa_max > 0.0)) o.kappa_max = kDefaultKappaMax;
   if (o.root_sign != -1 && o.root_sign != 1) return fail(SUBMAT_EINVAL, "root_sign must be -1 or +1");
   if (o.grad_deterministic != 0 && o.grad_deterministic != 1)
     return fail(SUBMAT_EINVAL, "grad_deterministic must be 0 or 1");
@@ -597,10 +603,11 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
   // engine runs: the plan's rows are ordered by decreasing m, so each size bucket is one
   // contiguous run of the order
   size_t scratch_bytes = stride * (size_t)P->grid;
-  // options that steer the coupled iteration, its refinement or its fallback keep it
-  const bool steered = opts && ((opts->k_max >= 1 && opts->k_max != 40) || opts->tol > 0.0 ||
-                                opts->refine_steps >= 0 || o.kappa_max != 100.0 ||
-                                o.small_max_m != kTunedSmallMaxM || o.sync_max_m != kTunedSyncMaxM);
+  // options that steer the coupled iteration, its refinement or its fallback keep it: a value
+  // other than the default, however the default was given
+  const bool steered = o.k_max != kDefaultKMax || o.tol != default_tol(o.precision) ||
+                       o.refine_steps != default_refine(p) || o.kappa_max != kDefaultKappaMax ||
+                       o.small_max_m != kTunedSmallMaxM || o.sync_max_m != kTunedSyncMaxM;
   const int kry_max = steered ? 0 : krylov_max_m(o.precision, p);
   // (the inverse's adjoint stays with the Jacobi kernel, whose error there is the smaller one)
   const bool kry_bwd = p <= SUBMAT_MIXED_MAX_P && (p > 1 || o.root_sign > 0);
@@ -1096,6 +1103,16 @@ submat_status submat_plan_rows(submat_plan_t P, int32_t* m, int32_t* pos) {
   if (P->n == 0) return SUBMAT_OK;
   CUDA_TRY(cudaMemcpy(m, P->d_m, P->n * sizeof(int32_t), cudaMemcpyDeviceToHost));
   CUDA_TRY(cudaMemcpy(pos, P->d_pos, P->n * sizeof(int32_t), cudaMemcpyDeviceToHost));
+  return SUBMAT_OK;
+}
+
+submat_status submat_plan_launches(submat_plan_t P, int32_t* launches) {
+  g_last_error.clear();
+  if (!P || !launches) return fail(SUBMAT_EINVAL, "NULL argument");
+  // as enqueue_forward: the copy of the input, the engines' runs, the rows the Krylov engine left
+  // and the fallback
+  const size_t runs = (P->stalled ? P->runs_stall : P->runs).size();
+  *launches = P->n == 0 ? 0 : (int32_t)(1 + runs + (P->use_krylov ? 1 : 0) + 1);
   return SUBMAT_OK;
 }
 

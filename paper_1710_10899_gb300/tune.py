@@ -1,9 +1,10 @@
 """Tune the mixed-precision forward's size buckets on the GPU at hand and write them into
 ``csrc/engine_table.h`` (rebuild the library afterwards).
 
-For every row order m in the candidate list, a block-diagonal workload whose rows all have
-order m (``workloads.block_diagonal_spd``, enough rows to fill every SM several times) is run
-through each engine that can take it: the small engine (working set in shared memory, 16 x 8
+For every row order m in the candidate list, a workload whose rows all have order m and patterns
+of their own (``workloads.ring_spd``, enough rows to fill every SM several times; rows of one
+pattern would share a job of the tcgen05 engine) is run through each engine of the coupled
+iteration that can take it (a step limit other than the default keeps the Krylov engine out): the small engine (working set in shared memory, 16 x 8
 warp tiles), the mma.sync engine (64 x 64 tiles) and the tcgen05 engine (128 x 96 tiles in
 tensor memory).  The time per forward is the median of ``--steps`` CUDA-event timed calls
 after ``--warmup`` untimed ones.  The small engine takes the orders from 1 up to the largest
@@ -26,9 +27,9 @@ if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
 CANDIDATES = [8, 16, 24, 32, 48, 64, 96, 128]
-ENGINES = {"small": dict(small_max_m=32, sync_max_m=0),
-           "sync": dict(small_max_m=0, sync_max_m=1536),
-           "tcgen05": dict(small_max_m=0, sync_max_m=0)}
+ENGINES = {"small": dict(small_max_m=32, sync_max_m=0, k_max=41),
+           "sync": dict(small_max_m=0, sync_max_m=1536, k_max=41),
+           "tcgen05": dict(small_max_m=0, sync_max_m=0, k_max=41)}
 
 
 def time_forward(sm, a, p, opts, steps, warmup):
@@ -109,7 +110,7 @@ def main():
     sm.load_library()
     times = {}
     for m in CANDIDATES:
-        a = wl.block_diagonal_spd(max(1, args.rows // m), m, seed=m)
+        a = wl.ring_spd(args.rows, m, seed=m)
         times[m] = {}
         for name, opts in ENGINES.items():
             if name == "small" and m > sm.SUBMAT_SMALL_MAX_M:

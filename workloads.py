@@ -239,6 +239,32 @@ def block_diagonal_spd(blocks: int, size: int, seed: int = 0) -> CSR:
     return CSR(n, rowptr, colind, v, f"block_diagonal_spd(blocks={blocks},size={size})")
 
 
+def ring_spd(n: int, size: int, seed: int = 0) -> CSR:
+    """n rows (n even) of ``size`` stored entries (size even), every row with a pattern of its own:
+    the nearest size - 2 neighbours on a ring, the antipode and the diagonal.  Off-diagonal row
+    sums below 1 and the diagonal 1.2, so condition numbers below 11."""
+    assert n % 2 == 0 and size % 2 == 0 and 2 <= size < n
+    rng = np.random.default_rng(seed)
+    i = np.arange(n)
+    steps = list(range(1, size // 2)) + [n // 2]
+    rows, cols, vals = [i], [i], [np.full(n, 1.2)]
+    for k in steps:
+        v = rng.uniform(0.2, 1.0, n) / size
+        if k == n // 2:
+            v[n // 2:] = v[:n // 2]
+            rows += [i]
+            cols += [(i + k) % n]
+            vals += [v]
+        else:
+            rows += [i, (i + k) % n]
+            cols += [(i + k) % n, i]
+            vals += [v, v]
+    m = sp.csr_matrix((np.concatenate(vals), (np.concatenate(rows), np.concatenate(cols))), shape=(n, n))
+    m.sort_indices()
+    return CSR(n, m.indptr.astype(np.int32), m.indices.astype(np.int32), m.data.astype(np.float64),
+               f"ring_{n}_{size}")
+
+
 def stratified_rows(m: np.ndarray, k: int, seed: int = 3) -> np.ndarray:
     """A seeded sample of about k row indices stratified by row size: the sizes are binned
     by powers of two (below 32, 32..63, ..., 1024..2047, 2048 and above), each non-empty bin
