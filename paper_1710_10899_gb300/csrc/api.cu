@@ -51,7 +51,8 @@ struct EngineRun {
   size_t scratch_off = 0, stride = 0;
 };
 constexpr int kMaxRuns = 9;             // tcgen05, mma.sync, small and six Krylov classes
-static_assert(kMaxRuns <= (int)(sizeof(DevCounters::run_queue) / sizeof(int32_t)), "queue heads");
+static_assert(kMaxRuns < (int)(sizeof(DevCounters::run_queue) / sizeof(int32_t)),
+              "queue heads: the runs' and the small engine's over the left-over rows");
 
 // Defaults of the options that steer the coupled iteration (submat.h).
 constexpr int kDefaultKMax = 40;
@@ -151,8 +152,11 @@ struct submat_plan_s {
   int2* d_jobs = nullptr;             // tcgen05 engine's jobs
   bool stalled = false;
   bool use_krylov = false;            // some run is the Krylov engine's
+  bool redo_rest = false;             // rows above the small engine's orders are among its rows
+  int grid_redo_small = 0;            // small engine's launch over the left-over rows it takes (0: none)
   kry::Nodes nodes{};
-  int32_t* d_redo = nullptr;          // rows the Krylov engine left to the general path
+  int32_t* d_redo = nullptr;          // rows the Krylov engine left to the general path: n, then
+                                      // n for those of the small engine
   char* d_kry = nullptr;              // its scratch
   std::vector<cudaStream_t> side;     // runs after the first execute beside it
   std::vector<cudaEvent_t> side_ev;   // fork, then one join per side stream
@@ -225,6 +229,8 @@ kry::Args krylov_args(submat_plan_t P, const EngineRun& run, const double* in, d
   k.ctr = P->d_ctr;
   k.queue = &P->d_ctr->run_queue[r];
   k.redo_list = P->d_redo;
+  k.redo_small = P->d_redo + P->n;
+  k.small_max = P->grid_redo_small > 0 ? P->opts.small_max_m : 0;
   k.nonfinite = &P->d_ctr->nonfinite;   // of the last forward's input (the backward's, too)
   k.scratch = P->d_kry + run.scratch_off;
   k.stride = run.stride;
@@ -302,12 +308,22 @@ submat_status enqueue_forward(submat_plan_t P, const double* in, double* out, cu
   }
   for (size_t r = 1; r < runs.size(); ++r)
     if (runs[r].engine == kEngineKrylov) CUDA_TRY(cudaStreamWaitEvent(s, P->side_ev[r], 0));
-  if (P->use_krylov) {                  // the rows it left to the coupled iteration
+  // the rows it left to the coupled iteration, on the engine of their order
+  if (P->redo_rest) {
     FwdArgs b = a;
     b.order = P->d_redo;
     b.n_dev = &P->d_ctr->n_redo;
     if (fp64) CUDA_TRY(launch_fwd_fp64(b, P->grid, s));
     else CUDA_TRY(launch_fwd_mixed(b, P->grid, s));
+  }
+  if (P->grid_redo_small > 0) {
+    FwdArgs b = a;
+    b.engine = kEngineSmall;
+    b.order = P->d_redo + P->n;
+    b.n_dev = &P->d_ctr->n_redo_small;
+    b.queue = &P->d_ctr->run_queue[kMaxRuns];
+    b.scratch_stride = scratch_small();
+    CUDA_TRY(launch_fwd_mixed(b, P->grid_redo_small, s));
   }
   CUDA_TRY(cudaEventRecordWithFlags(P->ev[1], s, evf));
   CUDA_TRY(launch_fallback(a, P->grid, s));
@@ -624,13 +640,20 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
   P->runs_stall = o.precision != SUBMAT_PREC_MIXED_F16
                       ? P->runs
                       : plan_runs(P, sizes, std::min(kry_max, (int)o.small_max_m), &scratch_bytes, &kry_bytes);
+  // rows that the Krylov engine refuses go where their order would have taken them: short ones to
+  // the small engine (24 entries, 7200 rows refused: 4.0 ms on it, 10.9 with the tcgen05 engine)
+  const int redo_max = o.precision == SUBMAT_PREC_MIXED_F16 ? o.small_max_m : 0;
+  const int32_t n_short = (int32_t)(sizes.end() - std::partition_point(sizes.begin(), sizes.end(),
+                                                                       [&](int32_t m) { return m > redo_max; }));
+  const int redo_small = std::min(P->n_sm * mixed_ctas_per_sm(kEngineSmall), n_short);
+  scratch_bytes = std::max(scratch_bytes, scratch_small() * (size_t)redo_small);
   // what the plan cannot do without first; the Krylov engine's scratch (up to 12 MB a CTA) then
   // takes what is left, and without room for it the coupled iteration takes every row
   PLAN_TRY(cudaMalloc(&P->d_scratch, scratch_bytes));
   PLAN_TRY(cudaMalloc(&P->d_saved, (nnz > 0 ? nnz : 1) * sizeof(double)));
   if (kry_bytes > 0) {
     PLAN_TRY(kry::set_attr_fwd());
-    cudaError_t e = cudaMalloc(&P->d_redo, nb * sizeof(int32_t));
+    cudaError_t e = cudaMalloc(&P->d_redo, 2 * nb * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMalloc(&P->d_kry, kry_bytes);
     if (e == cudaErrorMemoryAllocation) {
       cudaGetLastError();
@@ -641,6 +664,8 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
     } else {
       PLAN_TRY(e);
       P->use_krylov = true;
+      P->grid_redo_small = redo_small;
+      P->redo_rest = sizes[0] > redo_max;
     }
   }
   // rows of one pattern share their submatrix: the tcgen05 engine takes them as one job (the
@@ -866,6 +891,7 @@ static submat_status enqueue_backward(submat_plan_t P, const BwdArgs& a, bool kr
     k.ctr = P->d_ctr_bwd;
     k.queue = &P->d_ctr_bwd->run_queue[r];
     k.redo_list = P->d_redo_bwd;
+    k.small_max = 0;                    // (one list: the Jacobi kernel takes every order)
     k.scratch = P->d_kry_bwd + run.scratch_off;
     k.fp64 = 0;
     k.grad_out = a.grad_out;
@@ -1112,7 +1138,7 @@ submat_status submat_plan_launches(submat_plan_t P, int32_t* launches) {
   // as enqueue_forward: the copy of the input, the engines' runs, the rows the Krylov engine left
   // and the fallback
   const size_t runs = (P->stalled ? P->runs_stall : P->runs).size();
-  *launches = P->n == 0 ? 0 : (int32_t)(1 + runs + (P->use_krylov ? 1 : 0) + 1);
+  *launches = P->n == 0 ? 0 : (int32_t)(1 + runs + (P->redo_rest ? 1 : 0) + (P->grid_redo_small > 0 ? 1 : 0) + 1);
   return SUBMAT_OK;
 }
 

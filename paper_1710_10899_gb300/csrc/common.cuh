@@ -31,7 +31,8 @@ struct DevCounters {
   unsigned long long n_illcond;        // rows sent to the fallback by the condition estimate
   int32_t error;                       // a device pipeline wait timed out
   int32_t run_queue[12];               // work-queue heads of the forward's engine launches
-  int32_t n_redo;                      // rows the Krylov engine left to the general path
+  int32_t n_redo, n_redo_small;        // rows the Krylov engine left to the general path, and
+                                       // to the small engine
   int32_t nonfinite;                   // some value of A is infinite or NaN
   double flops_alg;                    // sum over rows of k_j (p+1) 2 m_j^3 (+ 2 m_j^3 for
                                        // p = 1's final X product): executed iterations k_j,

@@ -84,7 +84,8 @@ struct Args {
   double* out;                             // forward: vals_out; backward: grad_in
   DevCounters* ctr;
   int32_t* queue;
-  int32_t* redo_list;                      // rows left to the general path
+  int32_t *redo_list, *redo_small;         // rows left to the general path; of order <= small_max
+  int32_t small_max;
   const int32_t* nonfinite;                // nonzero: some value is infinite or NaN
   char* scratch;
   size_t stride;                           // bytes per CTA
@@ -912,7 +913,9 @@ __device__ __forceinline__ float node_lo(const NodeState& s) {
   if (up >> 31) return sturm_shift(31);
   return up ? sturm_shift(__ffs(up) - 1) : 0.f;
 }
-// Bound after the step with alpha, beta.
+// Bound after the step with alpha, beta; kNoBound once a Ritz value lies below every shift (the
+// smallest one only falls, so the row is refused: lam / 2^11.2 is beyond kKappa).
+constexpr float kNoBound = 1e30f;
 __device__ __forceinline__ float node_step(NodeState& s, float alpha, float beta, float beta_prev) {
   if (s.first) {
     s.d = alpha + s.t;
@@ -927,7 +930,7 @@ __device__ __forceinline__ float node_step(NodeState& s, float alpha, float beta
   s.above = s.above && s.ds > 0.f;
   s.b2 = beta * beta;
   const float lo = node_lo(s) * s.lam;
-  return lo > 0.f ? warp_sum_f(__fdividef(s.wt * beta * fabsf(s.u), lo + s.t)) : 1e30f;
+  return lo > 0.f ? warp_sum_f(__fdividef(s.wt * beta * fabsf(s.u), lo + s.t)) : kNoBound;
 }
 
 // Lanczos from the vector the callers left in r.v (norm 1; NE elements per thread): T in
@@ -969,7 +972,7 @@ __device__ int lanczos(const Row<T, NW, GP, ALL, BWD>& r, int p, int sign, float
   }
   NodeState ns;
   if (node) node_init(ns, (float)r.nodes()[lane], (float)r.nodes()[kNodesAll + lane], r.lam, r.sigma, p, sign, lane);
-  float bound = 1e30f, bprev = 0.f, C = r.C;
+  float bound = kNoBound, bprev = 0.f, C = r.C;
   T beta = zero<T>(), inv = one<T>();
   int k = 0;
   for (;; ++k) {
@@ -1003,7 +1006,7 @@ __device__ int lanczos(const Row<T, NW, GP, ALL, BWD>& r, int p, int sign, float
       // NaN ends the run too: the row is then refused
       if (lane == 0) {
         r.be()[k - 1] = beta;
-        r.flag()[0] = !(bound > tol) || k >= cap;
+        r.flag()[0] = !(bound > tol) || bound >= kNoBound || k >= cap;
       }
     }
     sync_all<NW, ALL>();
@@ -1283,6 +1286,13 @@ __device__ void residual(const Row<T, NW, GP, ALL, BWD>& r, const Args& a, const
     s = warp_sum(s);
     if (lane == 0) out[k] = (k == r.pos ? 1.0 : 0.0) - s;
   }
+}
+
+// Row r.j goes to the general path.
+template <class T, int NW, bool GP, bool ALL, bool BWD>
+__device__ __forceinline__ void leave(const Row<T, NW, GP, ALL, BWD>& r, const Args& a) {
+  if (r.m <= a.small_max) a.redo_small[atomicAdd(&a.ctr->n_redo_small, 1)] = r.j;
+  else a.redo_list[atomicAdd(&a.ctr->n_redo, 1)] = r.j;
 }
 
 // Steps that the coupled iteration would take on spec(M) in [lo, 1] (reported as the row's

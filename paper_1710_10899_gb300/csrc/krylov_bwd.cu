@@ -121,6 +121,7 @@ __global__ void __launch_bounds__(threads_of<NW, ALL>(), MINB) bwd_kernel(const 
         for (int i = tid; i < r.mp; i += NT) r.set_v(i, i == r.pos ? one<T>() : zero<T>());
         sync_all<NW, ALL>();
         K0 = lanczos<NE>(r, p, a.sign, kTolGrad, &est0, &lo0);
+        if (node && lane == 0) r.flag()[8] = est0 <= kTolGrad && lo0 > 0.f;
         T n2 = zero<T>();
         for (int i = tid; i < r.mp; i += NT) {
           const T x = i < r.m ? scaled(a.grad_out[base + i], eg, (T*)nullptr) : zero<T>();
@@ -137,7 +138,8 @@ __global__ void __launch_bounds__(threads_of<NW, ALL>(), MINB) bwd_kernel(const 
         r.V = V1;
         r.o_t += t_bytes;
         sync_all<NW, ALL>();
-        K1 = lanczos<NE>(r, p, a.sign, kTolGrad, &est1, &lo1);
+        // (a row that the first process refuses needs no second)
+        if (r.flag()[8]) K1 = lanczos<NE>(r, p, a.sign, kTolGrad, &est1, &lo1);
         if (node) {
           lo = fminf(lo0, lo1);
           // the divided differences need the quadrature over both spectra
@@ -165,7 +167,7 @@ __global__ void __launch_bounds__(threads_of<NW, ALL>(), MINB) bwd_kernel(const 
       ok = Q > 0 && r.flag()[1] == 0;
     }
     if (!ok) {
-      if (tid == 0) a.redo_list[atomicAdd(&a.ctr->n_redo, 1)] = r.j;
+      if (tid == 0) leave(r, a);
       sync_all<NW, ALL>();
       continue;
     }

@@ -56,7 +56,13 @@ __global__ void __launch_bounds__(threads_of<NW, ALL>(), MINB) fwd_kernel(const 
         for (int i = tid; i < r.mp; i += NT) r.set_v(i, i == r.pos ? one<T>() : zero<T>());
         sync_all<NW, ALL>();
         K = lanczos<NE>(r, p, a.sign, Tol<T>::value, &est, &lo);
+        // the recurrence's bound not met (NaN is not): nothing more is spent on the row
+        if (node && lane == 0) r.flag()[6] = lo > 0.f && est <= Tol<T>::value ? 1 : 0;
+        sync_all<NW, ALL>();
+        ok = r.flag()[6] != 0;
       }
+    }
+    if (ok) {
       if constexpr (kDf<T>) {
         if (p == 1 && !direct) {
           // The inverse's column to FP64 accuracy (as the coupled iteration's): x from the
@@ -64,7 +70,7 @@ __global__ void __launch_bounds__(threads_of<NW, ALL>(), MINB) fwd_kernel(const 
           // for the correction, which needs few digits.  x stays in registers.
           if (node) {
             nc = root_coefs(r, K, p, lo, false, lane);
-            if (lane == 0) r.flag()[3] = lo > 0.f && est <= Tol<T>::value ? K + 1 : 0;
+            if (lane == 0) r.flag()[3] = K + 1;
           }
           sync_all<NW, ALL>();
           nc = r.flag()[3] - 1;
@@ -139,9 +145,9 @@ __global__ void __launch_bounds__(threads_of<NW, ALL>(), MINB) fwd_kernel(const 
           const double tau = (double)tau_f;
           const double al = a.sign < 0 ? 1.0 / (double)p : 1.0 - 1.0 / (double)p;
           *scale_s = exp2(E * ex) * (p > 1 ? pow(tau, -al) : 1.0);
-          // accepted only with the recurrence's bound met (NaN is not); for p = 1 the residual of
-          // the column (before its correction) is measured as well, as in refine_column
-          if (!fixed_up) r.flag()[3] = direct || (lo > 0.f && est <= Tol<T>::value && (double)est <= a.resid_tol) ? nc + 1 : 0;
+          // for p = 1 the residual of the column (before its correction) is what is compared, as in
+          // refine_column
+          if (!fixed_up) r.flag()[3] = direct || (double)est <= a.resid_tol ? nc + 1 : 0;
           else if (!(res1 <= a.resid_tol)) r.flag()[3] = 0;
         }
       }
@@ -198,7 +204,7 @@ __global__ void __launch_bounds__(threads_of<NW, ALL>(), MINB) fwd_kernel(const 
     }
     if (node && lane == 0) {
       if (!ok) {
-        a.redo_list[atomicAdd(&a.ctr->n_redo, 1)] = r.j;
+        leave(r, a);
       } else {
         // (without a recurrence: on the certified interval)
         const int iters = coupled_steps(direct ? r.sigma / r.lam : lo, p, r.m, a.fp64 != 0);

@@ -328,3 +328,31 @@ def test_inverse_column_residual_is_measured(sm):
     z, rep = forward(sm, a, 1, precision="fp64", resid_tol=2e-16)
     assert rep["n_fallback"] >= 1
     assert row_err(a, z, y, range(a.n)) <= 2e-12
+
+
+@pytest.mark.parametrize("p,sign", [(1, -1), (2, -1), (2, 1)])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_refused_rows_of_every_engine(sm, precision, p, sign):
+    """Rows beyond the engine's condition limit (one eigenvalue 1/5000, the others 0.1 to 1) at orders around the
+    small engine's: they come out of the coupled iteration or the fallback, short ones of the mixed mode out of
+    the small engine (whose products are counted), and the accepted rows beside them keep their bits.
+    Bars: the mixed one, and p m kappa eps = 2 * 64 * 2e4 * 2.2e-16 < 1e-9 in FP64."""
+    rng = np.random.default_rng(71)
+    orders, mats = [3, 31, 32, 33, 64], []
+    for n in orders:
+        q, _ = np.linalg.qr(rng.standard_normal((n, n)))
+        s = (q * np.r_[1.0 / 5000.0, np.linspace(0.1, 1.0, n - 1)]) @ q.T
+        mats += [0.5 * (s + s.T), np.eye(n) + 0.1 / n]
+    a = wl.dense_to_csr(sl.block_diag(*mats), keep=sl.block_diag(*[np.ones(x.shape, bool) for x in mats]))
+    ok = wl.dense_to_csr(sl.block_diag(*mats[1::2]), keep=sl.block_diag(*[np.ones(x.shape, bool) for x in mats[1::2]]))
+    y, rep = forward(sm, a, p, precision=precision, root_sign=sign)
+    ref = oracle.invroot(a.rowptr, a.colind, a.vals, p, sign=sign)
+    assert row_err(a, y, ref, range(a.n)) <= (1e-9 if precision == "fp64" else 1e-6)
+    assert rep["n_notspd"] == 0 and (rep["flops_tensor"] > 0) == (precision == "mixed")
+    z, _ = forward(sm, ok, p, precision=precision, root_sign=sign)
+    good, at = [], 0
+    for i, n in enumerate([n for n in orders for _ in range(2)]):
+        if i % 2:
+            good += range(a.rowptr[at], a.rowptr[at + n])
+        at += n
+    assert np.array_equal(y[good], z)
