@@ -237,6 +237,7 @@ kry::Args krylov_args(submat_plan_t P, const EngineRun& run, const double* in, d
   k.nb = run.cls.nb;
   k.ns = run.cls.ns;
   k.resid_tol = P->opts.resid_tol;
+  k.kappa_max = (float)P->opts.kappa_max;
   k.fp64 = P->opts.precision == SUBMAT_PREC_FP64 ? 1 : 0;
   k.nodes = P->nodes;
   return k;

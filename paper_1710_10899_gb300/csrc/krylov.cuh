@@ -92,7 +92,8 @@ struct Args {
   int32_t nb;                              // blocks per edge of the class
   int32_t ns;                              // blocks of S held in shared memory
   double resid_tol;
-  int32_t fp64;
+  float kappa_max;
+  int32_t fp64;                            // every row in FP64 (else double-float first)
   Nodes nodes;
   // backward
   const double* grad_out;
@@ -639,7 +640,7 @@ struct Row {
 };
 
 template <class T, int NW, bool GP, bool ALL, bool BWD>
-__device__ __forceinline__ void bind(Row<T, NW, GP, ALL, BWD>& r, const Args& a) {
+__device__ __forceinline__ void bind_storage(Row<T, NW, GP, ALL, BWD>& r, const Args& a) {
   const Layout L = layout(a.nb, a.ns, NW, !GP, BWD);
   char* scr = a.scratch + (size_t)blockIdx.x * a.stride;
   r.o_part = (int)L.part;
@@ -650,6 +651,17 @@ __device__ __forceinline__ void bind(Row<T, NW, GP, ALL, BWD>& r, const Args& a)
   r.V = reinterpret_cast<T*>(scr + L.g_v);
   r.X = reinterpret_cast<T*>(scr + L.g_x);
   r.AB = ALL || NW == 1 ? r.sblk() : reinterpret_cast<float4*>(scr + L.g_ab);
+}
+template <class T, int NW, bool GP, bool ALL, bool BWD>
+__device__ __forceinline__ void take_row(Row<T, NW, GP, ALL, BWD>& r, const Args& a, int j) {
+  r.j = j;
+  r.m = a.m[j];
+  r.pos = a.pos[j];
+  r.nb = (r.m + kB - 1) / kB;
+  r.mp = r.nb * kB;
+}
+template <class T, int NW, bool GP, bool ALL, bool BWD>
+__device__ __forceinline__ void load_nodes(const Row<T, NW, GP, ALL, BWD>& r, const Args& a) {
   for (int q = threadIdx.x; q < kNodesAll; q += threads_of<NW, ALL>()) {
     r.nodes()[q] = a.nodes.theta[q];
     r.nodes()[kNodesAll + q] = a.nodes.w[q];
@@ -1256,6 +1268,50 @@ __device__ bool cholesky(const Row<T, NW, GP, ALL, BWD>& r) {
     sync_mat<NW>();
   }
   return *bad == 0;
+}
+
+// The condition estimate lambda_bar / lambda_min that the mixed engines compare with kappa_max: eight
+// power steps on I - S / lambda_bar from a vector of +-1, in FP32 (see start_lo_slices).  S's blocks
+// are in place; the row's vector and sums are overwritten.  All warps.
+template <int NW, bool GP, bool ALL>
+__device__ __noinline__ float condition_estimate(const Args& a, int m, float lam) {
+  constexpr int NT = threads_of<NW, ALL>();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  Row<float, NW, GP, ALL, false> q;
+  bind_storage(q, a);
+  q.m = m;
+  q.nb = (m + kB - 1) / kB;
+  q.mp = q.nb * kB;
+  const float start = rsqrtf((float)m), scale = 1.f / lam;
+  for (int i = tid; i < q.mp; i += NT) q.set_v(i, i < m ? (i % 3 == 0 ? start : -start) : 0.f);
+  float norm = 1.f;
+  for (int t = 0; t < kStartLoSteps; ++t) {
+    sync_all<NW, ALL>();
+    if (warp < NW) {
+      float dot = 0.f;
+      for_blocks(q, warp, [&](int b, int I, int J) {
+        auto go = [&](const float4* x) {
+          if (I == J) block_mul<false>(x, q.v(), I, J, 0.f, q.part(), q.mp, lane, dot);
+          else block_mul<true>(x, q.v(), I, J, 0.f, q.part(), q.mp, lane, dot);
+        };
+        if (ALL || b < q.ns) go(q.sblk(b)); else go(q.gblk_at(b));
+      });
+    }
+    sync_all<NW, ALL>();
+    float n2 = 0.f;
+    for (int i = tid; i < q.mp; i += NT) {
+      const float d = q.v_at(i) - scale * row_sum<NW>(q.part(), i, q.mp, q.nb);
+      q.set_v(i, d);
+      n2 = fmaf(d, d, n2);
+    }
+    n2 = warp_total(n2);
+    if (lane == 0) q.red()[warp] = n2;
+    sync_all<NW, ALL>();
+    norm = sqrtf(total_of<NT / 32>(q.red(), lane, NT / 32));
+    const float inv = norm > 0.f ? 1.f / norm : 0.f;
+    for (int i = tid; i < q.mp; i += NT) q.set_v(i, q.v_at(i) * inv);
+  }
+  return norm < 1.f ? 1.f / (1.f - norm) : 3.0e38f;
 }
 
 // r = e_pos - S x in FP64 for x (FP64, r.m entries, in the units of the values): the pattern rows

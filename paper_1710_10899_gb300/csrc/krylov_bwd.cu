@@ -70,7 +70,8 @@ __global__ void __launch_bounds__(threads_of<NW, ALL>(), MINB) bwd_kernel(const 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool mat = warp < NW, node = kLone<NW, ALL> || warp == NW;
   Row<T, NW, GP, ALL, true> r;
-  bind(r, a);
+  bind_storage(r, a);
+  load_nodes(r, a);
   const Layout L = layout(a.nb, a.ns, NW, !GP, true);
   constexpr int t_bytes = decltype(r)::kF.t_bytes;
   T* const V0 = r.V;
@@ -88,12 +89,9 @@ __global__ void __launch_bounds__(threads_of<NW, ALL>(), MINB) bwd_kernel(const 
     const int idx = r.flag()[2];
     sync_all<NW, ALL>();
     if (idx >= a.n) break;
-    r.j = a.order[idx];
-    if (a.gbuf && (r.j < a.j0 || r.j >= a.j1)) continue;     // another wave's row
-    r.m = a.m[r.j];
-    r.pos = a.pos[r.j];
-    r.nb = (r.m + kB - 1) / kB;
-    r.mp = r.nb * kB;
+    const int j = a.order[idx];
+    if (a.gbuf && (j < a.j0 || j >= a.j1)) continue;         // another wave's row
+    take_row(r, a, j);
     const int base = a.rowptr[r.j];
     bool ok = gather(r, a);
     // g 2^-eg, eg the exponent of its largest entry
