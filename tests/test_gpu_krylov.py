@@ -356,3 +356,43 @@ def test_refused_rows_of_every_engine(sm, precision, p, sign):
             good += range(a.rowptr[at], a.rowptr[at + n])
         at += n
     assert np.array_equal(y[good], z)
+
+
+def low_block(n, kappa, rng):
+    """One eigenvalue 1, the others 1/kappa to 2/kappa: the condition estimate sees it whole."""
+    q, _ = np.linalg.qr(rng.standard_normal((n, n)))
+    s = (q * np.r_[np.linspace(1.0 / kappa, 2.0 / kappa, n - 1), 1.0]) @ q.T
+    return 0.5 * (s + s.T)
+
+
+@pytest.mark.parametrize("n", [30, 60, 120, 150])
+@pytest.mark.parametrize("p,sign", [(2, -1), (3, -1), (2, 1)])
+def test_wide_rows_of_the_mixed_mode_are_fp64(sm, n, p, sign):
+    """Rows whose condition estimate exceeds kappa_max = 100: FP64 arithmetic (counted), m kappa eps of the
+    column with kappa = 300; a narrow block beside them stays in double-float."""
+    rng = np.random.default_rng(81)
+    wide, narrow = low_block(n, 300.0, rng), np.eye(n) + 0.2 / n
+    a = wl.dense_to_csr(sl.block_diag(wide, narrow), keep=sl.block_diag(np.ones((n, n), bool), np.ones((n, n), bool)))
+    y, rep = forward(sm, a, p, precision="mixed", root_sign=sign)
+    ref = oracle.invroot(a.rowptr, a.colind, a.vals, p, sign=sign)
+    assert row_err(a, y, ref, range(n)) <= n * 300 * 2.2e-16
+    assert row_err(a, y, ref, range(n, 2 * n)) <= 1e-10
+    assert rep["n_fallback"] == 0 and rep["n_notspd"] == 0
+    # two flops a product, n^2 products a step, at least two steps a row, and not the narrow block's
+    assert 2 * 2 * n ** 3 <= rep["flops_fp64"] <= 2 * 64 * n ** 3
+
+
+@pytest.mark.parametrize("n", [30, 60, 120, 150, 200])
+@pytest.mark.parametrize("p,sign", [(2, -1), (3, -1), (2, 1)])
+def test_adjoint_of_wide_rows_is_fp64(sm, n, p, sign):
+    """The gradient at kappa = 600 (two passes of the wide rule) to m kappa eps, as the Jacobi adjoint
+    gave it (double-float: kappa 2^-45 times some tens)."""
+    rng = np.random.default_rng(82)
+    a = wl.dense_to_csr(low_block(n, 600.0, rng), keep=np.ones((n, n), bool))
+    w = wl.random_on_pattern(a, seed=5)
+    gref = oracle.grad(a.rowptr, a.colind, a.vals, p, w, sign=sign)
+    for det in (False, True):
+        plan = sm.submat_plan(a.rowptr, a.colind, p, root_sign=sign, grad_deterministic=det)
+        sm.submat_invroot(plan, torch.tensor(a.vals, device="cuda"))
+        g = sm.submat_invroot_backward(plan, torch.tensor(w, device="cuda")).cpu().numpy()
+        assert np.abs(g - gref).max() <= n * 600 * 2.2e-16 * np.abs(gref).max()
