@@ -642,7 +642,7 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
                       ? P->runs
                       : plan_runs(P, sizes, std::min(kry_max, (int)o.small_max_m), &scratch_bytes, &kry_bytes);
   // rows that the Krylov engine refuses go where their order would have taken them: short ones to
-  // the small engine (24 entries, 7200 rows refused: 4.0 ms on it, 10.9 with the tcgen05 engine)
+  // the small engine (7200 rows of 24 entries refused: 5.0 ms, 10.9 with the tcgen05 engine)
   const int redo_max = o.precision == SUBMAT_PREC_MIXED_F16 ? o.small_max_m : 0;
   const int32_t n_short = (int32_t)(sizes.end() - std::partition_point(sizes.begin(), sizes.end(),
                                                                        [&](int32_t m) { return m > redo_max; }));
@@ -690,7 +690,10 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
       if (joins) ++jobs.back().y;
       else jobs.push_back(make_int2(i, 1));
     }
-    if ((int32_t)jobs.size() < tc_rows) {
+    // The kernel's instance for groups takes 8 % longer on a row alone (its registers; n = 8192, 2670
+    // rows on this engine, one pair among them: 16.05 -> 17.2 ms in all), a row that joins
+    // another's job saves nearly all of its own: groups from one row in ten on.
+    if ((int64_t)jobs.size() * 10 <= (int64_t)tc_rows * 9) {
       PLAN_TRY(cudaMalloc(&P->d_jobs, jobs.size() * sizeof(int2)));
       PLAN_TRY(cudaMemcpy(P->d_jobs, jobs.data(), jobs.size() * sizeof(int2), cudaMemcpyHostToDevice));
       for (auto* rs : {&P->runs, &P->runs_stall})

@@ -1,6 +1,7 @@
 """Which engine a plan's options select: the tuner's cases, explicit defaults, launch counts."""
 import numpy as np
 import pytest
+import scipy.sparse as sp
 
 import oracle
 import workloads as wl
@@ -78,3 +79,28 @@ def test_a_default_given_explicitly_is_the_default(sm, precision, tol, p):
         assert torch.equal(sm.submat_invroot(other, v, sync=True), ref), kw
     steered = sm.submat_plan(a.rowptr, a.colind, p, precision=precision, k_max=41)
     assert not torch.equal(sm.submat_invroot(steered, v, sync=True), ref)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("twins,shared", [(1, False), (60, True)])
+def test_groups_from_one_row_in_ten_on(sm, twins, shared):
+    """Neighbouring rows of one pattern share a tcgen05 job only where enough rows do: the GEMMs are counted
+    once a job, so without groups the executed flops are p 10 / (p + 1) of the method's."""
+    r = wl.ring_spd(300, 200, seed=5)
+    a = sp.csr_matrix((r.vals, r.colind, r.rowptr), shape=(r.n, r.n))
+    twin = np.repeat(np.arange(r.n), np.where(np.arange(r.n) < twins, 2, 1))     # row i twice for i < twins
+    a = a[twin][:, twin].tolil()
+    for i in np.nonzero(twin[1:] == twin[:-1])[0]:
+        a[i, i + 1] = a[i + 1, i] = 0.1
+    a = (a + sp.diags(np.full(a.shape[0], 0.5))).tocsr()
+    a.sort_indices()
+    plan = sm.submat_plan(a.indptr.astype(np.int32), a.indices.astype(np.int32), 2)
+    y = sm.submat_invroot(plan, torch.tensor(a.data, device="cuda"), sync=True).cpu().numpy()
+    rep = plan.report()
+    ratio = rep["flops_tensor"] / rep["flops_alg"] / (20.0 / 3.0)
+    assert rep["n_fallback"] == 0 and (ratio < 0.95 if shared else abs(ratio - 1.0) < 1e-12)
+    rows = list(range(0, a.shape[0], 37))
+    ref = oracle.invroot(a.indptr, a.indices, a.data, 2, rows=rows)
+    for j in rows:
+        s = slice(a.indptr[j], a.indptr[j + 1])
+        assert np.linalg.norm(y[s] - ref[s]) <= 1e-6 * np.linalg.norm(ref[s])
