@@ -328,14 +328,29 @@ def timed_forward(sm, plan, vals, out, flush, steps, warmup):
     return ms, reps
 
 
-def roofline_mixed(reps, pk, pk_kind):
-    """Roofline of the mixed forward against the measured dense BF16 (= FP16) sustained rate: the
-    FP16 slice products that the tcgen05 rows execute, over the mean CUDA-event time of the whole
-    forward (the Krylov rows, on the FP32 units, share that time).  The coupled iteration's
-    flops on every row, whichever engine computed it, are given beside it as an equivalent."""
+DF_FLOPS = 11       # flops of a double-float multiply-add on the FP32 units: 5 fma, 1 add
+
+
+def roofline_mixed(reps, pk, pk_kind, work, clocks_mhz=None):
+    """Rooflines of the mixed forward, by what its kernels execute over the mean CUDA-event time of
+    the whole forward (both share it): the FP16 slice products of the tcgen05 rows against the
+    measured dense BF16 (= FP16) sustained rate, and the double-float products of the Krylov
+    rows against the FP32 rate.  A forward without tcgen05 rows has the second one alone.  The
+    coupled iteration's flops on every row, whichever engine computed it, are an equivalent."""
     kern_ms = statistics.mean(r["ms_kernel"] for r in reps)
     alg = statistics.mean(r["flops_alg"] for r in reps)
     executed = statistics.mean(r["flops_tensor"] for r in reps)
+    mhz = clocks_mhz or 2070.0
+    fp32 = fp32_alu_peak_tflops(mhz)
+    done = DF_FLOPS * work["fwd_products_df"] / (kern_ms / 1e3) / 1e12
+    krylov = {"bound": "alu", "kernel": "krylov fwd_kernel (double-float)", "achieved": done,
+              "peak": fp32, "unit": "TFLOP/s", "frac": done / fp32,
+              "peak_kind": f"FP32 FMA rate at {mhz:.0f} MHz (152 SMs x 128 lanes x 2)",
+              "flops_per_launch": DF_FLOPS * work["fwd_products_df"], "ms_kernel": kern_ms,
+              "work": "11 FP32 flops per double-float product, m_j^2 products per Lanczos step "
+                      "executed"}
+    if executed == 0.0:
+        return krylov
     peak = pk.get("bf16_tflops_sustained", pk.get("bf16_tflops"))
     achieved = executed / (kern_ms / 1e3) / 1e12
     return {"bound": "tensor", "kernel": "fwd_mixed_kernel", "achieved": achieved,
@@ -343,12 +358,10 @@ def roofline_mixed(reps, pk, pk_kind):
             "peak_kind": f"{pk_kind} bf16 dense sustained (FP16 rate = BF16 rate)",
             "flops_per_launch": executed, "ms_kernel": kern_ms,
             "work": "10 FP16 slice products x 2 m_j^3 per executed GEMM (tcgen05 rows only)",
+            "krylov_rows": krylov,
             "coupled_equivalent_tflops": alg / (kern_ms / 1e3) / 1e12,
             "coupled_equivalent_work": "sum over all rows of k_j (p+1) 2 m_j^3, not executed for the "
-                                       "rows of the Krylov engine",
-            "executed_tensor_tflops": executed / (kern_ms / 1e3) / 1e12,
-            "executed_tensor_frac": executed / (kern_ms / 1e3) / 1e12 / peak,
-            "executed_work": "10 FP16 slice products x 2 m_j^3 per executed GEMM"}
+                                       "rows of the Krylov engine"}
 
 
 def roofline_fp64(reps):
@@ -382,7 +395,8 @@ def run_extra(sm, spec, a, ref, rows_checked, flush, pk, pk_kind, clocks_mhz):
            "tol": 1e-10 if prec == "fp64" else 1e-6,
            "fallback_rows": int(reps[-1]["n_fallback"]),
            "iters_mean": reps[-1]["iters_sum"] / max(1, a.n),
-           "roofline": roofline_fp64(reps) if prec == "fp64" else roofline_mixed(reps, pk, pk_kind)}
+           "roofline": roofline_fp64(reps) if prec == "fp64" else
+           roofline_mixed(reps, pk, pk_kind, plan.work(), clocks_mhz)}
     if rows_checked is not None:
         rec["rows_sample"] = "seeded (seed 3) sample stratified by row size, incl. the " \
                              "smallest and largest rows"
@@ -403,6 +417,7 @@ def backward_block(sm, plan, a, vals, flush, steps, warm, clocks_mhz):
     sm.submat_invroot(plan, vals)
     ms, g = time_backward(sm, plan, w, flush, steps, warm)
     med = statistics.median(ms)
+    done = plan.work()
     gref = _PRE["grad_ref"]
     gh = g.cpu().numpy()
     # the deterministic (atomic-free) scatter: per-row gradients in waves, summed per entry
@@ -418,8 +433,7 @@ def backward_block(sm, plan, a, vals, flush, steps, warm, clocks_mhz):
            "bitwise_repeatable": bool(torch.equal(g_det, g_det2)),
            "max_abs_diff_vs_atomic_rel_to_max": float(np.abs(gd - gh).max() / np.abs(gh).max())}
     del pdet
-    m = a.row_sizes().astype(np.float64)
-    work = float((2.0 * m ** 2 * (2 * 30 + 2 * 20)).sum())
+    work = DF_FLOPS * done["bwd_products_df"]
     mhz = clocks_mhz or 2070.0
     peak = fp32_alu_peak_tflops(mhz)
     achieved = work / (med / 1e3) / 1e12
@@ -431,9 +445,9 @@ def backward_block(sm, plan, a, vals, flush, steps, warm, clocks_mhz):
         "roofline": {"bound": "alu", "kernel": "krylov bwd_kernel", "achieved": achieved,
                      "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                      "peak_kind": f"FP32 FMA rate at {mhz:.0f} MHz (152 SMs x 128 lanes x 2)",
-                     "work": "2 m_j^2 per Lanczos product and rank-one term, two processes of "
-                             "about 30 steps and 20 rank-two terms (an estimate; executed in "
-                             "double-float FP32 arithmetic, 6 operations a product)"},
+                     "work": "11 FP32 flops per double-float product executed: m_j^2 per Lanczos "
+                             "step of both processes and m_j per step and node (the rank-two "
+                             "terms of the stored entries come on top)"},
         "deterministic": det}}
 
 
@@ -711,7 +725,7 @@ def main():
 
     pk, pk_kind = peaks()
     if args.precision == "mixed":
-        roof = roofline_mixed(reps, pk, pk_kind)
+        roof = roofline_mixed(reps, pk, pk_kind, plan.work(), clocks["sm_mhz"] if clocks else None)
         roof["traffic"] = traffic_for("paper_1710_10899_gb300/csrc/fwd_mixed.cu")
     else:
         roof = roofline_fp64(reps)

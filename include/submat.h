@@ -186,6 +186,16 @@ typedef struct {
                               product); divide by ms_kernel for the roofline rate        */
 } submat_report;
 
+/* Work of the Krylov engine in the last forward and the last backward (submat_get_work). */
+typedef struct {
+  double fwd_products_df;  /* multiply-adds of double-floats (5 FP32 fma and 1 add each): m_j^2
+                              per Lanczos step of the rows in that arithmetic (FP64 rows:
+                              flops_fp64 of the report)                                   */
+  double bwd_products_df;  /* the same over both processes, and m_j per step and node for the
+                              node solutions (not the rank-two terms of the stored entries) */
+  double bwd_flops_fp64;   /* twice that for the rows that the backward takes in FP64      */
+} submat_work;
+
 typedef struct submat_plan_s* submat_plan_t;
 
 /*
@@ -311,6 +321,9 @@ SUBMAT_API submat_status submat_refine(submat_plan_t plan, const double* a_vals,
 
 /* Counters of the last forward (synchronises the plan's stream). */
 SUBMAT_API submat_status submat_get_report(submat_plan_t plan, submat_report* out);
+
+/* What the Krylov engine executed in the last forward and backward (synchronises the plan's stream). */
+SUBMAT_API submat_status submat_get_work(submat_plan_t plan, submat_work* out);
 
 /*
  * The integer plan as computed on the device (Alg. 1 index part): m[j] = |R_j| and

@@ -71,11 +71,20 @@ class Report(ctypes.Structure):
         return {k: getattr(self, k) for k, _ in self._fields_}
 
 
+class Work(ctypes.Structure):
+    _fields_ = [("fwd_products_df", ctypes.c_double), ("bwd_products_df", ctypes.c_double),
+                ("bwd_flops_fp64", ctypes.c_double)]
+
+    def as_dict(self):
+        return {k: getattr(self, k) for k, _ in self._fields_}
+
+
 EXPORTS = ["submat_default_opts", "submat_plan", "submat_invroot", "submat_invroot_host",
            "submat_invroot_backward",
            "submat_get_report", "submat_plan_rows", "submat_plan_shape", "submat_plan_destroy",
            "submat_status_string", "submat_last_error", "submat_invroot_noalloc", "submat_pcg",
-           "submat_shard_rows", "submat_test_stall", "submat_refine", "submat_plan_launches"]
+           "submat_shard_rows", "submat_test_stall", "submat_refine", "submat_plan_launches",
+           "submat_get_work"]
 
 _lib_handle = None
 
@@ -120,6 +129,8 @@ def load_library(path: str = LIB_PATH):
     lib.submat_shard_rows.restype = i32
     lib.submat_test_stall.argtypes = [vp, i32]
     lib.submat_test_stall.restype = i32
+    lib.submat_get_work.argtypes = [vp, ctypes.POINTER(Work)]
+    lib.submat_get_work.restype = i32
     lib.submat_plan_launches.argtypes = [vp, ctypes.POINTER(i32)]
     lib.submat_plan_launches.restype = i32
     lib.submat_refine.argtypes = [vp, vp, vp, i32, i32, vp, vp]
@@ -232,6 +243,12 @@ class Plan:
         r = Report()
         _check(self._lib, self._lib.submat_get_report(self._h, ctypes.byref(r)))
         return r.as_dict()
+
+    def work(self) -> dict:
+        """What the Krylov engine executed in the last forward and backward (``submat_get_work``)."""
+        w = Work()
+        _check(self._lib, self._lib.submat_get_work(self._h, ctypes.byref(w)))
+        return w.as_dict()
 
     def _vals(self, t):
         torch = _torch()

@@ -880,7 +880,7 @@ static bool ready_bwd(submat_plan_t P, cudaStream_t s) {
 // The adjoint of the rows of a's wave (all rows without waves): the Krylov runs side by side,
 // then the rows they left in the Jacobi kernel.
 static submat_status enqueue_backward(submat_plan_t P, const BwdArgs& a, bool krylov, cudaStream_t s) {
-  CUDA_TRY(cudaMemsetAsync(P->d_ctr_bwd, 0, sizeof(DevCounters), s));
+  CUDA_TRY(cudaMemsetAsync(P->d_ctr_bwd, 0, kCounterQueues, s));
   if (!krylov) {
     CUDA_TRY(launch_backward(a, P->grid, s));
     return SUBMAT_OK;
@@ -948,6 +948,7 @@ static submat_status backward_impl(submat_plan_t P, const double* grad_out, doub
   a.scratch_stride = P->stride;
   a.sign = P->opts.root_sign;
   CUDA_TRY(cudaMemsetAsync(grad_in, 0, (size_t)P->nnz * sizeof(double), s));
+  CUDA_TRY(cudaMemsetAsync(P->d_ctr_bwd, 0, sizeof(DevCounters), s));
   const bool krylov = ready_bwd(P, s);
   if (!P->opts.grad_deterministic) {
     const submat_status st = enqueue_backward(P, a, krylov, s);
@@ -1124,6 +1125,21 @@ submat_status submat_get_report(submat_plan_t P, submat_report* r) {
     CUDA_TRY(cudaEventElapsedTime(&r->ms_kernel, P->ev[0], P->ev[1]));
     CUDA_TRY(cudaEventElapsedTime(&r->ms_fallback, P->ev[1], P->ev[2]));
   }
+  return SUBMAT_OK;
+}
+
+submat_status submat_get_work(submat_plan_t P, submat_work* w) {
+  g_last_error.clear();
+  if (!P || !w) return fail(SUBMAT_EINVAL, "NULL argument");
+  std::memset(w, 0, sizeof(*w));
+  if (P->n == 0) return SUBMAT_OK;
+  CUDA_TRY(cudaStreamSynchronize(P->last_stream));
+  DevCounters c;
+  CUDA_TRY(cudaMemcpy(&c, P->d_ctr, sizeof(c), cudaMemcpyDeviceToHost));
+  w->fwd_products_df = c.products_df;
+  CUDA_TRY(cudaMemcpy(&c, P->d_ctr_bwd, sizeof(c), cudaMemcpyDeviceToHost));
+  w->bwd_products_df = c.products_df;
+  w->bwd_flops_fp64 = c.flops_fp64;
   return SUBMAT_OK;
 }
 

@@ -4,6 +4,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cuda_fp16.h>
+#include <stddef.h>
 #include <stdint.h>
 #include <string>
 #include <vector>
@@ -17,11 +18,15 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kMaxWarps = 16;          // largest CTA any helper below runs in (512 threads)
 constexpr int kRedDoubles = 2 * kMaxWarps;   // shared reduction scratch of the helpers
 
-// Device-side counters of one forward / backward call (zeroed before each call).
+// Device-side counters of one forward / backward call (zeroed before each call; each wave of a
+// deterministic backward zeroes the queues and lists at its start only).
 struct DevCounters {
   int32_t queue;              // persistent work queue head (rows handed out)
-  int32_t n_fallback;         // rows appended to the fallback list
   int32_t fb_queue;           // fallback work queue head
+  int32_t run_queue[12];      // work-queue heads of the forward's engine launches
+  int32_t n_redo, n_redo_small;        // rows the Krylov engine left to the general path, and
+                                       // to the small engine
+  int32_t n_fallback;         // rows appended to the fallback list
   int32_t iters_max;
   unsigned long long iters_sum;
   unsigned long long n_notspd;
@@ -30,14 +35,13 @@ struct DevCounters {
   double flops_tensor;
   unsigned long long n_illcond;        // rows sent to the fallback by the condition estimate
   int32_t error;                       // a device pipeline wait timed out
-  int32_t run_queue[12];               // work-queue heads of the forward's engine launches
-  int32_t n_redo, n_redo_small;        // rows the Krylov engine left to the general path, and
-                                       // to the small engine
   int32_t nonfinite;                   // some value of A is infinite or NaN
+  double products_df;                  // double-float multiply-adds of the Krylov engine
   double flops_alg;                    // sum over rows of k_j (p+1) 2 m_j^3 (+ 2 m_j^3 for
                                        // p = 1's final X product): executed iterations k_j,
                                        // true orders m_j, every product counted as a dense GEMM
 };
+constexpr size_t kCounterQueues = offsetof(DevCounters, n_fallback);
 
 // Arguments of the forward kernels.
 struct FwdArgs {

@@ -362,6 +362,9 @@ __device__ void vec_task(const VecTask& v) {
 // FP32 operations, the sums split into a part on the accumulator's grid and an exact rest, as in
 // krylov.cuh (6 operations a product, about 2^-44 of the row's norm).  sh: shared memory,
 // 8 nv mp bytes and 4 nv.
+// 12: the most whose split vectors fit the idle stage area at the largest order (one more does not,
+// see the assertion below), so a job holds 13 rows at most; a longer run of one pattern is cut into
+// jobs of 13 and a rest.
 constexpr int kGroupVecs = 12;
 __device__ __noinline__ void matvec_group(const __half* q, size_t plane, int ld, int e, const double* X, double* W,
                              int nv, int m, int mp, float* sh) {

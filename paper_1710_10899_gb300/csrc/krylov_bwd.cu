@@ -302,8 +302,10 @@ __device__ __forceinline__ bool row_gradient(Row<T, NW, GP, ALL, true>& r, const
   sync_all<NW, ALL>();
   }
   if (tid == 0) {
-    const double m2 = (double)r.m * r.m;
-    atomicAdd(&a.ctr->flops_fp64, 2.0 * m2 * (double)(K0 + K1) + 4.0 * m2 * Q * passes);
+    // products with S and of the Lanczos vectors with the node solutions
+    const double done = (double)r.m * (r.m + Q * passes) * (double)(K0 + K1);
+    if (kDf<T>) atomicAdd(&a.ctr->products_df, done);
+    else atomicAdd(&a.ctr->flops_fp64, 2.0 * done);
   }
   return false;
 }

@@ -210,6 +210,7 @@ __device__ __forceinline__ RowState column(Row<T, NW, GP, ALL, false>& r, const 
       atomicAdd(&a.ctr->iters_sum, (unsigned long long)iters);
       atomic_max_nonneg(&a.ctr->resid_max_bits, p == 1 && !direct ? res1 : (double)est);
       if (!kDf<T>) atomicAdd(&a.ctr->flops_fp64, 2.0 * m2 * (double)K);
+      else atomicAdd(&a.ctr->products_df, m2 * (double)K);
       atomicAdd(&a.ctr->flops_alg, ((double)iters * (p + 1) + (p == 1 ? 1.0 : 0.0)) * 2.0 * m2 * r.m);
     }
   }

@@ -396,3 +396,19 @@ def test_adjoint_of_wide_rows_is_fp64(sm, n, p, sign):
         sm.submat_invroot(plan, torch.tensor(a.vals, device="cuda"))
         g = sm.submat_invroot_backward(plan, torch.tensor(w, device="cuda")).cpu().numpy()
         assert np.abs(g - gref).max() <= n * 600 * 2.2e-16 * np.abs(gref).max()
+
+
+def test_executed_work_is_counted(sm):
+    """Products of the double-float rows: m^2 a step in the forward (two steps at least, 64 at most here), the same
+    for an adjoint in one launch and in waves of a few rows; FP64 rows are counted as FP64 flops."""
+    a = blocks([40, 150], seed=91)
+    v, w = torch.tensor(a.vals, device="cuda"), torch.ones(a.nnz, dtype=torch.float64, device="cuda")
+    m3 = float((a.row_sizes().astype(np.float64) ** 2).sum())
+    done = []
+    for kw in (dict(), dict(grad_deterministic=True, grad_wave_mib=1)):
+        plan = sm.submat_plan(a.rowptr, a.colind, 2, **kw)
+        sm.submat_invroot(plan, v, sync=True)
+        assert 2 * m3 <= plan.work()["fwd_products_df"] <= 64 * m3 and plan.report()["flops_fp64"] == 0
+        sm.submat_invroot_backward(plan, w)
+        done.append(plan.work())
+    assert done[0] == done[1] and done[0]["bwd_products_df"] >= 4 * m3 and done[0]["bwd_flops_fp64"] == 0
