@@ -412,3 +412,31 @@ def test_executed_work_is_counted(sm):
         sm.submat_invroot_backward(plan, w)
         done.append(plan.work())
     assert done[0] == done[1] and done[0]["bwd_products_df"] >= 4 * m3 and done[0]["bwd_flops_fp64"] == 0
+
+
+def test_mixed_inverse_is_refined_to_fp64(sm):
+    """The mixed mode's inverse at every class and block edge to FP64 accuracy, m kappa eps with kappa = 9
+    (its double-float recurrence alone stops at 1e-11)."""
+    a = blocks(ORDERS, seed=101)
+    y, rep = forward(sm, a, 1, precision="mixed")
+    ref = oracle.invroot(a.rowptr, a.colind, a.vals, 1)
+    m = a.row_sizes()
+    for n in ORDERS:
+        assert row_err(a, y, ref, np.nonzero(m == n)[0]) <= max(n, 2) * 9 * 2.2e-16, n
+    assert rep["n_fallback"] == 0 and rep["flops_tensor"] == 0
+
+
+def test_mixed_inverse_of_long_rows_is_refined(sm):
+    """The same for a row of 700 entries (four elements a thread, partial sums and most blocks in scratch; not a
+    multiple of the block or of the threads) among short ones, kappa < 4."""
+    n = 700
+    rng = np.random.default_rng(102)
+    off = 0.15 * rng.uniform(0.5, 1.0, n - 1)
+    dense = np.eye(n) * 2.0 + np.diag(off, 1) + np.diag(off, -1)
+    dense[0, 1:] = dense[1:, 0] = 0.02 * rng.uniform(0.5, 1.0, n - 1)
+    a = wl.dense_to_csr(dense)
+    y, rep = forward(sm, a, 1, precision="mixed")
+    rows = [0, 1, 2, 350, n - 1]
+    ref = oracle.invroot(a.rowptr, a.colind, a.vals, 1, rows=rows)
+    assert row_err(a, y, ref, rows) <= n * 4 * 2.2e-16
+    assert rep["n_fallback"] == 0 and rep["flops_tensor"] == 0
