@@ -440,3 +440,29 @@ def test_mixed_inverse_of_long_rows_is_refined(sm):
     ref = oracle.invroot(a.rowptr, a.colind, a.vals, 1, rows=rows)
     assert row_err(a, y, ref, rows) <= n * 4 * 2.2e-16
     assert rep["n_fallback"] == 0 and rep["flops_tensor"] == 0
+
+
+@pytest.mark.parametrize("deterministic", [False, True])
+def test_captured_backward_after_an_eager_one(sm, deterministic):
+    """A backward captured once the storage is there: the Krylov runs fork to the plan's streams and join again,
+    rows repeated in FP64 included; the replay on other values of the cotangent gives its gradient."""
+    a = blocks([20, 50, 150], seed=111)
+    vals = a.vals.copy()
+    vals[20 * 20:20 * 20 + 2500] = low_block(50, 300.0, np.random.default_rng(112)).ravel()
+    w = wl.random_on_pattern(a, seed=7)
+    plan = sm.submat_plan(a.rowptr, a.colind, 2, use_graph=False, grad_deterministic=deterministic)
+    v, wd = torch.tensor(vals, device="cuda"), torch.ones(a.nnz, dtype=torch.float64, device="cuda")
+    out, grad = torch.empty_like(v), torch.empty_like(v)
+    sm.submat_invroot(plan, v, out, sync=True)
+    sm.submat_invroot_backward(plan, wd, grad)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        sm.submat_invroot(plan, v, out)
+        sm.submat_invroot_backward(plan, wd, grad)
+    wd.copy_(torch.tensor(w))
+    grad.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    gref = oracle.grad(a.rowptr, a.colind, vals, 2, w)
+    assert np.abs(grad.cpu().numpy() - gref).max() <= 1e-10 * np.abs(gref).max()
