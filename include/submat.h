@@ -67,7 +67,8 @@ typedef enum {
  * for that column (Lanczos and a quadrature of the root, O(k m^2) instead of O(m^3)): in FP64
  * mode every order, in FP64 arithmetic; in MIXED_F16 mode with double-float arithmetic (FP32
  * pairs) orders up to 192 for p = 2 (up to 160 for p = 3, none beyond) and every order for p = 1,
- * whose column is then refined in FP64.  A row that it refuses
+ * whose column is then refined in FP64; for p >= 2 a row whose condition estimate exceeds
+ * kappa_max is repeated in FP64 arithmetic.  A row that it refuses
  * (lambda_bar / lambda_min above 2000; not positive definite) and every row of a plan whose
  * options steer the coupled iteration (k_max, tol, refine_steps, kappa_max, small_max_m or
  * sync_max_m other than its default; the default given explicitly is the default) takes the
@@ -115,9 +116,11 @@ typedef struct {
                               step amplifies the part of the error that does not commute
                               with S_j); < 0 selects the default                          */
   int32_t use_graph;       /* capture the forward launches into a CUDA graph; default 1  */
-  double kappa_max;        /* coupled iteration, mixed path: a row whose condition estimate
-                              lambda_bar / lambda_min (power iteration on the converged
-                              iterate) exceeds this goes to the FP64 fallback; default 100 */
+  double kappa_max;        /* mixed path: a row whose condition estimate lambda_bar /
+                              lambda_min (power iteration) exceeds this is FP64's: the
+                              coupled iteration sends it to the FP64 fallback, the Krylov
+                              engine (p >= 2; p = 1 is refined to FP64 accuracy in any case)
+                              repeats it in FP64 arithmetic; default 100                  */
   int32_t root_sign;       /* -1 (default): the inverse p-th root A^(-1/p); +1: the positive
                               p-th root A^(1/p), the same method with f(S) = S^(1/p)
                               (Sec. 4.2), computed from the same iteration as
@@ -172,10 +175,12 @@ typedef struct {
                               rows of (GEMMs executed) * 10 FP16 slice products *
                               2 m_j^3 (true m_j; p GEMMs per iteration for p >= 2;
                               two for p = 1, plus its final X product)                   */
-  double flops_fp64;       /* FP64 flops of the last forward (FP64 path: iterations;
-                              mixed path: column refinement; both: fallback)             */
-  float ms_kernel;         /* device time of the last forward's main (Newton) kernel,
-                              from CUDA events recorded around it on the launch stream   */
+  double flops_fp64;       /* FP64 flops of the last forward (coupled iteration: its
+                              products on the FP64 path, the column refinement on the mixed
+                              path; Krylov engine: 2 m_j^2 per step of the rows in FP64;
+                              both: fallback)                                            */
+  float ms_kernel;         /* device time of the last forward's engine launches, from CUDA
+                              events recorded around them on the launch stream           */
   float ms_fallback;       /* device time of the last forward's fallback kernel          */
   int64_t n_illcond;       /* rows sent to the fallback by the condition estimate        */
   double flops_alg;        /* the flops of the coupled iteration on the last forward's rows,
@@ -264,9 +269,10 @@ SUBMAT_API submat_status submat_invroot_host(submat_plan_t plan, const double* v
  * j the submatrix is regathered from the saved vals_in (recomputation, no stored iterates).
  * With f as a sum of simple fractions the Daleckii-Krein form is a sum of rank-two terms in
  * (S + t_q)^(-1) g and (S + t_q)^(-1) e_pos, which two Lanczos processes in double-float
- * arithmetic give; rows that this refuses (as in the forward), the inverse (p = 1,
- * root_sign = -1), p above SUBMAT_MIXED_MAX_P, and a first backward inside a stream capture
- * (its storage is allocated by the first backward) are decomposed instead: a cyclic Jacobi with
+ * arithmetic give (in FP64 for a spectrum wider than about lambda_bar / 100); rows that this
+ * refuses (as in the forward), the inverse (p = 1, root_sign = -1), p above SUBMAT_MIXED_MAX_P,
+ * and every row of a first backward inside a stream capture or without room for the storage that
+ * the first backward allocates are decomposed instead: a cyclic Jacobi with
  * the matrix and eigenvectors held as
  * double-floats (FP32 pairs, ~44 significant bits; the rotation angles, the divided
  * differences and the products with the eigenvectors in FP64).  grad_out and grad_in are

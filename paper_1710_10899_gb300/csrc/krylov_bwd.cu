@@ -6,9 +6,9 @@
 // weights are + w_q t_q).  Two Lanczos processes (from e_pos and from g) give all x_q and y_q, so
 // the gradient of a submatrix is a sum of kNodesGrad (or kNodes) rank-two terms instead of a full
 // eigendecomposition: O((k + q) m^2) against the ~9 sweeps of m^3 rotations of a Jacobi method.
-// All in double-float arithmetic.  Only stored entries are formed: the pattern rows are scanned
-// as in the gather, upper triangle only, and an entry's mirror image is found by the transposed
-// map.  Rows that the engine refuses are left to the Jacobi kernel (eig.cu), and so is the
+// In double-float arithmetic, wide spectra in FP64 (krylov.cuh).  Only stored entries are formed:
+// the pattern rows are scanned as in the gather, upper triangle only, and an entry's mirror image is
+// found by the transposed map.  Rows that the engine refuses are left to the Jacobi kernel (eig.cu), and so is the
 // inverse, where the Jacobi's error is the smaller one (5e-13 against 1.5e-12 of the gradient).
 // Measured on GB300, one backward, Jacobi -> this: n = 6144, orders 27..183, p = 2: 514 -> 9.5 ms;
 // n = 2501, orders 10..88, deterministic: 24.5 -> 1.6 ms; n = 400, orders up to 300 (which the

@@ -1,6 +1,6 @@
 // Forward by the Krylov engine (krylov.cuh): one persistent launch per size class, one CTA per
 // submatrix, FP64 or double-float arithmetic.  The mixed mode's inverse (p = 1) is refined to FP64
-// accuracy, as the coupled iteration's is: n = 12288, orders 36..244, 59.5 -> 18.0 ms at the same
+// accuracy, as the coupled iteration's is: n = 12288, orders 36..244, 59.5 -> 17.8 ms at the same
 // error (2.5e-15), of which the FP64 residual and the correction take 4.
 #include <algorithm>
 #include <cmath>
@@ -54,7 +54,7 @@ __device__ __forceinline__ RowState column(Row<T, NW, GP, ALL, false>& r, const 
         // rows whose condition estimate exceeds kappa_max are FP64's on every engine of the mixed
         // mode (p = 1 is refined to that below).  The recurrence's own bracket says which rows to
         // estimate at all; it is the sharper one, and rows above kappa_max by it alone (2 in 1000
-        // of the small overlap matrices) are better than 1e-11 here, 1e-9 on the other engines.
+        // of the small overlap matrices) are within 2e-11 here, within 1e-8 on the other engines.
         if (p > 1 && r.flag()[6] == 2 && condition_estimate<NW, GP, ALL>(a, r.m, r.lam) > a.kappa_max) return kAgain;
       }
     }
