@@ -335,31 +335,34 @@ def roofline_mixed(reps, pk, pk_kind, work, clocks_mhz=None):
     """Rooflines of the mixed forward, by what its kernels execute over the mean CUDA-event time of
     the whole forward (both share it): the FP16 slice products of the tcgen05 rows against the
     measured dense BF16 (= FP16) sustained rate, and the double-float products of the Krylov
-    rows against the FP32 rate.  A forward without tcgen05 rows has the second one alone.  The
-    coupled iteration's flops on every row, whichever engine computed it, are an equivalent."""
+    rows against the FP32 rate.  The one whose work takes longer at its peak comes first, the
+    other inside it.  The coupled iteration's flops on every row, whichever engine computed it,
+    are an equivalent."""
     kern_ms = statistics.mean(r["ms_kernel"] for r in reps)
     alg = statistics.mean(r["flops_alg"] for r in reps)
     executed = statistics.mean(r["flops_tensor"] for r in reps)
+    products = DF_FLOPS * work["fwd_products_df"]
     mhz = clocks_mhz or 2070.0
     fp32 = fp32_alu_peak_tflops(mhz)
-    done = DF_FLOPS * work["fwd_products_df"] / (kern_ms / 1e3) / 1e12
+    done = products / (kern_ms / 1e3) / 1e12
     krylov = {"bound": "alu", "kernel": "krylov fwd_kernel (double-float)", "achieved": done,
               "peak": fp32, "unit": "TFLOP/s", "frac": done / fp32,
               "peak_kind": f"FP32 FMA rate at {mhz:.0f} MHz (152 SMs x 128 lanes x 2)",
-              "flops_per_launch": DF_FLOPS * work["fwd_products_df"], "ms_kernel": kern_ms,
+              "flops_per_launch": products, "ms_kernel": kern_ms,
               "work": "11 FP32 flops per double-float product, m_j^2 products per Lanczos step "
                       "executed"}
-    if executed == 0.0:
-        return krylov
     peak = pk.get("bf16_tflops_sustained", pk.get("bf16_tflops"))
     achieved = executed / (kern_ms / 1e3) / 1e12
-    return {"bound": "tensor", "kernel": "fwd_mixed_kernel", "achieved": achieved,
-            "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-            "peak_kind": f"{pk_kind} bf16 dense sustained (FP16 rate = BF16 rate)",
-            "flops_per_launch": executed, "ms_kernel": kern_ms,
-            "work": "10 FP16 slice products x 2 m_j^3 per executed GEMM (tcgen05 rows only)",
-            "krylov_rows": krylov,
-            "coupled_equivalent_tflops": alg / (kern_ms / 1e3) / 1e12,
+    tensor = {"bound": "tensor", "kernel": "fwd_mixed_kernel", "achieved": achieved,
+              "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+              "peak_kind": f"{pk_kind} bf16 dense sustained (FP16 rate = BF16 rate)",
+              "flops_per_launch": executed, "ms_kernel": kern_ms,
+              "work": "10 FP16 slice products x 2 m_j^3 per executed GEMM (tcgen05 rows only)"}
+    if products / fp32 > executed / peak:
+        roof = {**krylov, "tcgen05_rows": tensor}
+    else:
+        roof = {**tensor, "krylov_rows": krylov}
+    return {**roof, "coupled_equivalent_tflops": alg / (kern_ms / 1e3) / 1e12,
             "coupled_equivalent_work": "sum over all rows of k_j (p+1) 2 m_j^3, not executed for the "
                                        "rows of the Krylov engine"}
 
