@@ -1,5 +1,5 @@
 // One column of a root of a symmetric positive definite submatrix by a Krylov method
-// (internal header; kernels in krylov_fwd.cu and krylov_bwd.cu).
+// (internal header; kernels in krylov_fwd.cuh and krylov_bwd.cu).
 //
 // The method keeps one column of F = f(S), f(x) = x^(-1/p) or x^(1/p).  From the Lanczos
 // recurrence S V = V T + beta v e^T started at e_pos (or at a cotangent), f(S) e_pos is
@@ -181,6 +181,15 @@ cudaError_t launch_fwd(const Args& a, const Class& c, int grid, cudaStream_t s);
 cudaError_t launch_bwd(const Args& a, const Class& c, int grid, cudaStream_t s);
 cudaError_t set_attr_fwd();
 cudaError_t set_attr_bwd();
+// the forward's instances (krylov_fwd.cuh)
+cudaError_t launch_roots_df(const Args& a, const Class& c, int grid, cudaStream_t s);
+cudaError_t launch_roots_fp64(const Args& a, const Class& c, int grid, cudaStream_t s);
+cudaError_t launch_inverse_df(const Args& a, const Class& c, int grid, cudaStream_t s);
+cudaError_t launch_inverse_fp64(const Args& a, const Class& c, int grid, cudaStream_t s);
+cudaError_t set_attr_roots_df();
+cudaError_t set_attr_roots_fp64();
+cudaError_t set_attr_inverse_df();
+cudaError_t set_attr_inverse_fp64();
 
 }  // namespace kry
 }  // namespace submat
@@ -1279,23 +1288,43 @@ __device__ bool cholesky(const Row<T, NW, GP, ALL, BWD>& r) {
 }
 
 // The condition estimate lambda_bar / lambda_min that the mixed engines compare with kappa_max: eight
-// power steps on I - S / lambda_bar from a vector of +-1, in FP32 (see start_lo_slices).  S's blocks
-// are in place; the row's vector and sums are overwritten.  All warps.
+// power steps on I - S / lambda_bar from a vector of +-1, in FP32 (see start_lo_slices; the norm
+// is taken of the last two vectors only).  S's blocks are in place; the row's vector and sums are
+// overwritten.  Called by the NW matrix warps, while the node warp solves for the coefficients
+// (rows of at most 32 entries: a lane per row of S, held in registers).
 template <int NW, bool GP, bool ALL>
 __device__ __noinline__ float condition_estimate(const Args& a, int m, float lam) {
-  constexpr int NT = threads_of<NW, ALL>();
+  constexpr int NM = NW * 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   Row<float, NW, GP, ALL, false> q;
-  bind_storage(q, a);
-  q.m = m;
-  q.nb = (m + kB - 1) / kB;
-  q.mp = q.nb * kB;
   const float start = rsqrtf((float)m), scale = 1.f / lam;
-  for (int i = tid; i < q.mp; i += NT) q.set_v(i, i < m ? (i % 3 == 0 ? start : -start) : 0.f);
-  float norm = 1.f;
-  for (int t = 0; t < kStartLoSteps; ++t) {
-    sync_all<NW, ALL>();
-    if (warp < NW) {
+  float last = 0.f, before = 0.f;
+  if constexpr (NW == 1) {
+    const float4* b = q.sblk();
+    float s[kB], v = lane < m ? (lane % 3 == 0 ? start : -start) : 0.f;
+#pragma unroll
+    for (int c = 0; c < kB; c += 2) {
+      const float4 x = b[pair_at(lane, c)];
+      s[c] = x.x;
+      s[c + 1] = x.y;
+    }
+#pragma unroll 1
+    for (int t = 0; t < kStartLoSteps; ++t) {
+      float y[4] = {};
+#pragma unroll
+      for (int c = 0; c < kB; ++c) y[c & 3] = fmaf(s[c], __shfl_sync(0xffffffffu, v, c), y[c & 3]);
+      if (t + 1 == kStartLoSteps) before = warp_total(v * v);
+      v -= scale * ((y[0] + y[1]) + (y[2] + y[3]));
+    }
+    last = warp_total(v * v);
+  } else {
+    bind_storage(q, a);
+    q.m = m;
+    q.nb = (m + kB - 1) / kB;
+    q.mp = q.nb * kB;
+    for (int i = tid; i < q.mp; i += NM) q.set_v(i, i < m ? (i % 3 == 0 ? start : -start) : 0.f);
+    for (int t = 0; t < kStartLoSteps; ++t) {
+      sync_mat<NW>();
       float dot = 0.f;
       for_blocks(q, warp, [&](int b, int I, int J) {
         auto go = [&](const float4* x) {
@@ -1304,21 +1333,26 @@ __device__ __noinline__ float condition_estimate(const Args& a, int m, float lam
         };
         if (ALL || b < q.ns) go(q.sblk(b)); else go(q.gblk_at(b));
       });
+      sync_mat<NW>();
+      before = last = 0.f;
+      for (int i = tid; i < q.mp; i += NM) {
+        const float v = q.v_at(i), d = v - scale * row_sum<NW>(q.part(), i, q.mp, q.nb);
+        q.set_v(i, d);
+        before = fmaf(v, v, before);
+        last = fmaf(d, d, last);
+      }
     }
-    sync_all<NW, ALL>();
-    float n2 = 0.f;
-    for (int i = tid; i < q.mp; i += NT) {
-      const float d = q.v_at(i) - scale * row_sum<NW>(q.part(), i, q.mp, q.nb);
-      q.set_v(i, d);
-      n2 = fmaf(d, d, n2);
+    before = warp_total(before);
+    last = warp_total(last);
+    if (lane == 0) {
+      q.red()[warp] = before;
+      q.red()[16 + warp] = last;
     }
-    n2 = warp_total(n2);
-    if (lane == 0) q.red()[warp] = n2;
-    sync_all<NW, ALL>();
-    norm = sqrtf(total_of<NT / 32>(q.red(), lane, NT / 32));
-    const float inv = norm > 0.f ? 1.f / norm : 0.f;
-    for (int i = tid; i < q.mp; i += NT) q.set_v(i, q.v_at(i) * inv);
+    sync_mat<NW>();
+    before = total_of<NW>(q.red(), lane, NW);
+    last = total_of<NW>(q.red() + 16, lane, NW);
   }
+  const float norm = before > 0.f ? sqrtf(last / before) : 0.f;
   return norm < 1.f ? 1.f / (1.f - norm) : 3.0e38f;
 }
 
