@@ -654,7 +654,7 @@ static submat_status plan_impl(const submat_csr* csr, int32_t p, const submat_op
   PLAN_TRY(cudaMalloc(&P->d_scratch, scratch_bytes));
   PLAN_TRY(cudaMalloc(&P->d_saved, (nnz > 0 ? nnz : 1) * sizeof(double)));
   if (kry_bytes > 0) {
-    PLAN_TRY(kry::set_attr_fwd());
+    PLAN_TRY(kry::set_attr_fwd(p, o.root_sign, !mixed));
     cudaError_t e = cudaMalloc(&P->d_redo, 2 * nb * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMalloc(&P->d_kry, kry_bytes);
     if (e == cudaErrorMemoryAllocation) {

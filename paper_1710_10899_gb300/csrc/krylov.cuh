@@ -179,7 +179,7 @@ int class_of(int m);                       // class index of a row of order m
 Class make_class(int index, int m_max, int rows, int n_sm, bool bwd);
 cudaError_t launch_fwd(const Args& a, const Class& c, int grid, cudaStream_t s);
 cudaError_t launch_bwd(const Args& a, const Class& c, int grid, cudaStream_t s);
-cudaError_t set_attr_fwd();
+cudaError_t set_attr_fwd(int p, int sign, bool fp64);
 cudaError_t set_attr_bwd();
 // the forward's instances (krylov_fwd.cuh)
 cudaError_t launch_roots_df(const Args& a, const Class& c, int grid, cudaStream_t s);

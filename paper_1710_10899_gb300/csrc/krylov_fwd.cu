@@ -13,11 +13,9 @@ cudaError_t launch_fwd(const Args& a, const Class& c, int grid, cudaStream_t s) 
   return a.fp64 ? launch_roots_fp64(a, c, grid, s) : launch_roots_df(a, c, grid, s);
 }
 
-cudaError_t set_attr_fwd() {
-  cudaError_t e;
-  if ((e = set_attr_roots_df()) != cudaSuccess || (e = set_attr_roots_fp64()) != cudaSuccess) return e;
-  if ((e = set_attr_inverse_df()) != cudaSuccess) return e;
-  return set_attr_inverse_fp64();
+cudaError_t set_attr_fwd(int p, int sign, bool fp64) {
+  if (p == 1 && sign < 0) return fp64 ? set_attr_inverse_fp64() : set_attr_inverse_df();
+  return fp64 ? set_attr_roots_fp64() : set_attr_roots_df();
 }
 
 // Gauss-Jacobi nodes for the weight (1-s)^(-a) (1+s)^(a-1): Newton's method on the Jacobi
