@@ -7,14 +7,14 @@
 // Device: NVIDIA GB300; p = 2; 7296 rows of one order per case; ms per forward
 // (median):
 //     m        small      sync   tcgen05
-//     8        1.904     6.145     4.508
-//    16        2.047     6.788     4.716
-//    24        2.291     7.345     5.517
-//    32        2.380     7.573     5.630
-//    48            -     8.371     6.596
-//    64            -     8.975     7.806
-//    96            -    25.950    11.104
-//   128            -    27.932    15.184
+//     8        1.806     4.832     3.745
+//    16        1.823     4.978     3.874
+//    24        2.115     5.206     4.234
+//    32        2.265     5.398     4.360
+//    48            -     6.325     5.252
+//    64            -     6.827     6.324
+//    96            -    16.404     8.414
+//   128            -    18.568    11.695
 #pragma once
 namespace submat {
 constexpr int kTunedSmallMaxM = 32;
