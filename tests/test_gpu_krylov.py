@@ -424,22 +424,27 @@ def test_mixed_inverse_is_refined_to_fp64(sm):
     for n in ORDERS:
         assert row_err(a, y, ref, np.nonzero(m == n)[0]) <= max(n, 2) * 9 * 2.2e-16, n
     assert rep["n_fallback"] == 0 and rep["flops_tensor"] == 0
+    z, _ = forward(sm, a, 1, precision="mixed", root_sign=1)          # A itself, once it is found definite
+    assert np.array_equal(z, a.vals)
 
 
-def test_mixed_inverse_of_long_rows_is_refined(sm):
-    """The same for a row of 700 entries (four elements a thread, partial sums and most blocks in scratch; not a
-    multiple of the block or of the threads) among short ones, kappa < 4."""
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_inverse_of_long_rows(sm, precision):
+    """The same in both modes for a row of 700 entries (four elements a thread, partial sums and most blocks in
+    scratch; not a multiple of the block or of the threads) among short ones, kappa < 4."""
     n = 700
     rng = np.random.default_rng(102)
     off = 0.15 * rng.uniform(0.5, 1.0, n - 1)
     dense = np.eye(n) * 2.0 + np.diag(off, 1) + np.diag(off, -1)
     dense[0, 1:] = dense[1:, 0] = 0.02 * rng.uniform(0.5, 1.0, n - 1)
     a = wl.dense_to_csr(dense)
-    y, rep = forward(sm, a, 1, precision="mixed")
+    y, rep = forward(sm, a, 1, precision=precision)
     rows = [0, 1, 2, 350, n - 1]
     ref = oracle.invroot(a.rowptr, a.colind, a.vals, 1, rows=rows)
     assert row_err(a, y, ref, rows) <= n * 4 * 2.2e-16
-    assert rep["n_fallback"] == 0 and rep["flops_tensor"] == 0
+    assert rep["n_fallback"] == 0 and rep["flops_tensor"] == 0 and rep["max_resid"] < 1e-9
+    z, _ = forward(sm, a, 1, precision=precision, root_sign=1)
+    assert np.array_equal(z, a.vals)
 
 
 @pytest.mark.parametrize("deterministic", [False, True])
@@ -466,3 +471,40 @@ def test_captured_backward_after_an_eager_one(sm, deterministic):
     torch.cuda.synchronize()
     gref = oracle.grad(a.rowptr, a.colind, vals, 2, w)
     assert np.abs(grad.cpu().numpy() - gref).max() <= 1e-10 * np.abs(gref).max()
+
+
+def test_wide_rows_of_one_warp(sm):
+    """More rows of order 30 than two waves, all wide: the instance with one warp a row repeats them in FP64,
+    forward and adjoint (bars as above, kappa = 300)."""
+    rng = np.random.default_rng(121)
+    mats = [low_block(30, 300.0, rng) for _ in range(90)]
+    a = wl.dense_to_csr(sl.block_diag(*mats), keep=sl.block_diag(*[np.ones((30, 30), bool)] * 90))
+    y, rep = forward(sm, a, 2, precision="mixed")
+    rows = list(range(0, a.n, 13))
+    ref = oracle.invroot(a.rowptr, a.colind, a.vals, 2, rows=rows)
+    assert row_err(a, y, ref, rows) <= 30 * 300 * 2.2e-16 and rep["n_fallback"] == 0
+    w = wl.random_on_pattern(a, seed=5)
+    plan = sm.submat_plan(a.rowptr, a.colind, 2)
+    sm.submat_invroot(plan, torch.tensor(a.vals, device="cuda"))
+    g = sm.submat_invroot_backward(plan, torch.tensor(w, device="cuda")).cpu().numpy()
+    gref = oracle.grad(a.rowptr, a.colind, a.vals, 2, w)
+    assert np.abs(g - gref).max() <= 30 * 300 * 2.2e-16 * np.abs(gref).max()
+    assert plan.work()["bwd_products_df"] == 0 and plan.work()["bwd_flops_fp64"] > 0
+
+
+@pytest.mark.parametrize("n", [300, 520])
+def test_adjoint_of_a_long_wide_row(sm, n):
+    """A wide row with blocks (300) and with its partial sums and factors (520) in scratch, among rows of two
+    entries: an arrow with one diagonal entry 1 and the others 1/300 to 2/300."""
+    d = np.r_[1.0, np.linspace(1.0 / 300.0, 2.0 / 300.0, n - 1)]
+    dense = np.diag(d)
+    dense[0, 1:] = dense[1:, 0] = 1e-4 * np.random.default_rng(131).uniform(0.5, 1.0, n - 1)
+    a = wl.dense_to_csr(dense)
+    w = wl.random_on_pattern(a, seed=5)
+    gref = oracle.grad(a.rowptr, a.colind, a.vals, 2, w)
+    for det in (False, True):
+        plan = sm.submat_plan(a.rowptr, a.colind, 2, grad_deterministic=det)
+        sm.submat_invroot(plan, torch.tensor(a.vals, device="cuda"))
+        g = sm.submat_invroot_backward(plan, torch.tensor(w, device="cuda")).cpu().numpy()
+        assert np.abs(g - gref).max() <= n * 300 * 2.2e-16 * np.abs(gref).max()
+        assert plan.work()["bwd_flops_fp64"] > 0
