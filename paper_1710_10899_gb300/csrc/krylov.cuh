@@ -1082,21 +1082,15 @@ __device__ __forceinline__ float tau_of(float lam, float lo) {
 // Node solutions x = (T + t)^(-1) e_1 (node q of the lane, the whole warp calls it), times the
 // node's weight, in r.X[k][lane]; a bottom-up elimination leaves the right-hand side e_1 alone,
 // so one sweep up for the pivots and one down for x.
-// The weight is tau w_q times `extra` (times t for x^(1/p), whose adjoint weighs
-// t (x + t)^(-1)); wt0 multiplies every weight.
+// The weight is tau w_q wt0 (times t for x^(1/p), whose adjoint weighs t (x + t)^(-1)).
 template <class T, int NW, bool GP, bool ALL, bool BWD>
-__device__ void node_solve(const Row<T, NW, GP, ALL, BWD>& r, int K, int p, float tau_f, int q, bool weighted,
+__device__ void node_solve(const Row<T, NW, GP, ALL, BWD>& r, int K, float tau_f, int q, bool weighted,
                            bool times_t, T wt0) {
   const int lane = threadIdx.x & 31;
   const T tau = as(tau_f, (T*)nullptr);
-  T t = zero<T>(), wt = one<T>();
-  if (p > 1) {
-    t = mul(tau, as(r.nodes()[q], (T*)nullptr));
-    wt = mul(tau, as(r.nodes()[kNodesAll + q], (T*)nullptr));
-    if (times_t) wt = mul(wt, t);
-  } else if (lane > 0) {
-    wt = zero<T>();
-  }
+  const T t = mul(tau, as(r.nodes()[q], (T*)nullptr));
+  T wt = mul(tau, as(r.nodes()[kNodesAll + q], (T*)nullptr));
+  if (times_t) wt = mul(wt, t);
   wt = mul(wt, wt0);
   T x = rcp(add(r.al()[K - 1], t));
   for (int k = K - 2; k >= 0; --k) {
@@ -1129,14 +1123,34 @@ __device__ void sum_nodes(const Row<T, NW, GP, ALL, BWD>& r, int K, bool more) {
 // adds the component K.  Returns the number of coefficients.  The whole (node) warp calls it.
 template <class T, int NW, bool GP, bool ALL, bool BWD>
 __device__ int root_coefs(const Row<T, NW, GP, ALL, BWD>& r, int K, int p, float lo, bool times_t, int lane) {
+  if (p == 1) {
+    // one node, t = 0: a lane's work, all of it in shared memory (through X and the sum over the
+    // nodes: mixed inverse n = 2000, orders up to 28, 175 -> 165 us; FP64, where nothing hides it,
+    // 256 -> 248)
+    if (lane == 0) {
+      T x = rcp(r.al()[K - 1]);
+      for (int k = K - 2; k >= 0; --k) {
+        const T g = mul(r.be()[k], x);
+        r.coef()[k + 1] = g;
+        x = rcp(sub(r.al()[k], mul(r.be()[k], g)));
+      }
+      r.coef()[0] = x;
+      for (int k = 1; k < K; ++k) {
+        x = neg(mul(r.coef()[k], x));
+        r.coef()[k] = x;
+      }
+    }
+    __syncwarp();
+    return K;
+  }
   const float tau = tau_of(r.lam, lo);
-  if (p == 1 || lo >= kLoWide) {
-    node_solve(r, K, p, tau, lane, true, false, one<T>());
+  if (lo >= kLoWide) {
+    node_solve(r, K, tau, lane, true, false, one<T>());
     sum_nodes(r, K, false);
   } else {
 #pragma unroll 1
     for (int h = 0; h < kNodesWide / 32; ++h) {
-      node_solve(r, K, p, tau, kNodes + 32 * h + lane, true, false, one<T>());
+      node_solve(r, K, tau, kNodes + 32 * h + lane, true, false, one<T>());
       sum_nodes(r, K, h > 0);
     }
   }

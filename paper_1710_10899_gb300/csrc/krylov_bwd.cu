@@ -43,9 +43,9 @@ __device__ void solve_nodes(Row<T, NW, GP, ALL, true>& r, const Args& a, int K0,
   const float lo = __int_as_float(r.flag()[4]);
   const float tau = r.lam * sqrtf(lo);
   const int q0 = lo >= 0.02f ? kNodes + kNodesWide : (lo >= kLoWide ? 0 : kNodes + 32 * pass);
-  const int q = p == 1 ? 0 : q0 + min(lane, Q - 1);
+  const int q = q0 + min(lane, Q - 1);
   const double al = a.sign < 0 ? 1.0 / (double)p : 1.0 - 1.0 / (double)p;
-  double f = (p > 1 ? pow((double)tau, -al) : 1.0) * 0.5 * join(gnorm);
+  double f = pow((double)tau, -al) * 0.5 * join(gnorm);
   const double E = (double)(r.e0 - 1023) * ((double)a.sign / (double)p - 1.0);
   const double fl = floor(E);
   f *= exp2(E - fl);
@@ -54,10 +54,10 @@ __device__ void solve_nodes(Row<T, NW, GP, ALL, true>& r, const Args& a, int K0,
   T wt0 = as(a.sign < 0 ? -f : f, (T*)nullptr);
   if (lane >= Q) wt0 = zero<T>();
   r.X = X0;
-  node_solve(r, K1, p, tau, q, false, false, one<T>());
+  node_solve(r, K1, tau, q, false, false, one<T>());
   r.X = X1;
   r.o_t -= t_bytes;
-  node_solve(r, K0, p, tau, q, true, a.sign > 0, wt0);
+  node_solve(r, K0, tau, q, true, a.sign > 0, wt0);
   r.o_t += t_bytes;
   r.X = X0;
   if (lane == 0) r.flag()[5] = ef + (int)fl + (eg - 1023);

@@ -3,7 +3,7 @@
 // their own (what only one of them needs costs the other up to 5 % at orders up to 32: registers),
 // compiled in files of their own.
 // The mixed mode's inverse (p = 1) is refined to FP64 accuracy, as the coupled iteration's is: n =
-// 12288, orders 36..244, 59.5 -> 17.7 ms at the same error (2.5e-15), of which the FP64 residual and the
+// 12288, orders 36..244, 59.5 -> 17.9 ms at the same error (2.5e-15), of which the FP64 residual and the
 // correction take 4.
 #pragma once
 #include "krylov.cuh"
@@ -126,9 +126,9 @@ __device__ __forceinline__ RowState column(Row<T, NW, GP, ALL, false>& r, const 
     }
     if constexpr (!kDf<T> && INV) {
       // The inverse's column in FP64 (in registers) and its residual, by one more product.  It needs S,
-      // so the node solve is not hidden behind the factorisation: n = 2048, orders 28..239, 6.65 ->
-      // 7.00 ms (from the pattern rows instead, after the factorisation: 7.04; n = 2000, orders up to
-      // 28: 251 us without, 256 so, 281 from the rows).
+      // so the node solve is not hidden behind the factorisation: n = 2048, orders 28..239, 6.66 ->
+      // 6.96 ms (from the pattern rows instead, after the factorisation: 7.04; n = 2000, orders up to
+      // 28: 248 us, 281 from the rows).
       if (node) {
         nc = root_coefs(r, K, p, lo, false, lane);
         if (lane == 0) r.flag()[3] = nc + 1;
