@@ -42,13 +42,13 @@
 // 28..239, 301 -> 6.4 ms (bound: the FP64 pipe, 30 products of m^2 a row); FP64 n = 2000,
 // orders 1..28, 11.6 -> 0.26 ms; double-float n = 8192, orders 19..119, 11.1 -> 2.6 ms and
 // n = 9973, orders 25..169, 23.0 -> 4.7 ms.  By the counters (classes of 64 to 250): FP64 keeps its
-// pipe 60..82 % busy; double-float issues in 27..42 % of the slots (adjoint 32..50 %) and waits at
+// pipe 60..82 % busy; double-float issues in 27..43 % of the slots (adjoint 33..50 %) and waits at
 // the step's two barriers first.
 //
 // Wide spectra.  Double-float errors grow as kappa 2^-45, so rows beyond lam / 100 are FP64's where
 // the coupled iteration and the Jacobi adjoint gave them that accuracy: the kernel repeats such a
 // row with its FP64 instance.  7200 rows of order 24 / 1800 of order 150 at kappa = 300, forward
-// p = 2: 45 / 1929 ms (fallback), 0.39 / 1.26 (double-float, 2e-12..1e-11 off), 1.28 / 5.4 (2e-14);
+// p = 2: 45 / 1929 ms (fallback), 0.39 / 1.26 (double-float, 2e-12..1e-11 off), 1.37 / 5.4 (2e-14);
 // adjoint 19 / 217 ms (Jacobi), 1.8 / 4.4 (double-float, up to 1e-10 off), 5.0 / 17.2 (1e-14..1e-13).
 #pragma once
 #include "common.cuh"
